@@ -16,6 +16,8 @@
 #include <type_traits>
 #include <utility>
 
+#include "bm64.cuh"
+
 namespace lbfd {
 
 enum LatticeId : int { kD1Q3 = 0, kD2Q9 = 1, kD3Q19 = 2, kD2Q5 = 3 };
@@ -516,7 +518,8 @@ __host__ __device__ __forceinline__ float2 noise_amplitude<float2>(float2 x) {
 
 // Box-Muller pair (z0, z1) = sqrt(-2 ln u0) (cos 2 pi u1, sin 2 pi u1) from
 // two Philox words, u = ((r >> 8) + 1/2) 2^-24.
-// FP64: the uniforms are exact; CUDA's log / sqrt / sincospi.
+// FP64 on the device: fixed-point logarithm, Newton square root and tabled
+// angles (bm64.cuh).
 // FP32 on the device: the special-function unit.  An odd multiple of 2^-25
 // above 1/2 has no FP32 representation, so the quantities that need it are
 // formed exactly from the integer word instead:
@@ -530,12 +533,16 @@ __host__ __device__ __forceinline__ float2 noise_amplitude<float2>(float2 x) {
 template <typename R>
 struct BoxMuller {
   __host__ __device__ static __forceinline__ void pair(uint32_t r0, uint32_t r1, R &z0, R &z1) {
+#ifdef __CUDA_ARCH__
+    bm64::pair(r0, r1, bm64::kTables, z0, z1);
+#else
     const R u0 = unit24<R>(r0), u1 = unit24<R>(r1);
     const R rad = Math<R>::sqrt(R(-2) * Math<R>::log(u0));
     R s, c;
     Math<R>::sincospi(R(2) * u1, &s, &c);
     z0 = rad * c;
     z1 = rad * s;
+#endif
   }
 };
 
