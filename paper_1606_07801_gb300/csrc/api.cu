@@ -557,7 +557,7 @@ int lbfd_step(lbfd_t h, int64_t n) {
       const int chunk = int(std::min<int64_t>(std::min<int64_t>(kChunk, n - done), until));
       const int to = h->cur ^ (chunk & 1);
       a.ph = make_philox_step(o.seed, o.lattice_id, uint64_t(h->t));
-      cudaError_t e = launch_step_small(o.lattice, o.precision, h->f[h->cur], h->f[to], a, o.seed, o.lattice_id,
+      cudaError_t e = launch_step_small(o.lattice, o.precision, h->f[h->cur], h->f[to], a, o.lattice_id,
                                         uint64_t(h->t), chunk, h->stream);
       if (e == cudaErrorNotSupported) {
         // the cluster cannot be placed on this GPU: one launch per step instead

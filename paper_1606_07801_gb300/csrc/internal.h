@@ -99,7 +99,7 @@ template <>
 __host__ __device__ __forceinline__ float step_param<float>(double, float f) { return f; }
 
 // CTAs of the many-steps-per-launch path for a small lattice: 1 = one block
-// (k_step_small), 2..8 = a thread-block cluster (k_step_cluster), 0 = the
+// (LBFD_KERNEL_SMALL), 2..16 = a thread-block cluster (LBFD_KERNEL_CLUSTER), 0 = the
 // lattice does not fit it (or its lattice type has no such path).
 int small_path_ctas(int lattice, int precision, int64_t N);
 
@@ -173,11 +173,10 @@ cudaError_t launch_step_mrt(int lattice, int precision, const void *src, void *d
 
 // Many steps of a small lattice in one launch (step_small.cu), in one
 // block's shared memory or in a thread-block cluster's distributed shared
-// memory (up to 8 x kSmallMaxBytes): src holds the stored state at step t0,
-// dst receives it after nsteps steps (dst may equal src).
+// memory (at most kSmallMaxBytes per CTA): src holds the stored state at step
+// t0, dst receives it after nsteps steps (dst may equal src).
 constexpr size_t kSmallMaxBytes = 200 * 1024;
-bool small_path_fits(int lattice, int precision, int64_t N);
-cudaError_t launch_step_small(int lattice, int precision, const void *src, void *dst, const StepArgs &a, uint64_t seed,
+cudaError_t launch_step_small(int lattice, int precision, const void *src, void *dst, const StepArgs &a,
                               uint32_t lattice_id, uint64_t t0, int nsteps, cudaStream_t stream);
 
 // D2Q5 weights and moment basis (m[a*5 + i]) for second moment theta.

@@ -17,28 +17,40 @@ enum StepNoise : int { kStepNoiseOff = 0, kStepNoiseGauss = 1, kStepNoiseFlat = 
 // device.cuh's lane arithmetic: V = R for one site, V = float2 (R = float)
 // for sites s and s + 1 in the two lanes.  Every floating-point operation is
 // an explicit add_rn / sub_rn / mul_rn / fma_rn, so both forms round alike.
+// It has two halves: the noise of a site, which depends on the site and the
+// step alone (noise_sums), and the update given it (collide_given).
+
+// The back-transformed unit noise T_i (w_i T_i where
+// NoiseTransform::kWeighted) of site s; zero without noise.
+template <int LAT, typename R, int NOISE, typename V>
+__device__ __forceinline__ void noise_sums(V (&T)[Lattice<LAT>::Q], uint32_t s, const PhiloxStep &ph) {
+  constexpr int Q = Lattice<LAT>::Q;
+  static_for<Q>([&](auto I) { T[decltype(I)::value] = splat<V>(R(0)); });
+  if constexpr (NOISE != kStepNoiseOff) {
+    V zz[Q - 1];
+    if constexpr (LaneOf<V>::kLanes == 2)
+      draw_variates_pair<Q - 1, NOISE == kStepNoiseGauss>(zz, s, ph);
+    else
+      draw_variates_t<R, Q - 1, NOISE == kStepNoiseGauss>(zz, s, ph);
+    NoiseTransform<LAT, R>::apply(zz, T);
+  }
+}
+
 template <int LAT, typename R, int NOISE, bool DEV, typename V>
-__device__ __forceinline__ void collide_lanes(V (&f)[Lattice<LAT>::Q], uint32_t s, const StepArgs &a) {
+__device__ __forceinline__ void collide_given(V (&f)[Lattice<LAT>::Q], const V (&T)[Lattice<LAT>::Q],
+                                              const StepArgs &a) {
   using L = Lattice<LAT>;
   constexpr int Q = L::Q;
   V rho = f[0];  // drho for DEV
   static_for<Q - 1>([&](auto I) { rho = add_rn(rho, f[decltype(I)::value + 1]); });
 
   V sigma = splat<V>(R(0));
-  V T[Q];
-  static_for<Q>([&](auto I) { T[decltype(I)::value] = splat<V>(R(0)); });
   if constexpr (NOISE != kStepNoiseOff) {
     // local noise: max(rho, 0); global noise: rho^eq (a select, not a branch)
     const V rho_eq = splat<V>(step_param<R>(a.rho_eq, a.rho_eq_f));
     const V rho_loc = positive_part(DEV ? add_rn(rho_eq, rho) : rho);
     const V rho_n = a.noise_mode == kNoiseLocal ? rho_loc : rho_eq;
     sigma = noise_amplitude<V>(mul_rn(rho_n, splat<V>(step_param<R>(a.noise_var, a.noise_var_f))));
-    V zz[Q - 1];
-    if constexpr (LaneOf<V>::kLanes == 2)
-      draw_variates_pair<Q - 1, NOISE == kStepNoiseGauss>(zz, s, a.ph);
-    else
-      draw_variates_t<R, Q - 1, NOISE == kStepNoiseGauss>(zz, s, a.ph);
-    NoiseTransform<LAT, R>::apply(zz, T);
   }
 
   const V omega = splat<V>(step_param<R>(a.omega, a.omega_f));
@@ -64,6 +76,13 @@ __device__ __forceinline__ void collide_lanes(V (&f)[Lattice<LAT>::Q], uint32_t 
     moved = add_rn(moved, f[i]);
   });
   f[0] = sub_rn(rho, moved);
+}
+
+template <int LAT, typename R, int NOISE, bool DEV, typename V>
+__device__ __forceinline__ void collide_lanes(V (&f)[Lattice<LAT>::Q], uint32_t s, const StepArgs &a) {
+  V T[Lattice<LAT>::Q];
+  noise_sums<LAT, R, NOISE>(T, s, a.ph);
+  collide_given<LAT, R, NOISE, DEV>(f, T, a);
 }
 
 // Collision of one site in registers: f holds the pulled populations
@@ -105,6 +124,14 @@ __device__ __forceinline__ void collide_pair(float (&fa)[Lattice<LAT>::Q], float
 template <int LAT, typename R, int NOISE, bool DEV = false>
 struct SrtCollide {
   static constexpr bool kPairs = std::is_same<R, float>::value;
+  // the two halves, for kernels that make the noise ahead of the update
+  static constexpr int kAhead = Lattice<LAT>::Q;  // values of the first half
+  __device__ __forceinline__ void ahead(R (&T)[kAhead], uint32_t s, const PhiloxStep &ph) const {
+    noise_sums<LAT, R, NOISE>(T, s, ph);
+  }
+  __device__ __forceinline__ void given(R (&f)[Lattice<LAT>::Q], const R (&T)[kAhead], const StepArgs &a) const {
+    collide_given<LAT, R, NOISE, DEV>(f, T, a);
+  }
   __device__ __forceinline__ void operator()(R (&f)[Lattice<LAT>::Q], uint32_t s, const StepArgs &a) const {
     collide_site<LAT, R, NOISE, DEV>(f, s, a);
   }
