@@ -273,7 +273,7 @@ static int step_path(const lbfd_sim *h, int64_t n) {
   }
   if (o.step_kernel != LBFD_KERNEL_AUTO) return o.step_kernel;
   if (h->staged_ok && staged_default()) return LBFD_KERNEL_STAGED;
-  return step_vec_width(o.lattice, o.precision, int32_t(o.dims[0])) >= 2 ? LBFD_KERNEL_VEC : LBFD_KERNEL_SCALAR;
+  return step_vec_width(o.lattice, o.precision, int32_t(o.dims[0]), h->N) >= 2 ? LBFD_KERNEL_VEC : LBFD_KERNEL_SCALAR;
 }
 
 static void free_sim(lbfd_sim *h) {
@@ -578,7 +578,7 @@ int lbfd_step(lbfd_t h, int64_t n) {
   const int kernel = step_path(h, 1);
   int vec_width = 1;
   if (kernel == LBFD_KERNEL_VEC) {
-    vec_width = step_vec_width(o.lattice, o.precision, a.Lx);
+    vec_width = step_vec_width(o.lattice, o.precision, a.Lx, h->N);
     if (vec_width == 1) vec_width = 2;  // asked for by step_kernel: Lx is even
   }
   const bool fusable = o.sample_every > 0 && !h->mrt &&

@@ -432,7 +432,7 @@ inline bool step_pdl() {
 template <int LAT, typename S, int NOISE, typename Idx>
 cudaError_t step_noise_idx(const S *s, S *d, const StepArgs &a, int vx, cudaStream_t stream) {
   dim3 grid, block;
-  step_shape(a.Lx, a.Ly, a.Lz, grid, block, vx);
+  step_shape(a.Lx, a.Ly, a.Lz, grid, block, vx, step_threads(LAT, sizeof(typename Store<S>::R) == 8 ? kStoreF64 : kStoreF32));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;

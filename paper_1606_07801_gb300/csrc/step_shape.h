@@ -11,14 +11,22 @@
 namespace lbfd {
 
 // Sites per thread of the register-pull step kernel (k_step_vec; 1 is
-// k_step): 4 (16-byte loads and stores of FP32) where that measured faster on
-// GB300 and Lx allows, else 2 where Lx is even, else 1.  Four sites won for
-// D2Q9 in every FP32-arithmetic format (84.5 against 83.9 GLUPS at 2048^2)
-// and for D3Q19 with 16-bit storage (37.9 against 37.6 at 256^3); D3Q19 in
-// FP32 needs too many registers for four (31.7 against 38.9), and FP64 keeps
-// two.  A tuning knob only; results do not depend on it.  LBFD_STEP_VX = 1,
-// 2 or 4 overrides the choice where Lx allows.
-inline int step_vec_width(int lattice, int precision, int32_t Lx) {
+// k_step), where Lx allows: several share the address and load instructions,
+// but are updated one after the other, which a lattice of few warps per SM
+// pays in full.  Measured on GB300, microseconds per step:
+//   4 (16-byte loads and stores of FP32) for D2Q9 and for D3Q19 with 16-bit
+//     storage from 2^19 sites: D3Q19 FP16 128^3 49.1 against 53.2 with two,
+//     but 64^3 13.8 against 8.2; D2Q9 FP16 1024^2 12.1 against 12.9, but D2Q9
+//     FP32 320^2 6.0 against 3.3.  D3Q19 in FP32 needs too many registers for
+//     four (31.7 against 38.9 GLUPS).
+//   2 otherwise, but 1 for the smallest: D2Q9 200^2 2.8 against 3.7 with two,
+//     D3Q19 22^3 2.8 against 6.3, 32^3 5.5 against 7.0 (16-bit 5.5 against
+//     6.9; 48^3 7.0 against 7.2).
+//   1 in FP64, whose narrow pipe hides the extra instructions: D2Q9 512 x 384
+//     47.0 against 50.3 with two, 60 x 50 6.1 against 10.3.
+// A tuning knob only; results do not depend on it.  LBFD_STEP_VX = 1, 2 or 4
+// overrides the choice where Lx allows.
+inline int step_vec_width(int lattice, int precision, int32_t Lx, int64_t sites = INT64_MAX) {
   static int forced = [] {
     const char *e = getenv("LBFD_STEP_VX");
     const int r = e ? atoi(e) : 0;
@@ -26,22 +34,33 @@ inline int step_vec_width(int lattice, int precision, int32_t Lx) {
   }();
   int vx = forced;
   if (vx == 0) {
-    const bool four = precision != kStoreF64 && (lattice == kD2Q9 || (lattice == kD3Q19 && precision != kStoreF32));
-    vx = four ? 4 : 2;
+    const int64_t few = lattice != kD3Q19 ? 48 << 10 : (precision == kStoreF32 ? 40 << 10 : 24 << 10);
+    const bool four = lattice == kD2Q9 || (lattice == kD3Q19 && precision != kStoreF32);
+    vx = precision == kStoreF64 || sites <= few ? 1 : (four && sites >= (1 << 19) ? 4 : 2);
   }
   if (vx == 4 && precision == kStoreF64) vx = 2;
   if (Lx % vx == 0) return vx;
   return Lx % 2 == 0 ? 2 : 1;
 }
 
+// Threads of a block of the one-launch-per-step kernels.  FP64: one warp, so
+// that the blocks spread evenly over the SMs' narrow FP64 pipes (D2Q9 60 x 50:
+// 18.8 us with 256 threads and two sites each, 6.1 with 32 and one; D3Q19
+// 64^3 168.8 and 147.4).  FP32 arithmetic: 128 for the lattices whose
+// registers fill the SM, a finer last wave at the same occupancy (D3Q19 FP32
+// 64^3 9.3 -> 8.3 us, 128^3 54.5 -> 53.6, FP16 128^3 51.3 -> 49.1).
+inline int step_threads(int lattice, int precision) {
+  return precision == kStoreF64 ? 32 : (lattice == kD1Q3 ? 256 : 128);
+}
+
 // Block and grid of the one-launch-per-step kernels for vx sites per thread:
-// 256-thread blocks, x fastest (at least one warp along x), one grid plane
+// blocks of `threads` threads, x fastest (at least one warp along x), one grid plane
 // per z.
-inline void step_shape(int32_t Lx, int32_t Ly, int32_t Lz, dim3 &grid, dim3 &block, int vx = 1) {
+inline void step_shape(int32_t Lx, int32_t Ly, int32_t Lz, dim3 &grid, dim3 &block, int vx = 1, int threads = 256) {
   const int cols = Lx / vx;
-  int bx = 256;
+  int bx = threads;
   while (bx > 32 && bx / 2 >= cols) bx /= 2;
-  int by = 256 / bx;
+  int by = threads / bx;
   while (by > 1 && by / 2 >= Ly) by /= 2;
   block = dim3(bx, by, 1);
   grid = dim3((cols + bx - 1) / bx, (Ly + by - 1) / by, Lz);
