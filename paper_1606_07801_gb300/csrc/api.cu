@@ -264,13 +264,13 @@ static bool staged_default() {
 // per launch, so they need n >= 2; otherwise one launch per step.
 static int step_path(const lbfd_sim *h, int64_t n) {
   const lbfd_options &o = h->opt;
-  if (h->mrt) return LBFD_KERNEL_MRT;
   if (h->slab) return LBFD_KERNEL_STAGED;
   if (n >= 2) {
     const int ctas = small_path_ctas(o.lattice, o.precision, h->N);
     if (ctas == 1) return LBFD_KERNEL_SMALL;
     if (ctas > 1) return LBFD_KERNEL_CLUSTER;
   }
+  if (h->mrt) return LBFD_KERNEL_MRT;
   if (o.step_kernel != LBFD_KERNEL_AUTO) return o.step_kernel;
   if (h->staged_ok && staged_default()) return LBFD_KERNEL_STAGED;
   return step_vec_width(o.lattice, o.precision, int32_t(o.dims[0]), h->N) >= 2 ? LBFD_KERNEL_VEC : LBFD_KERNEL_SCALAR;
@@ -557,8 +557,10 @@ int lbfd_step(lbfd_t h, int64_t n) {
       const int chunk = int(std::min<int64_t>(std::min<int64_t>(kChunk, n - done), until));
       const int to = h->cur ^ (chunk & 1);
       a.ph = make_philox_step(o.seed, o.lattice_id, uint64_t(h->t));
-      cudaError_t e = launch_step_small(o.lattice, o.precision, h->f[h->cur], h->f[to], a, o.lattice_id,
-                                        uint64_t(h->t), chunk, h->stream);
+      cudaError_t e = h->mrt ? launch_step_small_mrt(o.lattice, o.precision, h->f[h->cur], h->f[to], a, h->m, h->w,
+                                                     h->tau_m, o.lattice_id, uint64_t(h->t), chunk, h->stream)
+                             : launch_step_small(o.lattice, o.precision, h->f[h->cur], h->f[to], a, o.lattice_id,
+                                                 uint64_t(h->t), chunk, h->stream);
       if (e == cudaErrorNotSupported) {
         // the cluster cannot be placed on this GPU: one launch per step instead
         (void)cudaGetLastError();

@@ -178,6 +178,10 @@ cudaError_t launch_step_mrt(int lattice, int precision, const void *src, void *d
 constexpr size_t kSmallMaxBytes = 200 * 1024;
 cudaError_t launch_step_small(int lattice, int precision, const void *src, void *dst, const StepArgs &a,
                               uint32_t lattice_id, uint64_t t0, int nsteps, cudaStream_t stream);
+// The same with the moment-space collision (arguments as launch_step_mrt).
+cudaError_t launch_step_small_mrt(int lattice, int precision, const void *src, void *dst, const StepArgs &a,
+                                  const double *m, const double *w, const double *tau, uint32_t lattice_id,
+                                  uint64_t t0, int nsteps, cudaStream_t stream);
 
 // D2Q5 weights and moment basis (m[a*5 + i]) for second moment theta.
 void d2q5_tables(double theta, double *w, double *m);

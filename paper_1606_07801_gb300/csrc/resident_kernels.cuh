@@ -19,6 +19,7 @@
 // FP32 16^3 8.24 -> 1.37, D1Q3 FP64 256 sites 2.75 -> 2.26.
 #pragma once
 
+#include <algorithm>
 #include <cuda_runtime.h>
 
 #include "fastdiv.cuh"
@@ -178,6 +179,52 @@ __global__ void __launch_bounds__(resident_threads(LAT, sizeof(typename Store<S>
     }
     resident_wait<CL>();
   }
+}
+
+template <int LAT, typename S, class C, bool CL>
+cudaError_t resident_launch(const void *src, void *dst, const StepArgs &a, const ResidentArgs &ra, const C &c, int ctas,
+                            int threads, cudaStream_t stream) {
+  auto kern = k_step_resident<LAT, S, C, CL>;
+  const size_t bytes = 2 * size_t(Lattice<LAT>::Q) * size_t(ra.chunk) * sizeof(S);
+  // the opt-ins above 48 KB of dynamic shared memory and above 8 CTAs, on the current device
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmallMaxBytes));
+  if (e == cudaSuccess && CL && ctas > 8)
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(ctas, 1, 1);
+  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.dynamicSmemBytes = bytes;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = ctas;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = CL ? 1 : 0;
+  if (CL) {
+    // a cluster that the GPU cannot place is reported, not launched
+    int placeable = 0;
+    e = cudaOccupancyMaxActiveClusters(&placeable, kern, &cfg);
+    if (e != cudaSuccess) return e;
+    if (placeable < 1) return cudaErrorNotSupported;
+  }
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<const S *>(src), static_cast<S *>(dst), a, ra, c);
+}
+
+template <int LAT, typename S, class C>
+cudaError_t resident_t(const void *src, void *dst, const StepArgs &a, ResidentArgs ra, const C &c, int precision,
+                       cudaStream_t stream) {
+  const int ctas = small_path_ctas(LAT, precision, a.N);
+  if (ctas == 0) return cudaErrorInvalidValue;
+  ra.chunk = int((a.N + ctas - 1) / ctas);
+  ra.div_x = make_fastdiv(uint32_t(a.Lx));
+  ra.div_y = make_fastdiv(uint32_t(a.Ly));
+  ra.div_chunk = make_fastdiv(uint32_t(ra.chunk));
+  const int threads = (ra.chunk + 31) / 32 * 32;
+  return ctas > 1 ? resident_launch<LAT, S, C, true>(src, dst, a, ra, c, ctas, threads, stream)
+                  : resident_launch<LAT, S, C, false>(src, dst, a, ra, c, 1, threads, stream);
 }
 
 }  // namespace lbfd

@@ -429,24 +429,31 @@ inline bool step_pdl() {
   return v;
 }
 
+// Launch configuration of a step kernel, with the dependent-launch attribute.
+struct StepLaunch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  StepLaunch(dim3 grid, dim3 block, cudaStream_t stream) {
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = stream;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = step_pdl() ? 1 : 0;
+  }
+  StepLaunch(const StepLaunch &) = delete;
+};
+
 template <int LAT, typename S, int NOISE, typename Idx>
 cudaError_t step_noise_idx(const S *s, S *d, const StepArgs &a, int vx, cudaStream_t stream) {
   dim3 grid, block;
   step_shape(a.Lx, a.Ly, a.Lz, grid, block, vx, step_threads(LAT, sizeof(typename Store<S>::R) == 8 ? kStoreF64 : kStoreF32));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = step_pdl() ? 1 : 0;
-  if (vx == 2) return cudaLaunchKernelEx(&cfg, k_step_vec<LAT, S, 2, NOISE, Idx>, s, d, a);
+  StepLaunch launch(grid, block, stream);
+  if (vx == 2) return cudaLaunchKernelEx(&launch.cfg, k_step_vec<LAT, S, 2, NOISE, Idx>, s, d, a);
   if constexpr (sizeof(typename Store<S>::R) == 4)
-    if (vx == 4) return cudaLaunchKernelEx(&cfg, k_step_vec<LAT, S, 4, NOISE, Idx>, s, d, a);
-  return cudaLaunchKernelEx(&cfg, k_step<LAT, S, NOISE, Idx>, s, d, a);
+    if (vx == 4) return cudaLaunchKernelEx(&launch.cfg, k_step_vec<LAT, S, 4, NOISE, Idx>, s, d, a);
+  return cudaLaunchKernelEx(&launch.cfg, k_step<LAT, S, NOISE, Idx>, s, d, a);
 }
 
 template <int LAT, typename S, int NOISE>

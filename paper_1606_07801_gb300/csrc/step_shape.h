@@ -14,11 +14,14 @@ namespace lbfd {
 // k_step), where Lx allows: several share the address and load instructions,
 // but are updated one after the other, which a lattice of few warps per SM
 // pays in full.  Measured on GB300, microseconds per step:
-//   4 (16-byte loads and stores of FP32) for D2Q9 and for D3Q19 with 16-bit
-//     storage from 2^19 sites: D3Q19 FP16 128^3 49.1 against 53.2 with two,
+//   4 (16-byte loads and stores of FP32) for all but D3Q19 in FP32 from 2^19
+//     sites: D1Q3 FP32 2^24 63.9 against 68.2 with two (10^5 sites 2.7 against
+//     2.0), D3Q19 FP16 128^3 49.1 against 53.2 with two,
 //     but 64^3 13.8 against 8.2; D2Q9 FP16 1024^2 12.1 against 12.9, but D2Q9
 //     FP32 320^2 6.0 against 3.3.  D3Q19 in FP32 needs too many registers for
-//     four (31.7 against 38.9 GLUPS).
+//     four (31.7 against 38.9 GLUPS).  D2Q5, whose sites are short, takes four
+//     from the start (moment-space 400^2 2.9 against 3.4, 2048^2 26.2 against
+//     27.2).
 //   2 otherwise, but 1 for the smallest: D2Q9 200^2 2.8 against 3.7 with two,
 //     D3Q19 22^3 2.8 against 6.3, 32^3 5.5 against 7.0 (16-bit 5.5 against
 //     6.9; 48^3 7.0 against 7.2).
@@ -35,8 +38,8 @@ inline int step_vec_width(int lattice, int precision, int32_t Lx, int64_t sites 
   int vx = forced;
   if (vx == 0) {
     const int64_t few = lattice != kD3Q19 ? 48 << 10 : (precision == kStoreF32 ? 40 << 10 : 24 << 10);
-    const bool four = lattice == kD2Q9 || (lattice == kD3Q19 && precision != kStoreF32);
-    vx = precision == kStoreF64 || sites <= few ? 1 : (four && sites >= (1 << 19) ? 4 : 2);
+    const bool four = lattice != kD3Q19 || precision != kStoreF32;
+    vx = precision == kStoreF64 || sites <= few ? 1 : (lattice == kD2Q5 || (four && sites >= (1 << 19)) ? 4 : 2);
   }
   if (vx == 4 && precision == kStoreF64) vx = 2;
   if (Lx % vx == 0) return vx;

@@ -1,13 +1,11 @@
 // Many steps of a small lattice in one launch: which lattices take the
-// resident kernel (resident_kernels.cuh), and its launch.
+// resident kernel (resident_kernels.cuh), and the single-relaxation launches.
 #include <algorithm>
 #include <cuda_runtime.h>
 
 #include "resident_kernels.cuh"
 
 namespace lbfd {
-
-namespace {
 
 // CTAs of a lattice (1: a single block, else a cluster), 0 where the resident
 // kernel is not taken.  One site per thread bounds the lattice: 16 CTAs of
@@ -25,60 +23,19 @@ namespace {
 // FP64 arithmetic, 2 lanes per clock and SM, takes a CTA per 32 sites, and up
 // to 128 sites on each (D2Q9 1600 sites 5.5 against 6.0 launched, 3000 sites
 // 7.2 against 6.1; D3Q19 1728 sites 12.3 and 12.3, 4096 sites 20.8 and 12.4).
-int resident_ctas(int lattice, int64_t N, int elem, bool f64) {
-  const int Q = lattice == kD1Q3 ? 3 : (lattice == kD2Q9 ? 9 : 19);
+int small_path_ctas(int lattice, int precision, int64_t N) {
+  if (N < 1) return 0;
+  const int elem = storage_bytes(precision);
+  const bool f64 = precision == kStoreF64;
+  const int Q = lattice == kD1Q3 ? 3 : (lattice == kD2Q9 ? 9 : (lattice == kD2Q5 ? 5 : 19));
   const int64_t by_smem = int64_t(kSmallMaxBytes) / (2 * int64_t(Q) * elem);
   if (N > kResidentCtas * std::min<int64_t>(by_smem, resident_threads(lattice, f64))) return 0;
   if (f64) return int(std::min<int64_t>(kResidentCtas, (N + 31) / 32));
-  const int64_t one = lattice == kD1Q3 ? 512 : (lattice == kD2Q9 ? 256 : 128);
+  const int64_t one = lattice == kD1Q3 ? 512 : (lattice == kD3Q19 ? 128 : 256);
   return N <= one ? 1 : (N <= 512 ? 8 : kResidentCtas);
 }
 
-template <int LAT, typename S, class C, bool CL>
-cudaError_t resident_launch(const void *src, void *dst, const StepArgs &a, const ResidentArgs &ra, const C &c, int ctas,
-                            int threads, cudaStream_t stream) {
-  auto kern = k_step_resident<LAT, S, C, CL>;
-  const size_t bytes = 2 * size_t(Lattice<LAT>::Q) * size_t(ra.chunk) * sizeof(S);
-  // the opt-ins above 48 KB of dynamic shared memory and above 8 CTAs, on the current device
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmallMaxBytes));
-  if (e == cudaSuccess && CL && ctas > 8)
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(ctas, 1, 1);
-  cfg.blockDim = dim3(threads, 1, 1);
-  cfg.dynamicSmemBytes = bytes;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = ctas;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = CL ? 1 : 0;
-  if (CL) {
-    // a cluster that the GPU cannot place is reported, not launched
-    int placeable = 0;
-    e = cudaOccupancyMaxActiveClusters(&placeable, kern, &cfg);
-    if (e != cudaSuccess) return e;
-    if (placeable < 1) return cudaErrorNotSupported;
-  }
-  return cudaLaunchKernelEx(&cfg, kern, static_cast<const S *>(src), static_cast<S *>(dst), a, ra, c);
-}
-
-template <int LAT, typename S, class C>
-cudaError_t resident_t(const void *src, void *dst, const StepArgs &a, ResidentArgs ra, const C &c,
-                       cudaStream_t stream) {
-  const int ctas = resident_ctas(LAT, a.N, sizeof(S), sizeof(typename Store<S>::R) == 8);
-  if (ctas == 0) return cudaErrorInvalidValue;
-  ra.chunk = int((a.N + ctas - 1) / ctas);
-  ra.div_x = make_fastdiv(uint32_t(a.Lx));
-  ra.div_y = make_fastdiv(uint32_t(a.Ly));
-  ra.div_chunk = make_fastdiv(uint32_t(ra.chunk));
-  const int threads = (ra.chunk + 31) / 32 * 32;
-  return ctas > 1 ? resident_launch<LAT, S, C, true>(src, dst, a, ra, c, ctas, threads, stream)
-                  : resident_launch<LAT, S, C, false>(src, dst, a, ra, c, 1, threads, stream);
-}
+namespace {
 
 template <int LAT>
 cudaError_t resident_lat(int precision, const void *src, void *dst, const StepArgs &a, const ResidentArgs &ra,
@@ -86,22 +43,16 @@ cudaError_t resident_lat(int precision, const void *src, void *dst, const StepAr
   return dispatch_storage(precision, [&](auto tag) -> cudaError_t {
     using S = typename decltype(tag)::type;
     if (a.noise_mode == kNoiseOff)
-      return resident_t<LAT, S>(src, dst, a, ra, SrtCollideFor<LAT, S, kStepNoiseOff>{}, stream);
+      return resident_t<LAT, S>(src, dst, a, ra, SrtCollideFor<LAT, S, kStepNoiseOff>{}, precision, stream);
     if (a.noise_dist == kGaussian)
-      return resident_t<LAT, S>(src, dst, a, ra, SrtCollideFor<LAT, S, kStepNoiseGauss>{}, stream);
-    return resident_t<LAT, S>(src, dst, a, ra, SrtCollideFor<LAT, S, kStepNoiseFlat>{}, stream);
+      return resident_t<LAT, S>(src, dst, a, ra, SrtCollideFor<LAT, S, kStepNoiseGauss>{}, precision, stream);
+    return resident_t<LAT, S>(src, dst, a, ra, SrtCollideFor<LAT, S, kStepNoiseFlat>{}, precision, stream);
   });
 }
 
 }  // namespace
 
-int small_path_ctas(int lattice, int precision, int64_t N) {
-  if (lattice != kD1Q3 && lattice != kD2Q9 && lattice != kD3Q19) return 0;
-  if (N < 1) return 0;
-  return resident_ctas(lattice, N, storage_bytes(precision), precision == kStoreF64);
-}
-
-// Single-relaxation lattices only (D2Q5 and moment-space runs take their own kernel).
+// Single-relaxation lattices (moment-space runs: launch_step_small_mrt).
 cudaError_t launch_step_small(int lattice, int precision, const void *src, void *dst, const StepArgs &a,
                               uint32_t lattice_id, uint64_t t0, int nsteps, cudaStream_t stream) {
   if (nsteps < 1 || a.N < 1) return cudaErrorInvalidValue;
