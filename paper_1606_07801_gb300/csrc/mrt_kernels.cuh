@@ -95,10 +95,10 @@ __device__ __forceinline__ void mrt_forward(const V (&f)[Lattice<LAT>::Q], V (&M
   }
 }
 
-// The update given the site's variates z.
-template <int LAT, typename R, int NOISE, typename V>
-__device__ __forceinline__ void mrt_given(V (&f)[Lattice<LAT>::Q], const V (&z)[Lattice<LAT>::Q - 1],
-                                          const StepArgs &a, const MrtParams<R, Lattice<LAT>::Q> &p) {
+// The update given the site's variates z(a - 1).
+template <int LAT, typename R, int NOISE, typename V, class ZF>
+__device__ __forceinline__ void mrt_given(V (&f)[Lattice<LAT>::Q], const ZF &z, const StepArgs &a,
+                                          const MrtParams<R, Lattice<LAT>::Q> &p) {
   using L = Lattice<LAT>;
   constexpr int Q = L::Q;
   V rho = f[0];
@@ -112,7 +112,7 @@ __device__ __forceinline__ void mrt_given(V (&f)[Lattice<LAT>::Q], const V (&z)[
     const V sr = noise_amplitude<V>(rho_n);
     static_for<Q - 1>([&](auto A) {
       constexpr int k = decltype(A)::value;
-      M[k] = fma_rn(splat<V>(p.omega[k + 1]), M[k], mul_rn(mul_rn(sr, splat<V>(p.amp[k + 1])), z[k]));
+      M[k] = fma_rn(splat<V>(p.omega[k + 1]), M[k], mul_rn(mul_rn(sr, splat<V>(p.amp[k + 1])), z(k)));
     });
   } else {
     static_for<Q - 1>([&](auto A) {
@@ -156,24 +156,32 @@ struct MrtCollide {
   static constexpr bool kPairs = std::is_same<R, float>::value;
   static constexpr int kAhead = Q - 1, kNoise = NOISE;
   MrtParams<R, Q> p;
-  __device__ __forceinline__ void ahead(R (&z)[kAhead], uint32_t s, const PhiloxStep &ph) const {
-    if constexpr (NOISE != kStepNoiseOff) draw_variates_t<R, Q - 1, NOISE == kStepNoiseGauss>(z, s, ph);
+  template <typename V>
+  __device__ __forceinline__ void ahead(V (&z)[kAhead], uint32_t s, const PhiloxStep &ph, uint32_t apart = 1u) const {
+    if constexpr (NOISE != kStepNoiseOff) {
+      if constexpr (LaneOf<V>::kLanes == 2)
+        draw_variates_pair<Q - 1, NOISE == kStepNoiseGauss>(z, s, ph, apart);
+      else
+        draw_variates_t<R, Q - 1, NOISE == kStepNoiseGauss>(z, s, ph);
+    }
   }
-  __device__ __forceinline__ void given(R (&f)[Q], const R (&z)[kAhead], const StepArgs &a) const {
+  template <typename V, class ZF>
+  __device__ __forceinline__ void given(V (&f)[Q], const ZF &z, const StepArgs &a) const {
     mrt_given<LAT, R, NOISE>(f, z, a, p);
   }
-  __device__ __forceinline__ void operator()(R (&f)[Q], uint32_t s, const StepArgs &a) const {
-    R z[Q - 1];
+  template <typename V>
+  __device__ __forceinline__ void whole(V (&f)[Q], uint32_t s, const StepArgs &a) const {
+    V z[kAhead];
     ahead(z, s, a.ph);
-    given(f, z, a);
+    given(f, [&](int k) -> V { return z[k]; }, a);
   }
+  __device__ __forceinline__ void operator()(R (&f)[Q], uint32_t s, const StepArgs &a) const { whole(f, s, a); }
   __device__ __forceinline__ void pair(R (&fa)[Q], R (&fb)[Q], uint32_t s, const StepArgs &a) const {
     if constexpr (kPairs) {
-      float2 f[Q], z[Q - 1];
+      float2 f[Q];
 #pragma unroll
       for (int i = 0; i < Q; ++i) f[i] = make_float2(fa[i], fb[i]);
-      if constexpr (NOISE != kStepNoiseOff) draw_variates_pair<Q - 1, NOISE == kStepNoiseGauss>(z, s, a.ph);
-      mrt_given<LAT, float, NOISE>(f, z, a, p);
+      whole(f, s, a);
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
         fa[i] = f[i].x;
@@ -185,7 +193,7 @@ struct MrtCollide {
 
 template <int LAT, typename S, int VX, int NOISE>
 __global__ void __launch_bounds__(128, 2 * step_min_blocks<LAT, S, VX>())
-    k_step_mrt(const S *__restrict__ src, S *__restrict__ dst, const StepArgs a,
+    k_step_mrt(const S *src, S *dst, const StepArgs a,
                const MrtCollide<LAT, typename Store<S>::R, NOISE> c) {
   using C = MrtCollide<LAT, typename Store<S>::R, NOISE>;
   pdl_launch_dependents();
@@ -196,10 +204,7 @@ __global__ void __launch_bounds__(128, 2 * step_min_blocks<LAT, S, VX>())
   pdl_wait();
   if (x0 >= a.Lx || y >= a.Ly) return;
   // value offsets fit 32 bits (checked by the API)
-  if constexpr (VX == 1)
-    step_scalar_body<LAT, S, NOISE, C, uint32_t>(src, dst, a, x0, y, z, c);
-  else
-    step_vec_body<LAT, S, VX, NOISE, C, uint32_t>(src, dst, a, x0, y, z, c);
+  step_vec_body<LAT, S, VX, NOISE, C, uint32_t>(src, dst, a, x0, y, z, c);
 }
 
 // Calls go(c) with the collision of a lattice and precision: m (Q*Q, [a][i])
@@ -233,17 +238,21 @@ cudaError_t step_mrt_t(const void *src, void *dst, const StepArgs &a, const doub
                        const double *tau, cudaStream_t stream) {
   constexpr int precision = sizeof(S) == 8 ? kStoreF64 : kStoreF32;
   return mrt_collide_t<LAT, S>(a, m, w, tau, [&](auto c) -> cudaError_t {
-    constexpr int NOISE = decltype(c)::kNoise;
+    using C = decltype(c);
+    constexpr int NOISE = C::kNoise;
     const int vx = step_vec_width(LAT, precision, a.Lx, a.N);
     dim3 grid, block;
     step_shape(a.Lx, a.Ly, a.Lz, grid, block, vx, std::min(step_threads(LAT, precision), 128));
     StepLaunch launch(grid, block, stream);
     const S *s = static_cast<const S *>(src);
     S *d = static_cast<S *>(dst);
-    if constexpr (sizeof(S) == 4)
+    if (vx == 1) return cudaLaunchKernelEx(&launch.cfg, k_step<LAT, S, NOISE, uint32_t, C>, s, d, a, c);
+    if constexpr (sizeof(S) == 4) {
+      if constexpr (NOISE != kStepNoiseOff)
+        if (vx == 2) return cudaLaunchKernelEx(&launch.cfg, k_step_ahead<LAT, S, 2, NOISE, uint32_t, C>, s, d, a, c);
       if (vx == 4) return cudaLaunchKernelEx(&launch.cfg, k_step_mrt<LAT, S, 4, NOISE>, s, d, a, c);
-    if (vx == 2) return cudaLaunchKernelEx(&launch.cfg, k_step_mrt<LAT, S, 2, NOISE>, s, d, a, c);
-    return cudaLaunchKernelEx(&launch.cfg, k_step_mrt<LAT, S, 1, NOISE>, s, d, a, c);
+    }
+    return cudaLaunchKernelEx(&launch.cfg, k_step_mrt<LAT, S, 2, NOISE>, s, d, a, c);
   });
 }
 

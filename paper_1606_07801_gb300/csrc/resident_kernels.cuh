@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(resident_threads(LAT, sizeof(typename Store<S>
         constexpr int i = decltype(I)::value;
         f[i] = Store<S>::load(ld_resident<CL, S>(at[i] + from));
       });
-      collide.given(f, ahead, a);
+      collide.given(f, [&](int k) -> R { return ahead[k]; }, a);
       static_for<Q>([&](auto I) {
         constexpr int i = decltype(I)::value;
         if (last)

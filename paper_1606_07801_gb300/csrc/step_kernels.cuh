@@ -23,22 +23,22 @@ enum StepNoise : int { kStepNoiseOff = 0, kStepNoiseGauss = 1, kStepNoiseFlat = 
 // The back-transformed unit noise T_i (w_i T_i where
 // NoiseTransform::kWeighted) of site s; zero without noise.
 template <int LAT, typename R, int NOISE, typename V>
-__device__ __forceinline__ void noise_sums(V (&T)[Lattice<LAT>::Q], uint32_t s, const PhiloxStep &ph) {
+__device__ __forceinline__ void noise_sums(V (&T)[Lattice<LAT>::Q], uint32_t s, const PhiloxStep &ph,
+                                           uint32_t apart = 1u) {
   constexpr int Q = Lattice<LAT>::Q;
   static_for<Q>([&](auto I) { T[decltype(I)::value] = splat<V>(R(0)); });
   if constexpr (NOISE != kStepNoiseOff) {
     V zz[Q - 1];
     if constexpr (LaneOf<V>::kLanes == 2)
-      draw_variates_pair<Q - 1, NOISE == kStepNoiseGauss>(zz, s, ph);
+      draw_variates_pair<Q - 1, NOISE == kStepNoiseGauss>(zz, s, ph, apart);
     else
       draw_variates_t<R, Q - 1, NOISE == kStepNoiseGauss>(zz, s, ph);
     NoiseTransform<LAT, R>::apply(zz, T);
   }
 }
 
-template <int LAT, typename R, int NOISE, bool DEV, typename V>
-__device__ __forceinline__ void collide_given(V (&f)[Lattice<LAT>::Q], const V (&T)[Lattice<LAT>::Q],
-                                              const StepArgs &a) {
+template <int LAT, typename R, int NOISE, bool DEV, typename V, class TF>
+__device__ __forceinline__ void collide_given(V (&f)[Lattice<LAT>::Q], const TF &T, const StepArgs &a) {
   using L = Lattice<LAT>;
   constexpr int Q = L::Q;
   V rho = f[0];  // drho for DEV
@@ -69,9 +69,9 @@ __device__ __forceinline__ void collide_given(V (&f)[Lattice<LAT>::Q], const V (
       if constexpr (!NoiseTransform<LAT, R>::kWeighted) wsig[i] = mul_rn(cst<V>(L::w(i)), sigma);
     }
     if constexpr (NoiseTransform<LAT, R>::kWeighted) {
-      f[i] = fma_rn(omega, f[i], fma_rn(sigma, T[i], wrel[k]));
+      f[i] = fma_rn(omega, f[i], fma_rn(sigma, T(i), wrel[k]));
     } else {
-      f[i] = fma_rn(omega, f[i], fma_rn(wsig[k], T[i], wrel[k]));
+      f[i] = fma_rn(omega, f[i], fma_rn(wsig[k], T(i), wrel[k]));
     }
     moved = add_rn(moved, f[i]);
   });
@@ -82,7 +82,7 @@ template <int LAT, typename R, int NOISE, bool DEV, typename V>
 __device__ __forceinline__ void collide_lanes(V (&f)[Lattice<LAT>::Q], uint32_t s, const StepArgs &a) {
   V T[Lattice<LAT>::Q];
   noise_sums<LAT, R, NOISE>(T, s, a.ph);
-  collide_given<LAT, R, NOISE, DEV>(f, T, a);
+  collide_given<LAT, R, NOISE, DEV>(f, [&](int i) -> const V & { return T[i]; }, a);
 }
 
 // Collision of one site in registers: f holds the pulled populations
@@ -124,13 +124,20 @@ __device__ __forceinline__ void collide_pair(float (&fa)[Lattice<LAT>::Q], float
 template <int LAT, typename R, int NOISE, bool DEV = false>
 struct SrtCollide {
   static constexpr bool kPairs = std::is_same<R, float>::value;
-  // the two halves, for kernels that make the noise ahead of the update
-  static constexpr int kAhead = Lattice<LAT>::Q;  // values of the first half
-  __device__ __forceinline__ void ahead(R (&T)[kAhead], uint32_t s, const PhiloxStep &ph) const {
-    noise_sums<LAT, R, NOISE>(T, s, ph);
+  // The two halves, for kernels that make the noise ahead of the update: the
+  // kAhead values of a site (or, V = float2, of sites s and s + apart), and
+  // the update of f given ahead(k), k < kAhead.
+  static constexpr int kAhead = Lattice<LAT>::Q - 1;
+  template <typename V>
+  __device__ __forceinline__ void ahead(V (&t)[kAhead], uint32_t s, const PhiloxStep &ph, uint32_t apart = 1u) const {
+    V T[kAhead + 1];
+    noise_sums<LAT, R, NOISE>(T, s, ph, apart);
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) t[k] = T[k + 1];
   }
-  __device__ __forceinline__ void given(R (&f)[Lattice<LAT>::Q], const R (&T)[kAhead], const StepArgs &a) const {
-    collide_given<LAT, R, NOISE, DEV>(f, T, a);
+  template <typename V, class TF>
+  __device__ __forceinline__ void given(V (&f)[Lattice<LAT>::Q], const TF &t, const StepArgs &a) const {
+    collide_given<LAT, R, NOISE, DEV>(f, [&](int i) -> V { return t(i - 1); }, a);
   }
   __device__ __forceinline__ void operator()(R (&f)[Lattice<LAT>::Q], uint32_t s, const StepArgs &a) const {
     collide_site<LAT, R, NOISE, DEV>(f, s, a);
@@ -165,15 +172,14 @@ __device__ __forceinline__ uint3 sweep_block(int32_t sweep) {
   return make_uint3(gridDim.x - 1 - blockIdx.x, gridDim.y - 1 - blockIdx.y, gridDim.z - 1 - blockIdx.z);
 }
 
-// Update of site (x, y, z) of one lattice (any shape).  S is the storage
-// type (float, double, or a 16-bit deviation format with FP32 arithmetic).
-// Idx is the type of the value offsets i N + site: uint32_t when Q N < 2^32
-// (fewer address instructions), size_t otherwise.
-template <int LAT, typename S, int NOISE, class C = SrtCollideFor<LAT, S, NOISE>, typename Idx = size_t>
-__device__ __forceinline__ void step_scalar_body(const S *__restrict__ src, S *__restrict__ dst, const StepArgs &a,
-                                                 int x, int y, int z, const C &collide = C()) {
+// Pull of site (x, y, z) of one lattice (any shape) into f, returning its
+// index.  S is the storage type (float, double, or a 16-bit deviation format
+// with FP32 arithmetic), Idx the type of the value offsets i N + site:
+// uint32_t when Q N < 2^32 (fewer address instructions), size_t otherwise.
+template <int LAT, typename S, typename Idx>
+__device__ __forceinline__ uint32_t scalar_pull(const S *src, const StepArgs &a, int x, int y, int z,
+                                                typename Store<S>::R (&f)[Lattice<LAT>::Q]) {
   using L = Lattice<LAT>;
-  using R = typename Store<S>::R;
   constexpr int Q = L::Q;
   const uint32_t Lx = static_cast<uint32_t>(a.Lx), Lxy = Lx * static_cast<uint32_t>(a.Ly);
   const uint32_t Lxyz = Lxy * static_cast<uint32_t>(a.Lz);
@@ -183,9 +189,7 @@ __device__ __forceinline__ void step_scalar_body(const S *__restrict__ src, S *_
   const uint32_t dxm = x == 0 ? Lx - 1u : 0u - 1u, dxp = x + 1 == a.Lx ? 1u - Lx : 1u;
   const uint32_t dym = y == 0 ? Lxy - Lx : 0u - Lx, dyp = y + 1 == a.Ly ? Lx - Lxy : Lx;
   const uint32_t dzm = z == 0 ? Lxyz - Lxy : 0u - Lxy, dzp = z + 1 == a.Lz ? Lxy - Lxyz : Lxy;
-
-  // pull: population i arrives from x - v_i
-  R f[Q];
+  // population i arrives from x - v_i
   static_for<Q>([&](auto I) {
     constexpr int i = decltype(I)::value;
     constexpr int vx = L::v(i, 0), vy = L::v(i, 1), vz = L::v(i, 2);
@@ -195,34 +199,107 @@ __device__ __forceinline__ void step_scalar_body(const S *__restrict__ src, S *_
     const uint32_t so = s + ox + oy + oz;
     f[i] = Store<S>::load(src[static_cast<Idx>(i) * static_cast<Idx>(a.N) + so]);
   });
-  collide(f, s, a);
-  static_for<Q>([&](auto I) {
+  return s;
+}
+template <int LAT, typename S, typename Idx>
+__device__ __forceinline__ void scalar_store(S *dst, const StepArgs &a, uint32_t s,
+                                             const typename Store<S>::R (&f)[Lattice<LAT>::Q]) {
+  static_for<Lattice<LAT>::Q>([&](auto I) {
     constexpr int i = decltype(I)::value;
     dst[static_cast<Idx>(i) * static_cast<Idx>(a.N) + s] = Store<S>::store(f[i]);
   });
+}
+
+// Update of site (x, y, z) of one lattice (any shape).
+template <int LAT, typename S, int NOISE, class C = SrtCollideFor<LAT, S, NOISE>, typename Idx = size_t>
+__device__ __forceinline__ void step_scalar_body(const S *src, S *dst, const StepArgs &a,
+                                                 int x, int y, int z, const C &collide = C()) {
+  typename Store<S>::R f[Lattice<LAT>::Q];
+  const uint32_t s = scalar_pull<LAT, S, Idx>(src, a, x, y, z, f);
+  collide(f, s, a);
+  scalar_store<LAT, S, Idx>(dst, a, s, f);
 }
 
 // Programmatic dependent launch.  A step kernel lets the next kernel of its
 // stream launch once all of its own blocks have started, so the next step's
 // blocks take the SM slots that this step's last blocks free; each block then
 // waits for the previous grid's completion (and memory) before its first
-// load.  Without the launch attribute both instructions do nothing.
+// load.  Without the launch attribute both instructions do nothing.  The
+// populations' pointers of these kernels are not __restrict__: the previous
+// grid may still be writing them when a block starts, and the compiler moves
+// loads it takes for invariant across the wait.
 __device__ __forceinline__ void pdl_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// The noise of a step depends on the site and the step alone, so a kernel
+// that draws it first has work for the time in which the previous step's last
+// blocks still run: it waits for them after the noise, before its first load.
+// A lattice whose blocks fill the GPU once or a few times gains most (D3Q19
+// FP32 64^3 8.0 -> 6.1 us per step, D2Q9 FP32 512^2 4.4 -> 3.05 on GB300).
+
 // Scalar kernel: one site per thread, any lattice shape.
-template <int LAT, typename S, int NOISE, typename Idx>
-__global__ void __launch_bounds__(256) k_step(const S *__restrict__ src, S *__restrict__ dst, const StepArgs a) {
+template <int LAT, typename S, int NOISE, typename Idx, class C>
+__global__ void __launch_bounds__(256)
+    k_step(const S *src, S *dst, const StepArgs a, const C collide) {
+  using R = typename Store<S>::R;
   pdl_launch_dependents();
   const uint3 b = sweep_block(a.sweep);
   const int x = b.x * blockDim.x + threadIdx.x;
   const int y = b.y * blockDim.y + threadIdx.y;
   const int z = b.z;
-  pdl_wait();
   if (x >= a.Lx || y >= a.Ly) return;
-  step_scalar_body<LAT, S, NOISE, SrtCollideFor<LAT, S, NOISE>, Idx>(src, dst, a, x, y, z);
+  const uint32_t Lx = static_cast<uint32_t>(a.Lx);
+  R t[C::kAhead];
+  collide.ahead(t, static_cast<uint32_t>(x) + Lx * (static_cast<uint32_t>(y) + static_cast<uint32_t>(a.Ly) * static_cast<uint32_t>(z)),
+                a.ph);
+  pdl_wait();
+  R f[Lattice<LAT>::Q];
+  const uint32_t s = scalar_pull<LAT, S, Idx>(src, a, x, y, z, f);
+  collide.given(f, [&](int k) -> R { return t[k]; }, a);
+  scalar_store<LAT, S, Idx>(dst, a, s, f);
+}
+
+// Twin kernel: site x of a row's first half and site x + apart of its second
+// per thread, apart = ceil(Lx / 2), updated at once on the packed FP32
+// instructions; the loads and stores are those of the scalar kernel, so Lx
+// may be odd.  For lattices of few populations (D3Q19
+// spills: 107 us at 127 x 128 x 128 against 56).  D2Q9 FP32 1023 x 771 11.0 ->
+// 10.5 us per step, 511 x 513 5.2 -> 4.35 on GB300.
+template <int LAT, typename S, int NOISE, typename Idx>
+__global__ void __launch_bounds__(128, 6)
+    k_step_twin(const S *src, S *dst, const StepArgs a) {
+  constexpr int Q = Lattice<LAT>::Q;
+  const SrtCollideFor<LAT, S, NOISE> collide;
+  pdl_launch_dependents();
+  const uint3 b = sweep_block(a.sweep);
+  const int apart = (a.Lx + 1) / 2;
+  const int x = b.x * blockDim.x + threadIdx.x;
+  const int y = b.y * blockDim.y + threadIdx.y;
+  const int z = b.z;
+  if (x >= apart || y >= a.Ly) return;
+  const uint32_t Lx = static_cast<uint32_t>(a.Lx);
+  const uint32_t s = static_cast<uint32_t>(x) + Lx * (static_cast<uint32_t>(y) + static_cast<uint32_t>(a.Ly) * static_cast<uint32_t>(z));
+  float2 t[Q - 1];
+  collide.ahead(t, s, a.ph, static_cast<uint32_t>(apart));
+  pdl_wait();
+  // the middle of an odd row has no twin: its second site is itself, not stored
+  const bool two = x + apart < a.Lx;
+  float fa[Q], fb[Q];
+  float2 f[Q];
+  scalar_pull<LAT, S, Idx>(src, a, x, y, z, fa);
+  const uint32_t s2 = scalar_pull<LAT, S, Idx>(src, a, two ? x + apart : x, y, z, fb);
+#pragma unroll
+  for (int i = 0; i < Q; ++i) f[i] = make_float2(fa[i], fb[i]);
+  collide.given(f, [&](int k) -> float2 { return t[k]; }, a);
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    fa[i] = f[i].x;
+    fb[i] = f[i].y;
+  }
+  scalar_store<LAT, S, Idx>(dst, a, s, fa);
+  if (two) scalar_store<LAT, S, Idx>(dst, a, s2, fb);
 }
 
 // Vector kernel: VX consecutive sites of a row per thread (needs Lx % VX == 0).
@@ -331,7 +408,7 @@ __device__ __forceinline__ void collide_sites(typename Store<S>::R (&f)[VX][Latt
 // the first half of step_vec_body (Lx % VX == 0).  Returns the row offset
 // Lx (y + Ly z) of the sites.
 template <int LAT, typename S, int VX, typename Idx>
-__device__ __forceinline__ uint32_t vec_pull(const S *__restrict__ src, const StepArgs &a, int x0, int y, int z,
+__device__ __forceinline__ uint32_t vec_pull(const S *src, const StepArgs &a, int x0, int y, int z,
                                              typename Store<S>::R (&f)[VX][Lattice<LAT>::Q]) {
   using L = Lattice<LAT>;
   using R = typename Store<S>::R;
@@ -371,7 +448,7 @@ __device__ __forceinline__ uint32_t vec_pull(const S *__restrict__ src, const St
 // Store of f*_i of sites (x0 .. x0 + VX - 1) of the row at offset `row`:
 // the second half of step_vec_body (VX-wide stores).
 template <int LAT, typename S, int VX, typename Idx>
-__device__ __forceinline__ void vec_store(S *__restrict__ dst, const StepArgs &a, uint32_t row, int x0,
+__device__ __forceinline__ void vec_store(S *dst, const StepArgs &a, uint32_t row, int x0,
                                           const typename Store<S>::R (&f)[VX][Lattice<LAT>::Q]) {
   using R = typename Store<S>::R;
   using P = Pack<S, VX>;
@@ -386,7 +463,7 @@ __device__ __forceinline__ void vec_store(S *__restrict__ dst, const StepArgs &a
 }
 
 template <int LAT, typename S, int VX, int NOISE, class C = SrtCollideFor<LAT, S, NOISE>, typename Idx = size_t>
-__device__ __forceinline__ void step_vec_body(const S *__restrict__ src, S *__restrict__ dst, const StepArgs &a, int x0,
+__device__ __forceinline__ void step_vec_body(const S *src, S *dst, const StepArgs &a, int x0,
                                               int y, int z, const C &collide = C()) {
   typename Store<S>::R f[VX][Lattice<LAT>::Q];
   const uint32_t row = vec_pull<LAT, S, VX, Idx>(src, a, x0, y, z, f);
@@ -402,7 +479,7 @@ __device__ __forceinline__ void step_vec_body(const S *__restrict__ src, S *__re
 
 template <int LAT, typename S, int VX, int NOISE, typename Idx>
 __global__ void __launch_bounds__(256, step_min_blocks<LAT, S, VX>())
-    k_step_vec(const S *__restrict__ src, S *__restrict__ dst, const StepArgs a) {
+    k_step_vec(const S *src, S *dst, const StepArgs a) {
   pdl_launch_dependents();
   const uint3 b = sweep_block(a.sweep);
   const int x0 = (b.x * blockDim.x + threadIdx.x) * VX;
@@ -411,6 +488,72 @@ __global__ void __launch_bounds__(256, step_min_blocks<LAT, S, VX>())
   pdl_wait();
   if (x0 >= a.Lx || y >= a.Ly) return;
   step_vec_body<LAT, S, VX, NOISE, SrtCollideFor<LAT, S, NOISE>, Idx>(src, dst, a, x0, y, z);
+}
+
+// Vector kernel with the noise ahead: the variates' sums of the thread's
+// sites, two sites per packed instruction, wait in the thread's own column of
+// shared memory while it pulls the populations, so that neither half holds
+// the other's registers: two D3Q19 sites fit 64-72 registers paired, where the
+// one-piece form spills at 80.
+template <int LAT, typename S, int VX>
+constexpr int ahead_min_blocks() {  // 128-thread blocks
+  return LAT == kD3Q19 ? 7 : (Store<S>::kDeviation ? 7 : 6);
+}
+template <int LAT, typename S, int VX, int NOISE, typename Idx, class C>
+__global__ void __launch_bounds__(128, ahead_min_blocks<LAT, S, VX>())
+    k_step_ahead(const S *src, S *dst, const StepArgs a, const C collide) {
+  constexpr int Q = Lattice<LAT>::Q, K = C::kAhead;
+  __shared__ float2 column[VX / 2][K][128];
+  pdl_launch_dependents();
+  const uint3 b = sweep_block(a.sweep);
+  const int x0 = (b.x * blockDim.x + threadIdx.x) * VX;
+  const int y = b.y * blockDim.y + threadIdx.y;
+  const int z = b.z;
+  if (x0 >= a.Lx || y >= a.Ly) return;
+  const uint32_t s0 = static_cast<uint32_t>(x0) + static_cast<uint32_t>(a.Lx) *
+                      (static_cast<uint32_t>(y) + static_cast<uint32_t>(a.Ly) * static_cast<uint32_t>(z));
+  const uint32_t at = static_cast<uint32_t>(__cvta_generic_to_shared(&column[0][0][threadIdx.x + blockDim.x * threadIdx.y]));
+  auto slot = [&](int p, int k) { return at + static_cast<uint32_t>((p * K + k) * 128 * sizeof(float2)); };
+  // volatile: the compiler may not carry the values past the pull in registers
+#pragma unroll
+  for (int p = 0; p < VX / 2; ++p) {
+    float2 t[K];
+    collide.ahead(t, s0 + 2u * static_cast<uint32_t>(p), a.ph);
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(slot(p, k)), "f"(t[k].x), "f"(t[k].y));
+  }
+  pdl_wait();
+  float f[VX][Q];
+  const uint32_t row = vec_pull<LAT, S, VX, Idx>(src, a, x0, y, z, f);
+#pragma unroll
+  for (int p = 0; p < VX / 2; ++p) {
+    float2 g[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) g[i] = make_float2(f[2 * p][i], f[2 * p + 1][i]);
+    collide.given(g, [&](int k) -> float2 {
+      float2 t;
+      asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(t.x), "=f"(t.y) : "r"(slot(p, k)));
+      return t;
+    }, a);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      f[2 * p][i] = g[i].x;
+      f[2 * p + 1][i] = g[i].y;
+    }
+  }
+  vec_store<LAT, S, VX, Idx>(dst, a, row, x0, f);
+}
+// Where k_step_ahead replaces k_step_vec (noisy steps in FP32 arithmetic),
+// microseconds per step on GB300: D3Q19 FP32 at every size (256^3 390 -> 375,
+// 1.004 of the copy bandwidth),
+// D3Q19 16-bit below the sizes of four sites per thread (64^3 7.95 -> 6.3; at
+// 256^3 351 against 356), D2Q9 FP32 below 2^21 sites (1024^2 11.5 -> 10.7,
+// 2048^2 45.1 against 45.3) and D2Q9 16-bit (2048^2 40.0 -> 39.2).
+template <int LAT, typename S>
+inline bool step_ahead(int vx, int64_t sites) {
+  if (LAT == kD3Q19) return vx == 2;
+  return LAT == kD2Q9 && (Store<S>::kDeviation || sites < (int64_t(1) << 21));
 }
 
 // True when every value offset i N + site of a lattice fits 32 bits.
@@ -450,10 +593,26 @@ cudaError_t step_noise_idx(const S *s, S *d, const StepArgs &a, int vx, cudaStre
   dim3 grid, block;
   step_shape(a.Lx, a.Ly, a.Lz, grid, block, vx, step_threads(LAT, sizeof(typename Store<S>::R) == 8 ? kStoreF64 : kStoreF32));
   StepLaunch launch(grid, block, stream);
-  if (vx == 2) return cudaLaunchKernelEx(&launch.cfg, k_step_vec<LAT, S, 2, NOISE, Idx>, s, d, a);
-  if constexpr (sizeof(typename Store<S>::R) == 4)
+  const SrtCollideFor<LAT, S, NOISE> c;
+  using C = SrtCollideFor<LAT, S, NOISE>;
+  if constexpr (sizeof(typename Store<S>::R) == 4) {
+    if constexpr (NOISE != kStepNoiseOff && LAT != kD1Q3) {
+      if (vx > 1 && step_ahead<LAT, S>(vx, a.N)) {
+        if (vx == 2) return cudaLaunchKernelEx(&launch.cfg, k_step_ahead<LAT, S, 2, NOISE, Idx, C>, s, d, a, c);
+        if constexpr (LAT != kD3Q19)
+          return cudaLaunchKernelEx(&launch.cfg, k_step_ahead<LAT, S, 4, NOISE, Idx, C>, s, d, a, c);
+      }
+    }
+    if constexpr (NOISE != kStepNoiseOff && LAT == kD2Q9) {
+      if (vx == 1 && a.Lx % 2 != 0 && step_vec_width(LAT, kStoreF32, 4, a.N) > 1) {  // above the smallest sizes
+        step_shape((a.Lx + 1) / 2, a.Ly, a.Lz, launch.cfg.gridDim, launch.cfg.blockDim, 1, 128);
+        return cudaLaunchKernelEx(&launch.cfg, k_step_twin<LAT, S, NOISE, Idx>, s, d, a);
+      }
+    }
     if (vx == 4) return cudaLaunchKernelEx(&launch.cfg, k_step_vec<LAT, S, 4, NOISE, Idx>, s, d, a);
-  return cudaLaunchKernelEx(&launch.cfg, k_step<LAT, S, NOISE, Idx>, s, d, a);
+  }
+  if (vx == 2) return cudaLaunchKernelEx(&launch.cfg, k_step_vec<LAT, S, 2, NOISE, Idx>, s, d, a);
+  return cudaLaunchKernelEx(&launch.cfg, k_step<LAT, S, NOISE, Idx, C>, s, d, a, c);
 }
 
 template <int LAT, typename S, int NOISE>
