@@ -382,8 +382,8 @@ int lbfd_mass_noalloc(int32_t lattice, int32_t precision, const void *f_dev, int
  * would under lbfd_create_ex with the same parameters (same arithmetic,
  * same noise keys).  Members share one precision, noise mode and law, and
  * each member has Q * sites < 2^32.  Work decomposition: a work item is 1
- * or 2 sites of a row (2 only where Lx is even), a tile is `passes` x 256
- * items of one member, and the tiles go to blocks in one of the orders
+ * or 2 sites of a row (neighbours where Lx is even, else one of each half of
+ * the row), a tile is at most `passes` x 256 items of one member, and the tiles go to blocks in one of the orders
  * LBFD_WALK_* (see lbfd_ensemble_tune / lbfd_ensemble_plan). */
 typedef struct lbfd_member {
     int64_t dims[3];    /* Lx, Ly, Lz; trailing dims of lower-D lattices must be 1 */
@@ -503,8 +503,8 @@ typedef struct lbfd_server_options {
                                _PER_TILE (default) or _PARAM (the members' arguments in the kernel
                                parameters, one launch per group of up to 112 residents, regrouped
                                whenever the resident set changes) */
-    int32_t vx_max;         /* sites per work item of the batched kernel at most: 2 (members with even Lx
-                               take two) or 1 (a kernel without the two-site path, fewer registers) */
+    int32_t vx_max;         /* sites per work item of the batched kernel at most: 2 (pairs of sites where
+                               that is faster) or 1 (a kernel without the two-site path, fewer registers) */
     int32_t reserved[5];
     int64_t solo_sites;     /* simulations of at least this many sites are stepped by their own
                                single-lattice launch (parameters as kernel arguments) instead of the

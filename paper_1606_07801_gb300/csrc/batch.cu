@@ -17,8 +17,8 @@ __global__ void k_batch_prep(const BatchMember *__restrict__ members, int n, con
     out[m] = batch_step_of(members[m], now, noise_mode, noise_dist);
 }
 
-__global__ void k_clock_advance(uint64_t *clock_dev) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) *clock_dev += 1;
+__global__ void k_clock_advance(uint64_t *clock_dev, uint64_t by) {
+  if (threadIdx.x == 0 && blockIdx.x == 0) *clock_dev += by;
 }
 
 cudaError_t launch_batch_prep(const BatchMember *members, int n, const uint64_t *clock_dev, uint64_t clock,
@@ -29,8 +29,8 @@ cudaError_t launch_batch_prep(const BatchMember *members, int n, const uint64_t 
   return cudaGetLastError();
 }
 
-cudaError_t launch_clock_advance(uint64_t *clock_dev, cudaStream_t stream) {
-  k_clock_advance<<<1, 32, 0, stream>>>(clock_dev);
+cudaError_t launch_clock_advance(uint64_t *clock_dev, cudaStream_t stream, uint64_t by) {
+  k_clock_advance<<<1, 32, 0, stream>>>(clock_dev, by);
   return cudaGetLastError();
 }
 
@@ -52,17 +52,17 @@ cudaError_t launch_batch_step(int lattice, int precision, void *base, const Batc
 }
 
 cudaError_t launch_batch_param(int lattice, int precision, void *base, const BatchParams *groups, int ngroups,
-                               const BatchStep *steps, int passes, int occ, int vx_max, int noise_mode, int noise_dist,
+                               const BatchWhen &when, int passes, int occ, int vx_max, int noise_mode, int noise_dist,
                                cudaStream_t stream) {
   switch (lattice) {
     case kD1Q3:
-      return launch_batch_param_d1q3(precision, base, groups, ngroups, steps, passes, occ, vx_max, noise_mode,
+      return launch_batch_param_d1q3(precision, base, groups, ngroups, when, passes, occ, vx_max, noise_mode,
                                      noise_dist, stream);
     case kD2Q9:
-      return launch_batch_param_d2q9(precision, base, groups, ngroups, steps, passes, occ, vx_max, noise_mode,
+      return launch_batch_param_d2q9(precision, base, groups, ngroups, when, passes, occ, vx_max, noise_mode,
                                      noise_dist, stream);
     case kD3Q19:
-      return launch_batch_param_d3q19(precision, base, groups, ngroups, steps, passes, occ, vx_max, noise_mode,
+      return launch_batch_param_d3q19(precision, base, groups, ngroups, when, passes, occ, vx_max, noise_mode,
                                       noise_dist, stream);
   }
   return cudaErrorInvalidValue;
@@ -77,13 +77,13 @@ int batch_blocks_per_sm(int lattice, int precision, int occ, int vx_max, int wal
   return 1;
 }
 
-BatchMember make_batch_member(const int64_t dims[3], double tau, double rho_mean, uint64_t seed, uint32_t lattice_id,
-                              int64_t off0, int64_t off1, uint64_t t0, int vx_max) {
+BatchMember make_batch_member(int lattice, const int64_t dims[3], double tau, double rho_mean, uint64_t seed, uint32_t lattice_id,
+                              int64_t off0, int64_t off1, uint64_t t0, int vx_max, int precision) {
   BatchMember m{};
   m.Lx = static_cast<int32_t>(dims[0]);
   m.Ly = static_cast<int32_t>(dims[1]);
   m.Lz = static_cast<int32_t>(dims[2]);
-  m.vx = (vx_max >= 2 && m.Lx % 2 == 0) ? 2 : 1;
+  m.vx = batch_vx(lattice, m.Lx, vx_max, precision);
   m.N = dims[0] * dims[1] * dims[2];
   m.off[0] = off0;
   m.off[1] = off1;
@@ -107,6 +107,9 @@ int batch_build_params(const BatchMember *members, int n, int64_t ntiles, int no
       const BatchMember &mb = members[first + k];
       p.tile_start[k] = static_cast<int32_t>(mb.tile0 - base);
       p.mem[k] = batch_step_of(mb, mb.t0, noise_mode, noise_dist);
+      p.mem[k].a.ph.e[0] = static_cast<uint32_t>(mb.t0);
+      p.mem[k].a.ph.e[1] = static_cast<uint32_t>(mb.t0 >> 32);
+      p.mem[k].a.ph.f = mb.lattice_id;
     }
     const int64_t end = first + p.n < n ? members[first + p.n].tile0 : ntiles;
     p.tile_start[p.n] = static_cast<int32_t>(end - base);
@@ -115,12 +118,19 @@ int batch_build_params(const BatchMember *members, int n, int64_t ntiles, int no
   return static_cast<int>(groups.size());
 }
 
+int batch_passes(const BatchMember *members, int n, int passes, int64_t slots) {
+  int64_t items = 0;
+  for (int m = 0; m < n; ++m) items += int64_t((members[m].Lx + members[m].vx - 1) / members[m].vx) * members[m].Ly * members[m].Lz;
+  while (passes > 1 && items < 4 * slots * passes * kBatchThreads) passes /= 2;
+  return passes;
+}
+
 int64_t batch_assign_tiles(BatchMember *members, int n, int passes, int64_t *tile_start) {
   const int64_t per_tile = int64_t(passes) * kBatchThreads;
   int64_t next = 0;
   for (int m = 0; m < n; ++m) {
     BatchMember &mb = members[m];
-    const int64_t items = int64_t(mb.Lx / mb.vx) * mb.Ly * mb.Lz;
+    const int64_t items = int64_t((mb.Lx + mb.vx - 1) / mb.vx) * mb.Ly * mb.Lz;
     mb.tile0 = next;
     tile_start[m] = next;
     next += (items + per_tile - 1) / per_tile;

@@ -8,17 +8,28 @@
 
 namespace lbfd {
 
-// A member of a batched launch: vx is 2 when vx_max >= 2 and Lx is even,
-// else 1; the two population blocks start at value offsets off0 and off1 of
+// Sites per work item: 2 when vx_max >= 2 and Lx is even, and for odd Lx in
+// FP32 arithmetic but for D3Q19, whose twins measured slower than one site
+// (32.3 against 36.0 GLUPS; the pairs' registers and scalar loads together).
+inline int batch_vx(int lattice, int32_t Lx, int vx_max, int precision) {
+  return vx_max >= 2 && (Lx % 2 == 0 || (precision != kStoreF64 && lattice != kD3Q19)) ? 2 : 1;
+}
+
+// A member of a batched launch (vx by batch_vx); the two population blocks start at value offsets off0 and off1 of
 // the batch buffer; t0 is the batch clock value at which its t is 0.
-BatchMember make_batch_member(const int64_t dims[3], double tau, double rho_mean, uint64_t seed, uint32_t lattice_id,
-                              int64_t off0, int64_t off1, uint64_t t0, int vx_max);
+BatchMember make_batch_member(int lattice, const int64_t dims[3], double tau, double rho_mean, uint64_t seed, uint32_t lattice_id,
+                              int64_t off0, int64_t off1, uint64_t t0, int vx_max, int precision);
 
 // Groups of at most kParamMembers consecutive members with their
 // t-independent arguments, for the parameter-space launches (tile order 3);
 // tile0 of every member must be assigned.  Returns the number of groups.
 int batch_build_params(const BatchMember *members, int n, int64_t ntiles, int noise_mode, int noise_dist,
                        std::vector<BatchParams> &groups);
+
+// Tile passes for a launch of the members: at most `passes`, fewer where the
+// tiles would not fill the GPU's `slots` resident blocks four times (a last
+// wave that is nearly empty costs more than longer tiles save).
+int batch_passes(const BatchMember *members, int n, int passes, int64_t slots);
 
 // Assigns consecutive tiles of passes x 256 items to members[0..n) in order
 // (tile0 and tile_start[m]); returns the number of tiles.

@@ -11,9 +11,11 @@
 //
 // Work.  Member m owns tiles [tile_start[m], tile_start[m + 1]) of a flat
 // tile list; a tile is `passes` x 256 consecutive work items of one member,
-// and an item is vx sites of a row (vx = 2 for even Lx, else 1).  Every item
-// runs the per-site code of the single-lattice kernels, so a member evolves
-// bit-identically to the same lattice stepped alone.  The step arguments
+// and an item is vx sites of a row: neighbours where Lx is even, a site of the
+// row's first half and its twin in the second where it is odd (twin_update;
+// D3Q19 takes one site there).
+// Every item runs the per-site code of the single-lattice kernels, so a member
+// evolves bit-identically to the same lattice stepped alone.  The step arguments
 // (relaxation constants and the Philox words of the member's t) are written
 // once per launch and member by k_batch_prep.  Three kernels take the tiles:
 //   k_batch_tile   one block per tile; warp 0 finds the member by a 32-way
@@ -21,8 +23,8 @@
 //                  memory;
 //   k_batch_param  one block per tile, one launch per group of up to
 //                  kParamMembers members whose t-independent arguments are a
-//                  kernel parameter (uniform operands, fewer registers); only
-//                  the t words come from k_batch_prep's output;
+//                  kernel parameter (uniform operands, fewer registers); the
+//                  t words are formed in the block, without k_batch_prep;
 //   k_batch_step   a persistent grid whose blocks take every grid-th tile or
 //                  one run of consecutive tiles, reloading the arguments when
 //                  the member changes.
@@ -42,7 +44,7 @@ constexpr int kWalkStrided = 0, kWalkContiguous = 1, kWalkPerTile = 2, kWalkPara
 
 // One member, as the host builds it (constant while the member is listed).
 struct BatchMember {
-  int32_t Lx, Ly, Lz, vx;  // vx: sites per work item, 1 or 2 (2 needs Lx even)
+  int32_t Lx, Ly, Lz, vx;  // vx: sites per work item, 1 or 2 (batch_vx)
   int64_t N;               // sites
   int64_t off[2];          // first value of population block 0 / 1 in the batch buffer
   int64_t tile0;           // first tile of the member in the launch's tile list
@@ -84,7 +86,7 @@ __host__ __device__ inline BatchStep batch_step_of(const BatchMember &mb, uint64
   s.dst = mb.off[p ^ 1];
   s.tile0 = mb.tile0;
   s.vx = mb.vx;
-  s.cols = mb.Lx / mb.vx;
+  s.cols = (mb.Lx + mb.vx - 1) / mb.vx;
   s.items = static_cast<int32_t>(static_cast<int64_t>(s.cols) * mb.Ly * mb.Lz);
   s.div_cols = make_fastdiv(static_cast<uint32_t>(s.cols));
   s.div_Ly = make_fastdiv(static_cast<uint32_t>(mb.Ly));
@@ -116,28 +118,45 @@ __device__ __forceinline__ int batch_find_member(const int64_t *__restrict__ til
 }
 
 // Minimum resident blocks per SM asked of the register allocator: occupancy
-// variant 0 is the single-lattice kernel's choice, variant 1 one block fewer
-// (more registers per thread, no spills); the tuner picks between them.
-template <int LAT, typename S, int OCC>
+// variant 0 is 4 blocks (64 registers; D3Q19 with its arguments in shared
+// memory, which the compiler cannot keep as uniform operands, 3; FP64 2),
+// variant 1 one block fewer; the tuner picks between them.
+template <int LAT, typename S, int OCC, bool PARAM>
 constexpr int batch_min_blocks() {
-  return OCC == 0 ? step_min_blocks<LAT, S>() : (step_min_blocks<LAT, S>() > 1 ? step_min_blocks<LAT, S>() - 1 : 1);
+  return (sizeof(typename Store<S>::R) != 4 ? 2 : (LAT == kD3Q19 && !PARAM ? 3 : 4)) - OCC;
 }
 
-// The collision of the batched kernels: one site at a time.  With the
-// one-site and two-site item paths in one kernel, colliding two sites at once
-// on the packed instructions measured slower (D2Q9 ensemble of 4096
-// lattices: 78.6 against 81.2 GLUPS); the results are the same either way.
+// The collision of pairs without the packed form (FP64, no noise): one site
+// at a time.
 template <int LAT, typename S, int NOISE>
 struct BatchCollide : SrtCollideFor<LAT, S, NOISE> {
   static constexpr bool kPairs = false;
 };
 
+// Shared memory of the pair items' noise (NoiseColumn) of one block.
+template <int LAT, typename S, int NOISE, int VXMAX>
+__host__ __device__ constexpr int batch_column() {
+  return VXMAX == 2 && NOISE != kStepNoiseOff && sizeof(typename Store<S>::R) == 4
+             ? SrtCollideFor<LAT, S, NOISE>::kAhead * kBatchThreads
+             : 1;
+}
+
 // The work items of one tile of member b (rel: the tile's index within the
 // member).  VXMAX = 1: every member takes one site per item (the two-site
-// path, with its larger register footprint, is not compiled in); VXMAX = 2:
-// members with even Lx take two.
-template <int LAT, typename S, int NOISE, int VXMAX>
-__device__ __forceinline__ void batch_tile_items(S *__restrict__ base, const BatchStep &b, int rel, int passes) {
+// path is not compiled in).  A pair of sites is updated at once on the packed
+// FP32 instructions with its noise parked in `column`, in FP64 and without
+// noise one site at a time.  Measured on GB300 in the parameter-space
+// launches, against one site at a time from registers with the arguments
+// prepared by a launch of its own: 60 D2Q9 members of 96..512 a side 62.8 ->
+// 80.0 GLUPS with even rows, 59.4 -> 73.3 odd; 40 D3Q19 members of 32..128 a
+// side 36.9 -> 42.1 even, 33.4 -> 36.0 odd.
+// ready() is called before an item's first load.
+template <int LAT, typename S, int NOISE, int VXMAX, class F>
+__device__ __forceinline__ void batch_tile_items(S *base, const BatchStep &b, int rel, int passes, float2 *column,
+                                                 F &&ready) {
+  using C = SrtCollideFor<LAT, S, NOISE>;
+  constexpr bool kPacked = NOISE != kStepNoiseOff && sizeof(typename Store<S>::R) == 4;
+  const C collide;
   const S *src = base + b.src;
   S *dst = base + b.dst;
   const int first = rel * passes * kBatchThreads + threadIdx.x;
@@ -149,11 +168,41 @@ __device__ __forceinline__ void batch_tile_items(S *__restrict__ base, const Bat
       const int z = static_cast<int>(fastdiv(static_cast<uint32_t>(row), b.div_Ly));
       const int y = row - z * b.a.Ly;
       // a member's value offsets fit 32 bits (checked when it is listed)
-      using C = BatchCollide<LAT, S, NOISE>;
-      if (VXMAX == 2 && b.vx == 2)
-        step_vec_body<LAT, S, 2, NOISE, C, uint32_t>(src, dst, b.a, col * 2, y, z);
-      else
-        step_scalar_body<LAT, S, NOISE, C, uint32_t>(src, dst, b.a, col, y, z);
+      if (VXMAX == 2 && b.vx == 2) {
+        if constexpr (kPacked) {
+          const NoiseColumn<C::kAhead, kBatchThreads> nc(column, static_cast<int>(threadIdx.x));
+          if (LAT != kD3Q19 && (b.a.Lx & 1)) {  // (D3Q19: batch_vx)
+            twin_update<LAT, S, uint32_t>(src, dst, b.a, col, y, z, collide, nc, ready);
+          } else {
+            float2 t[C::kAhead];
+            collide.ahead(t, site_index(b.a, 2 * col, y, z), b.a.ph);
+#pragma unroll
+            for (int k = 0; k < C::kAhead; ++k) nc.put(k, t[k]);
+            ready();
+            float f[2][Lattice<LAT>::Q];
+            const uint32_t at = vec_pull<LAT, S, 2, uint32_t>(src, b.a, 2 * col, y, z, f);
+            collide_parked(collide, f[0], f[1], nc, 0, b.a);
+            vec_store<LAT, S, 2, uint32_t>(dst, b.a, at, 2 * col, f);
+          }
+        } else if (b.a.Lx & 1) {
+          ready();
+          const int apart = b.cols;
+          step_scalar_body<LAT, S, NOISE, C, uint32_t>(src, dst, b.a, col, y, z);
+          if (col + apart < b.a.Lx) step_scalar_body<LAT, S, NOISE, C, uint32_t>(src, dst, b.a, col + apart, y, z);
+        } else {
+          ready();
+          step_vec_body<LAT, S, 2, NOISE, BatchCollide<LAT, S, NOISE>, uint32_t>(src, dst, b.a, col * 2, y, z);
+        }
+      } else {
+        using R = typename Store<S>::R;
+        R t[C::kAhead];
+        collide.ahead(t, site_index(b.a, col, y, z), b.a.ph);
+        ready();
+        R f[Lattice<LAT>::Q];
+        const uint32_t s = scalar_pull<LAT, S, uint32_t>(src, b.a, col, y, z, f);
+        collide.given(f, [&](int k) -> R { return t[k]; }, b.a);
+        scalar_store<LAT, S, uint32_t>(dst, b.a, s, f);
+      }
     }
   }
 }
@@ -180,7 +229,7 @@ __device__ __forceinline__ void batch_load_member(const BatchStep *__restrict__ 
 // walk), in which the member changes only where the run crosses a member
 // boundary.
 template <int LAT, typename S, int NOISE, int OCC, int VXMAX>
-__global__ void __launch_bounds__(kBatchThreads, batch_min_blocks<LAT, S, OCC>())
+__global__ void __launch_bounds__(kBatchThreads, batch_min_blocks<LAT, S, OCC, false>())
     k_batch_step(S *__restrict__ base, const BatchStep *__restrict__ steps, const int64_t *__restrict__ tile_start,
                  int nmembers, int ntiles, int passes, int walk) {
   int tile, stop, stride;
@@ -198,6 +247,7 @@ __global__ void __launch_bounds__(kBatchThreads, batch_min_blocks<LAT, S, OCC>()
   // one any more (one barrier per change of member)
   __shared__ BatchStep sb[2];
   __shared__ int srange[2][2];
+  __shared__ float2 column[batch_column<LAT, S, NOISE, VXMAX>()];
   int buf = 1, lo = 0, hi = 0;
   for (; tile < stop; tile += stride) {
     if (tile < lo || tile >= hi) {
@@ -207,7 +257,7 @@ __global__ void __launch_bounds__(kBatchThreads, batch_min_blocks<LAT, S, OCC>()
       lo = srange[buf][0];
       hi = srange[buf][1];
     }
-    batch_tile_items<LAT, S, NOISE, VXMAX>(base, sb[buf], tile - lo, passes);
+    batch_tile_items<LAT, S, NOISE, VXMAX>(base, sb[buf], tile - lo, passes, column, [] {});
   }
 }
 
@@ -215,34 +265,40 @@ __global__ void __launch_bounds__(kBatchThreads, batch_min_blocks<LAT, S, OCC>()
 // across tiles, which leaves the per-site code the registers it has in the
 // single-lattice kernels.
 template <int LAT, typename S, int NOISE, int OCC, int VXMAX>
-__global__ void __launch_bounds__(kBatchThreads, batch_min_blocks<LAT, S, OCC>())
+__global__ void __launch_bounds__(kBatchThreads, batch_min_blocks<LAT, S, OCC, false>())
     k_batch_tile(S *__restrict__ base, const BatchStep *__restrict__ steps, const int64_t *__restrict__ tile_start,
                  int nmembers, int ntiles, int passes) {
   __shared__ BatchStep sb;
   __shared__ int lo;
+  __shared__ float2 column[batch_column<LAT, S, NOISE, VXMAX>()];
   batch_load_member(steps, tile_start, nmembers, ntiles, static_cast<int>(blockIdx.x), &sb, &lo, nullptr);
   __syncthreads();
-  batch_tile_items<LAT, S, NOISE, VXMAX>(base, sb, static_cast<int>(blockIdx.x) - lo, passes);
+  batch_tile_items<LAT, S, NOISE, VXMAX>(base, sb, static_cast<int>(blockIdx.x) - lo, passes, column, [] {});
 }
 
 // Members of one parameter-space launch (tile order LBFD_WALK_PARAM): the
 // t-independent arguments of at most kParamMembers consecutive members travel
 // as a kernel parameter (30.9 KB of the 32 KB parameter space), so the
 // per-site code reads them as uniform operands, as the single-lattice kernels
-// read theirs.  Only the Philox words of the member's t and the parity of its
-// blocks come from the BatchStep that k_batch_prep writes for the launch.
+// read theirs.  The Philox words of the member's t and the parity of its
+// blocks are formed by every block from the clock (a dozen instructions per
+// thread and tile), so nothing has to be prepared between two steps of a
+// group: its launches follow each other as dependent launches.
 constexpr int kParamMembers = 112;
 struct BatchParams {
   int32_t n, first;                      // members first .. first + n - 1 of the batch
   int32_t tile_start[kParamMembers + 1];  // first tile of each, relative to the launch; [n] = tiles
-  BatchStep mem[kParamMembers];          // arguments at t = 0 (the t words are replaced)
+  BatchStep mem[kParamMembers];          // arguments at t = 0; a.ph.e[0..1] hold t0 and a.ph.f the lattice id
 };
 static_assert(sizeof(BatchParams) + 64 <= 32764, "kernel parameters are limited to 32764 bytes");
 
+// clock: the batch clock of this step is *clock_dev (0 where null) + clock.
 template <int LAT, typename S, int NOISE, int OCC, int VXMAX>
-__global__ void __launch_bounds__(kBatchThreads, batch_min_blocks<LAT, S, OCC>())
-    k_batch_param(S *__restrict__ base, const __grid_constant__ BatchParams p, const BatchStep *__restrict__ steps,
+__global__ void __launch_bounds__(kBatchThreads, batch_min_blocks<LAT, S, OCC, true>())
+    k_batch_param(S *base, const __grid_constant__ BatchParams p, const uint64_t *clock_dev, uint64_t clock,
                   int passes) {
+  __shared__ float2 column[batch_column<LAT, S, NOISE, VXMAX>()];
+  pdl_launch_dependents();
   const int tile = static_cast<int>(blockIdx.x);
   // the member of this block: a search of uniform (parameter) words
   int lo = 0, hi = p.n;
@@ -253,51 +309,62 @@ __global__ void __launch_bounds__(kBatchThreads, batch_min_blocks<LAT, S, OCC>()
     else
       hi = mid;
   }
+  // (the clock does not change while launches that read it may run)
   BatchStep b = p.mem[lo];
-  const BatchStep &s = steps[p.first + lo];
-  // the t words: e[j] = ((t_hi << 3) | j) ^ K1[0] = e[0] ^ j for j < 8
-  const uint32_t e0 = s.a.ph.e[0];
-#pragma unroll
-  for (int j = 0; j < 8; ++j) b.a.ph.e[j] = e0 ^ static_cast<uint32_t>(j);
-  b.a.ph.f = s.a.ph.f;
-  b.a.ph.g = s.a.ph.g;
-  b.a.ph.q = s.a.ph.q;
-  b.src = s.src;
-  b.dst = s.dst;
-  batch_tile_items<LAT, S, NOISE, VXMAX>(base, b, tile - p.tile_start[lo], passes);
+  const uint64_t t0 = static_cast<uint64_t>(b.a.ph.e[1]) << 32 | b.a.ph.e[0];
+  const uint64_t t = (clock_dev ? *clock_dev : 0) + clock - t0;  // the member's own step counter
+  philox_step_set_t(b.a.ph, b.a.ph.f, t);
+  if (t & 1) {
+    const int64_t src = b.src;
+    b.src = b.dst;
+    b.dst = src;
+  }
+  batch_tile_items<LAT, S, NOISE, VXMAX>(base, b, tile - p.tile_start[lo], passes, column, [] { pdl_wait(); });
 }
 
+// When a launch happens: batch clock, and whether it may start before the
+// previous launch of its stream has ended (its blocks wait for it).
+struct BatchWhen {
+  const uint64_t *clock_dev;
+  uint64_t clock;
+  bool dependent;
+};
+
 template <int LAT, typename S, int NOISE, int OCC, int VXMAX>
-cudaError_t batch_param_k(S *b, const BatchParams *groups, int ngroups, const BatchStep *steps, int passes,
+cudaError_t batch_param_k(S *b, const BatchParams *groups, int ngroups, const BatchWhen &when, int passes,
                           cudaStream_t stream) {
   for (int g = 0; g < ngroups; ++g) {
     const int tiles = groups[g].tile_start[groups[g].n];
-    if (tiles > 0)
-      k_batch_param<LAT, S, NOISE, OCC, VXMAX><<<tiles, kBatchThreads, 0, stream>>>(b, groups[g], steps, passes);
+    if (tiles <= 0) continue;
+    StepLaunch launch(dim3(tiles), dim3(kBatchThreads), stream);
+    if (!when.dependent) launch.cfg.numAttrs = 0;
+    const cudaError_t e = cudaLaunchKernelEx(&launch.cfg, k_batch_param<LAT, S, NOISE, OCC, VXMAX>, b, groups[g],
+                                             when.clock_dev, when.clock, passes);
+    if (e != cudaSuccess) return e;
   }
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 template <int LAT, typename S, int OCC, int VXMAX>
-cudaError_t batch_param_occ(S *b, const BatchParams *groups, int ngroups, const BatchStep *steps, int passes,
+cudaError_t batch_param_occ(S *b, const BatchParams *groups, int ngroups, const BatchWhen &when, int passes,
                             int noise_mode, int noise_dist, cudaStream_t stream) {
   if (noise_mode == kNoiseOff)
-    return batch_param_k<LAT, S, kStepNoiseOff, OCC, VXMAX>(b, groups, ngroups, steps, passes, stream);
+    return batch_param_k<LAT, S, kStepNoiseOff, OCC, VXMAX>(b, groups, ngroups, when, passes, stream);
   if (noise_dist == kGaussian)
-    return batch_param_k<LAT, S, kStepNoiseGauss, OCC, VXMAX>(b, groups, ngroups, steps, passes, stream);
-  return batch_param_k<LAT, S, kStepNoiseFlat, OCC, VXMAX>(b, groups, ngroups, steps, passes, stream);
+    return batch_param_k<LAT, S, kStepNoiseGauss, OCC, VXMAX>(b, groups, ngroups, when, passes, stream);
+  return batch_param_k<LAT, S, kStepNoiseFlat, OCC, VXMAX>(b, groups, ngroups, when, passes, stream);
 }
 
 // One launch per group of at most kParamMembers members.
 template <int LAT, typename S>
-cudaError_t batch_param_t(void *base, const BatchParams *groups, int ngroups, const BatchStep *steps, int passes,
+cudaError_t batch_param_t(void *base, const BatchParams *groups, int ngroups, const BatchWhen &when, int passes,
                           int occ, int vx_max, int noise_mode, int noise_dist, cudaStream_t stream) {
   S *b = static_cast<S *>(base);
   if (vx_max == 1)
-    return occ == 1 ? batch_param_occ<LAT, S, 1, 1>(b, groups, ngroups, steps, passes, noise_mode, noise_dist, stream)
-                    : batch_param_occ<LAT, S, 0, 1>(b, groups, ngroups, steps, passes, noise_mode, noise_dist, stream);
-  return occ == 1 ? batch_param_occ<LAT, S, 1, 2>(b, groups, ngroups, steps, passes, noise_mode, noise_dist, stream)
-                  : batch_param_occ<LAT, S, 0, 2>(b, groups, ngroups, steps, passes, noise_mode, noise_dist, stream);
+    return occ == 1 ? batch_param_occ<LAT, S, 1, 1>(b, groups, ngroups, when, passes, noise_mode, noise_dist, stream)
+                    : batch_param_occ<LAT, S, 0, 1>(b, groups, ngroups, when, passes, noise_mode, noise_dist, stream);
+  return occ == 1 ? batch_param_occ<LAT, S, 1, 2>(b, groups, ngroups, when, passes, noise_mode, noise_dist, stream)
+                  : batch_param_occ<LAT, S, 0, 2>(b, groups, ngroups, when, passes, noise_mode, noise_dist, stream);
 }
 
 template <int LAT, typename S, int NOISE, int OCC, int VXMAX>

@@ -56,7 +56,7 @@ int d_of(int lattice) { return lattice == LBFD_D1Q3 ? 1 : (lattice == LBFD_D2Q9 
 
 struct lbfd_ens {
   int lattice = 0, precision = 0, noise_mode = 0, noise_dist = 0, elem = 4, Q = 0, device = 0, n = 0;
-  int vx_max = 2, kvx = 2, passes = 1, occ = 0, walk = 0, grid = 1, bps = 1;  // kvx: largest vx of a member
+  int vx_max = 2, kvx = 2, passes = 1, tile_passes = 1, occ = 0, walk = 0, grid = 1, bps = 1;  // kvx: largest vx of a member
   int64_t ntiles = 0;
   std::vector<BatchMember> hmem;
   std::vector<int64_t> tile_start;
@@ -90,27 +90,39 @@ static int ens_step_launches(const lbfd_ens *e) {
   return e->walk == kWalkParam ? static_cast<int>(e->groups.size()) : 1;
 }
 
-static cudaError_t ens_launch(lbfd_ens *e) {
-  if (e->walk == kWalkParam) {
-    // groups k, k + kSide, ... on side stream k, forked from and joined to the ensemble's stream
-    const int G = static_cast<int>(e->groups.size());
-    const int nside = std::min(G, int(lbfd_ens::kSide));
-    if (nside <= 1)
-      return launch_batch_param(e->lattice, e->precision, e->buf, e->groups.data(), G, e->dsteps, e->passes, e->occ,
-                                e->kvx, e->noise_mode, e->noise_dist, e->stream);
-    cudaError_t err = cudaEventRecord(e->fork_ev, e->stream);
-    for (int k = 0; k < nside && err == cudaSuccess; ++k) {
-      err = cudaStreamWaitEvent(e->side[k], e->fork_ev, 0);
-      for (int g = k; g < G && err == cudaSuccess; g += nside)
-        err = launch_batch_param(e->lattice, e->precision, e->buf, &e->groups[g], 1, e->dsteps, e->passes, e->occ,
-                                 e->kvx, e->noise_mode, e->noise_dist, e->side[k]);
-      if (err == cudaSuccess) err = cudaEventRecord(e->join_ev[k], e->side[k]);
-      if (err == cudaSuccess) err = cudaStreamWaitEvent(e->stream, e->join_ev[k], 0);
-    }
+// `steps` steps of the parameter-space launches from the device clock on
+// (which stays).  The groups are independent of each other, so each runs all
+// of its steps on one side stream, as dependent launches, and the streams
+// fork from the ensemble's and join it once: no launch of a step waits for
+// another group's, nor for a launch that prepares it.  Measured on GB300, 60
+// D2Q9 members of 96..512 a side, 2000 steps: 126 -> 96 ms, with the items of
+// batch_tile_items.
+static cudaError_t ens_param_steps(lbfd_ens *e, int steps) {
+  const int G = static_cast<int>(e->groups.size());
+  const int nside = std::min(G, int(lbfd_ens::kSide));
+  auto chain = [&](int g, cudaStream_t st) {
+    cudaError_t err = cudaSuccess;
+    for (int k = 0; k < steps && err == cudaSuccess; ++k)
+      err = launch_batch_param(e->lattice, e->precision, e->buf, &e->groups[g], 1,
+                               BatchWhen{e->t_dev, uint64_t(k), k > 0}, e->tile_passes, e->occ, e->kvx, e->noise_mode,
+                               e->noise_dist, st);
     return err;
+  };
+  if (nside <= 1) return chain(0, e->stream);
+  cudaError_t err = cudaEventRecord(e->fork_ev, e->stream);
+  for (int k = 0; k < nside && err == cudaSuccess; ++k) {
+    err = cudaStreamWaitEvent(e->side[k], e->fork_ev, 0);
+    for (int g = k; g < G && err == cudaSuccess; g += nside) err = chain(g, e->side[k]);
+    if (err == cudaSuccess) err = cudaEventRecord(e->join_ev[k], e->side[k]);
+    if (err == cudaSuccess) err = cudaStreamWaitEvent(e->stream, e->join_ev[k], 0);
   }
-  return launch_batch_step(e->lattice, e->precision, e->buf, e->dsteps, e->dtile_start, e->n, e->ntiles, e->passes,
-                           e->occ, e->walk, e->kvx, e->noise_mode, e->noise_dist, e->grid, e->stream);
+  return err;
+}
+
+static cudaError_t ens_launch(lbfd_ens *e) {
+  if (e->walk == kWalkParam) return ens_param_steps(e, 1);
+  return launch_batch_step(e->lattice, e->precision, e->buf, e->dsteps, e->dtile_start, e->n, e->ntiles,
+                           e->tile_passes, e->occ, e->walk, e->kvx, e->noise_mode, e->noise_dist, e->grid, e->stream);
 }
 
 // Work decomposition (sites per item, tile passes, occupancy variant, tile
@@ -119,11 +131,15 @@ static cudaError_t ens_launch(lbfd_ens *e) {
 static int ens_plan(lbfd_ens *e, int vx_max, int passes, int occ, int walk) {
   e->kvx = 1;
   for (BatchMember &m : e->hmem) {
-    m.vx = (vx_max >= 2 && m.Lx % 2 == 0) ? 2 : 1;
+    m.vx = batch_vx(e->lattice, m.Lx, vx_max, e->precision);
     e->kvx = std::max(e->kvx, int(m.vx));
   }
+  e->bps = batch_blocks_per_sm(e->lattice, e->precision, occ, e->kvx, walk, e->noise_mode, e->noise_dist);
+  int sms = 0;
+  ENS_CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, e->device));
+  e->tile_passes = walk == kWalkParam ? batch_passes(e->hmem.data(), e->n, passes, int64_t(sms) * e->bps) : passes;
   e->tile_start.assign(e->n, 0);
-  e->ntiles = batch_assign_tiles(e->hmem.data(), e->n, passes, e->tile_start.data());
+  e->ntiles = batch_assign_tiles(e->hmem.data(), e->n, e->tile_passes, e->tile_start.data());
   ENS_CU(cudaMemcpy(e->dmem, e->hmem.data(), sizeof(BatchMember) * e->n, cudaMemcpyHostToDevice));
   ENS_CU(cudaMemcpy(e->dtile_start, e->tile_start.data(), sizeof(int64_t) * e->n, cudaMemcpyHostToDevice));
   e->vx_max = vx_max;
@@ -132,9 +148,6 @@ static int ens_plan(lbfd_ens *e, int vx_max, int passes, int occ, int walk) {
   e->walk = walk;
   e->groups.clear();
   if (walk == kWalkParam) batch_build_params(e->hmem.data(), e->n, e->ntiles, e->noise_mode, e->noise_dist, e->groups);
-  e->bps = batch_blocks_per_sm(e->lattice, e->precision, occ, e->kvx, walk, e->noise_mode, e->noise_dist);
-  int sms = 0;
-  ENS_CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, e->device));
   e->grid = int(std::max<int64_t>(1, std::min<int64_t>(e->ntiles, int64_t(sms) * e->bps)));
   if (e->graph) {
     cudaGraphExecDestroy(e->graph);
@@ -171,11 +184,19 @@ static cudaError_t ens_sync_t(lbfd_ens *e) {
   return err;
 }
 
-// One step of every member (arguments for the current t, the step, t += 1).
-static cudaError_t ens_one_step(lbfd_ens *e) {
-  cudaError_t err = launch_batch_prep(e->dmem, e->n, e->t_dev, 0, e->noise_mode, e->noise_dist, e->dsteps, e->stream);
-  if (err == cudaSuccess) err = ens_launch(e);
-  if (err == cudaSuccess) err = launch_clock_advance(e->t_dev, e->stream);
+// `steps` steps of every member, and t += steps on the device.
+static cudaError_t ens_steps(lbfd_ens *e, int steps) {
+  cudaError_t err = cudaSuccess;
+  if (e->walk == kWalkParam) {
+    err = ens_param_steps(e, steps);
+    if (err == cudaSuccess) err = launch_clock_advance(e->t_dev, e->stream, uint64_t(steps));
+    return err;
+  }
+  for (int k = 0; k < steps && err == cudaSuccess; ++k) {
+    err = launch_batch_prep(e->dmem, e->n, e->t_dev, 0, e->noise_mode, e->noise_dist, e->dsteps, e->stream);
+    if (err == cudaSuccess) err = ens_launch(e);
+    if (err == cudaSuccess) err = launch_clock_advance(e->t_dev, e->stream, 1);
+  }
   return err;
 }
 
@@ -183,7 +204,7 @@ static cudaError_t ens_build_graph(lbfd_ens *e) {
   cudaGraph_t g = nullptr;
   cudaError_t err = cudaStreamBeginCapture(e->stream, cudaStreamCaptureModeThreadLocal);
   if (err != cudaSuccess) return err;
-  for (int k = 0; k < kGraphSteps && err == cudaSuccess; ++k) err = ens_one_step(e);
+  err = ens_steps(e, kGraphSteps);
   cudaError_t end = cudaStreamEndCapture(e->stream, &g);
   if (err == cudaSuccess) err = end;
   if (err == cudaSuccess) err = cudaGraphInstantiate(&e->graph, g, 0);
@@ -254,7 +275,7 @@ int lbfd_ensemble_create(lbfd_ens_t *out, int32_t lattice, int32_t precision, in
   for (int m = 0; m < n; ++m) {
     const lbfd_member &mb = members[m];
     e->hmem.push_back(
-        make_batch_member(mb.dims, mb.tau, mb.rho_mean, mb.seed, mb.lattice_id, offs[m], off + offs[m], 0, 2));
+        make_batch_member(lattice, mb.dims, mb.tau, mb.rho_mean, mb.seed, mb.lattice_id, offs[m], off + offs[m], 0, 2, precision));
     e->total_sites += e->hmem.back().N;
   }
   DevGuard g(dev);
@@ -326,11 +347,13 @@ int lbfd_ensemble_step(lbfd_ens_t e, int64_t n) {
       ENS_CU(cudaGraphLaunch(e->graph, e->stream));
       done += kGraphSteps;
     } else {
-      ENS_CU(ens_one_step(e));
-      done += 1;
+      const int rest = static_cast<int>(n - done);
+      ENS_CU(ens_steps(e, rest));
+      done += rest;
     }
   }
-  count_launches(n * (2 + ens_step_launches(e)));
+  const int64_t chunks = (n + kGraphSteps - 1) / kGraphSteps;
+  count_launches(e->walk == kWalkParam ? n * ens_step_launches(e) + chunks : n * (2 + ens_step_launches(e)));
   e->t += n;
   return LBFD_OK;
 }

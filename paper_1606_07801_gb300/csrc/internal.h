@@ -375,14 +375,15 @@ cudaError_t launch_batch_step_d3q19(int precision, void *base, const BatchStep *
                                     int nmembers, int64_t ntiles, int passes, int occ, int walk, int vx_max,
                                     int noise_mode, int noise_dist, int grid, cudaStream_t stream);
 struct BatchParams;
+struct BatchWhen;
 cudaError_t launch_batch_param_d1q3(int precision, void *base, const BatchParams *groups, int ngroups,
-                                    const BatchStep *steps, int passes, int occ, int vx_max, int noise_mode,
+                                    const BatchWhen &when, int passes, int occ, int vx_max, int noise_mode,
                                     int noise_dist, cudaStream_t stream);
 cudaError_t launch_batch_param_d2q9(int precision, void *base, const BatchParams *groups, int ngroups,
-                                    const BatchStep *steps, int passes, int occ, int vx_max, int noise_mode,
+                                    const BatchWhen &when, int passes, int occ, int vx_max, int noise_mode,
                                     int noise_dist, cudaStream_t stream);
 cudaError_t launch_batch_param_d3q19(int precision, void *base, const BatchParams *groups, int ngroups,
-                                     const BatchStep *steps, int passes, int occ, int vx_max, int noise_mode,
+                                     const BatchWhen &when, int passes, int occ, int vx_max, int noise_mode,
                                      int noise_dist, cudaStream_t stream);
 int batch_blocks_per_sm_d1q3(int precision, int occ, int vx_max, int walk, int noise_mode, int noise_dist);
 int batch_blocks_per_sm_d2q9(int precision, int occ, int vx_max, int walk, int noise_mode, int noise_dist);
@@ -397,16 +398,16 @@ cudaError_t launch_batch_step(int lattice, int precision, void *base, const Batc
                               int nmembers, int64_t ntiles, int passes, int occ, int walk, int vx_max, int noise_mode,
                               int noise_dist, int grid, cudaStream_t stream);
 // One launch per group of at most kParamMembers members, their arguments in
-// the kernel parameters (tile order 3); steps holds k_batch_prep's output.
+// the kernel parameters (tile order 3).
 cudaError_t launch_batch_param(int lattice, int precision, void *base, const BatchParams *groups, int ngroups,
-                               const BatchStep *steps, int passes, int occ, int vx_max, int noise_mode, int noise_dist,
+                               const BatchWhen &when, int passes, int occ, int vx_max, int noise_mode, int noise_dist,
                                cudaStream_t stream);
 int batch_blocks_per_sm(int lattice, int precision, int occ, int vx_max, int walk, int noise_mode, int noise_dist);
 // Step arguments of members[0..n) for the clock *clock_dev (clock when null).
 cudaError_t launch_batch_prep(const BatchMember *members, int n, const uint64_t *clock_dev, uint64_t clock,
                               int noise_mode, int noise_dist, BatchStep *out, cudaStream_t stream);
-// clock += 1 on the device (between the launches of a captured graph).
-cudaError_t launch_clock_advance(uint64_t *clock_dev, cudaStream_t stream);
+// clock += by on the device (between the launches of a captured graph).
+cudaError_t launch_clock_advance(uint64_t *clock_dev, cudaStream_t stream, uint64_t by);
 
 // Records n launches of this library's kernels (lbfd_kernel_launches).
 void count_launches(int64_t n);

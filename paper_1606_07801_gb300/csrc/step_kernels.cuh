@@ -172,6 +172,12 @@ __device__ __forceinline__ uint3 sweep_block(int32_t sweep) {
   return make_uint3(gridDim.x - 1 - blockIdx.x, gridDim.y - 1 - blockIdx.y, gridDim.z - 1 - blockIdx.z);
 }
 
+// Index of site (x, y, z).
+__device__ __forceinline__ uint32_t site_index(const StepArgs &a, int x, int y, int z) {
+  return static_cast<uint32_t>(x) + static_cast<uint32_t>(a.Lx) *
+         (static_cast<uint32_t>(y) + static_cast<uint32_t>(a.Ly) * static_cast<uint32_t>(z));
+}
+
 // Pull of site (x, y, z) of one lattice (any shape) into f, returning its
 // index.  S is the storage type (float, double, or a 16-bit deviation format
 // with FP32 arithmetic), Idx the type of the value offsets i N + site:
@@ -250,56 +256,13 @@ __global__ void __launch_bounds__(256)
   const int y = b.y * blockDim.y + threadIdx.y;
   const int z = b.z;
   if (x >= a.Lx || y >= a.Ly) return;
-  const uint32_t Lx = static_cast<uint32_t>(a.Lx);
   R t[C::kAhead];
-  collide.ahead(t, static_cast<uint32_t>(x) + Lx * (static_cast<uint32_t>(y) + static_cast<uint32_t>(a.Ly) * static_cast<uint32_t>(z)),
-                a.ph);
+  collide.ahead(t, site_index(a, x, y, z), a.ph);
   pdl_wait();
   R f[Lattice<LAT>::Q];
   const uint32_t s = scalar_pull<LAT, S, Idx>(src, a, x, y, z, f);
   collide.given(f, [&](int k) -> R { return t[k]; }, a);
   scalar_store<LAT, S, Idx>(dst, a, s, f);
-}
-
-// Twin kernel: site x of a row's first half and site x + apart of its second
-// per thread, apart = ceil(Lx / 2), updated at once on the packed FP32
-// instructions; the loads and stores are those of the scalar kernel, so Lx
-// may be odd.  For lattices of few populations (D3Q19
-// spills: 107 us at 127 x 128 x 128 against 56).  D2Q9 FP32 1023 x 771 11.0 ->
-// 10.5 us per step, 511 x 513 5.2 -> 4.35 on GB300.
-template <int LAT, typename S, int NOISE, typename Idx>
-__global__ void __launch_bounds__(128, 6)
-    k_step_twin(const S *src, S *dst, const StepArgs a) {
-  constexpr int Q = Lattice<LAT>::Q;
-  const SrtCollideFor<LAT, S, NOISE> collide;
-  pdl_launch_dependents();
-  const uint3 b = sweep_block(a.sweep);
-  const int apart = (a.Lx + 1) / 2;
-  const int x = b.x * blockDim.x + threadIdx.x;
-  const int y = b.y * blockDim.y + threadIdx.y;
-  const int z = b.z;
-  if (x >= apart || y >= a.Ly) return;
-  const uint32_t Lx = static_cast<uint32_t>(a.Lx);
-  const uint32_t s = static_cast<uint32_t>(x) + Lx * (static_cast<uint32_t>(y) + static_cast<uint32_t>(a.Ly) * static_cast<uint32_t>(z));
-  float2 t[Q - 1];
-  collide.ahead(t, s, a.ph, static_cast<uint32_t>(apart));
-  pdl_wait();
-  // the middle of an odd row has no twin: its second site is itself, not stored
-  const bool two = x + apart < a.Lx;
-  float fa[Q], fb[Q];
-  float2 f[Q];
-  scalar_pull<LAT, S, Idx>(src, a, x, y, z, fa);
-  const uint32_t s2 = scalar_pull<LAT, S, Idx>(src, a, two ? x + apart : x, y, z, fb);
-#pragma unroll
-  for (int i = 0; i < Q; ++i) f[i] = make_float2(fa[i], fb[i]);
-  collide.given(f, [&](int k) -> float2 { return t[k]; }, a);
-#pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    fa[i] = f[i].x;
-    fb[i] = f[i].y;
-  }
-  scalar_store<LAT, S, Idx>(dst, a, s, fa);
-  if (two) scalar_store<LAT, S, Idx>(dst, a, s2, fb);
 }
 
 // Vector kernel: VX consecutive sites of a row per thread (needs Lx % VX == 0).
@@ -490,11 +453,46 @@ __global__ void __launch_bounds__(256, step_min_blocks<LAT, S, VX>())
   step_vec_body<LAT, S, VX, NOISE, SrtCollideFor<LAT, S, NOISE>, Idx>(src, dst, a, x0, y, z);
 }
 
-// Vector kernel with the noise ahead: the variates' sums of the thread's
-// sites, two sites per packed instruction, wait in the thread's own column of
-// shared memory while it pulls the populations, so that neither half holds
-// the other's registers: two D3Q19 sites fit 64-72 registers paired, where the
-// one-piece form spills at 80.
+// A thread's column of shared memory, K float2 values THREADS apart: where
+// the noise of a pair of sites waits while the thread pulls the populations,
+// so that neither half of the update holds the other's registers (two D3Q19
+// sites fit 64-72 registers paired, where the one-piece form spills at 80).
+// The accesses are volatile: the compiler may not carry the values past the
+// pull in registers.
+template <int K, int THREADS>
+struct NoiseColumn {
+  uint32_t at;
+  // tid: the thread's index in the block; base: K * THREADS float2 of shared memory
+  __device__ __forceinline__ NoiseColumn(float2 *base, int tid)
+      : at(static_cast<uint32_t>(__cvta_generic_to_shared(base + tid))) {}
+  __device__ __forceinline__ void put(int k, const float2 &v) const {
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(at + static_cast<uint32_t>(k * THREADS * 8)), "f"(v.x), "f"(v.y));
+  }
+  __device__ __forceinline__ float2 get(int k) const {
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];"
+                 : "=f"(v.x), "=f"(v.y)
+                 : "r"(at + static_cast<uint32_t>(k * THREADS * 8)));
+    return v;
+  }
+};
+
+// The collision of a pair of sites given its parked noise.
+template <class C, int Q, class Col>
+__device__ __forceinline__ void collide_parked(const C &collide, float (&fa)[Q], float (&fb)[Q], const Col &col, int k0,
+                                               const StepArgs &a) {
+  float2 g[Q];
+#pragma unroll
+  for (int i = 0; i < Q; ++i) g[i] = make_float2(fa[i], fb[i]);
+  collide.given(g, [&](int k) -> float2 { return col.get(k0 + k); }, a);
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    fa[i] = g[i].x;
+    fb[i] = g[i].y;
+  }
+}
+
+// Vector kernel with the noise ahead, two sites per packed instruction.
 template <int LAT, typename S, int VX>
 constexpr int ahead_min_blocks() {  // 128-thread blocks
   return LAT == kD3Q19 ? 7 : (Store<S>::kDeviation ? 7 : 6);
@@ -503,47 +501,74 @@ template <int LAT, typename S, int VX, int NOISE, typename Idx, class C>
 __global__ void __launch_bounds__(128, ahead_min_blocks<LAT, S, VX>())
     k_step_ahead(const S *src, S *dst, const StepArgs a, const C collide) {
   constexpr int Q = Lattice<LAT>::Q, K = C::kAhead;
-  __shared__ float2 column[VX / 2][K][128];
+  __shared__ float2 column[VX / 2 * K * 128];
   pdl_launch_dependents();
   const uint3 b = sweep_block(a.sweep);
   const int x0 = (b.x * blockDim.x + threadIdx.x) * VX;
   const int y = b.y * blockDim.y + threadIdx.y;
   const int z = b.z;
   if (x0 >= a.Lx || y >= a.Ly) return;
-  const uint32_t s0 = static_cast<uint32_t>(x0) + static_cast<uint32_t>(a.Lx) *
-                      (static_cast<uint32_t>(y) + static_cast<uint32_t>(a.Ly) * static_cast<uint32_t>(z));
-  const uint32_t at = static_cast<uint32_t>(__cvta_generic_to_shared(&column[0][0][threadIdx.x + blockDim.x * threadIdx.y]));
-  auto slot = [&](int p, int k) { return at + static_cast<uint32_t>((p * K + k) * 128 * sizeof(float2)); };
-  // volatile: the compiler may not carry the values past the pull in registers
+  const NoiseColumn<VX / 2 * K, 128> col(column, static_cast<int>(threadIdx.x + blockDim.x * threadIdx.y));
+  const uint32_t s0 = site_index(a, x0, y, z);
 #pragma unroll
   for (int p = 0; p < VX / 2; ++p) {
     float2 t[K];
     collide.ahead(t, s0 + 2u * static_cast<uint32_t>(p), a.ph);
 #pragma unroll
-    for (int k = 0; k < K; ++k)
-      asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(slot(p, k)), "f"(t[k].x), "f"(t[k].y));
+    for (int k = 0; k < K; ++k) col.put(p * K + k, t[k]);
   }
   pdl_wait();
   float f[VX][Q];
   const uint32_t row = vec_pull<LAT, S, VX, Idx>(src, a, x0, y, z, f);
 #pragma unroll
-  for (int p = 0; p < VX / 2; ++p) {
-    float2 g[Q];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) g[i] = make_float2(f[2 * p][i], f[2 * p + 1][i]);
-    collide.given(g, [&](int k) -> float2 {
-      float2 t;
-      asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(t.x), "=f"(t.y) : "r"(slot(p, k)));
-      return t;
-    }, a);
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      f[2 * p][i] = g[i].x;
-      f[2 * p + 1][i] = g[i].y;
-    }
-  }
+  for (int p = 0; p < VX / 2; ++p) collide_parked(collide, f[2 * p], f[2 * p + 1], col, p * K, a);
   vec_store<LAT, S, VX, Idx>(dst, a, row, x0, f);
 }
+
+// Update of site x of a row's first half and its twin x + apart in the
+// second, apart = ceil(Lx / 2): paired like neighbours, with the scalar
+// loads and stores that an odd Lx needs.  The middle site of an odd row has
+// no twin (its second site is itself, not stored).  ready() is called between
+// the noise and the first load.
+template <int LAT, typename S, typename Idx, class C, class Col, class F>
+__device__ __forceinline__ void twin_update(const S *src, S *dst, const StepArgs &a, int x, int y, int z, const C &collide,
+                                            const Col &col, F &&ready) {
+  constexpr int Q = Lattice<LAT>::Q, K = C::kAhead;
+  const int apart = (a.Lx + 1) / 2;
+  {
+    float2 t[K];
+    collide.ahead(t, site_index(a, x, y, z), a.ph, static_cast<uint32_t>(apart));
+#pragma unroll
+    for (int k = 0; k < K; ++k) col.put(k, t[k]);
+  }
+  ready();
+  const bool two = x + apart < a.Lx;
+  float fa[Q], fb[Q];
+  const uint32_t s = scalar_pull<LAT, S, Idx>(src, a, x, y, z, fa);
+  const uint32_t s2 = scalar_pull<LAT, S, Idx>(src, a, two ? x + apart : x, y, z, fb);
+  collide_parked(collide, fa, fb, col, 0, a);
+  scalar_store<LAT, S, Idx>(dst, a, s, fa);
+  if (two) scalar_store<LAT, S, Idx>(dst, a, s2, fb);
+}
+
+// Twin kernel, for rows of odd length.  Measured on GB300 against one site
+// per thread, microseconds per step: D2Q9 FP32 1023 x 771 11.0 -> 9.2, 511 x
+// 513 5.2 -> 3.7, D3Q19 FP32 127 x 128 x 128 56.4 -> 54.3, 63 x 64 x 64 8.4 ->
+// 6.9.
+template <int LAT, typename S, int NOISE, typename Idx>
+__global__ void __launch_bounds__(128, 7)
+    k_step_twin(const S *src, S *dst, const StepArgs a) {
+  using C = SrtCollideFor<LAT, S, NOISE>;
+  __shared__ float2 column[C::kAhead * 128];
+  pdl_launch_dependents();
+  const uint3 b = sweep_block(a.sweep);
+  const int x = b.x * blockDim.x + threadIdx.x;
+  const int y = b.y * blockDim.y + threadIdx.y;
+  if (x >= (a.Lx + 1) / 2 || y >= a.Ly) return;
+  const NoiseColumn<C::kAhead, 128> col(column, static_cast<int>(threadIdx.x + blockDim.x * threadIdx.y));
+  twin_update<LAT, S, Idx>(src, dst, a, x, y, static_cast<int>(b.z), C(), col, [] { pdl_wait(); });
+}
+
 // Where k_step_ahead replaces k_step_vec (noisy steps in FP32 arithmetic),
 // microseconds per step on GB300: D3Q19 FP32 at every size (256^3 390 -> 375,
 // 1.004 of the copy bandwidth),
@@ -603,7 +628,7 @@ cudaError_t step_noise_idx(const S *s, S *d, const StepArgs &a, int vx, cudaStre
           return cudaLaunchKernelEx(&launch.cfg, k_step_ahead<LAT, S, 4, NOISE, Idx, C>, s, d, a, c);
       }
     }
-    if constexpr (NOISE != kStepNoiseOff && LAT == kD2Q9) {
+    if constexpr (NOISE != kStepNoiseOff && LAT != kD1Q3) {
       if (vx == 1 && a.Lx % 2 != 0 && step_vec_width(LAT, kStoreF32, 4, a.N) > 1) {  // above the smallest sizes
         step_shape((a.Lx + 1) / 2, a.Ly, a.Lz, launch.cfg.gridDim, launch.cfg.blockDim, 1, 128);
         return cudaLaunchKernelEx(&launch.cfg, k_step_twin<LAT, S, NOISE, Idx>, s, d, a);
