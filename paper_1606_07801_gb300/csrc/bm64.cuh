@@ -194,6 +194,24 @@ __host__ __device__ __forceinline__ double add_hi(double x, int32_t hi) {  // ad
 #endif
 }
 
+// sqrt(x) by two Newton steps on x / sqrt(x) from the seed, each correction
+// added with one rounding: within 0.501 units in the last place.  For x in
+// [2^-900, 2^900].  Five dependent FP64 operations, about three fewer than the
+// general square root (each some 50 clocks on the small lattices' chain).
+__host__ __device__ __forceinline__ double sqrt_newton(double x) {
+  const double y = rsqrt_seed(x), h = add_hi(y, -(1 << 20));  // y / 2
+  double g = x * y;
+  g = fma64(fma64(-g, g, x), h, g);
+  return fma64(fma64(-g, g, x), h, g);
+}
+#ifdef __CUDACC__
+// sqrt(x) for any x.
+__device__ __forceinline__ double sqrt_any(double x) {
+  const int hi = __double2hiint(x);  // the sign and exponent: 1023 - 900 .. 1023 + 900
+  return hi >= (123 << 20) && hi < (1923 << 20) ? sqrt_newton(x) : ::sqrt(x);
+}
+#endif
+
 // 2^28 sqrt(-2 ln u0), u0 = ((r >> 8) + 1/2) 2^-24.
 __host__ __device__ __forceinline__ double radius28(uint32_t r, const Tables &T) {
   const uint32_t K = (r >> 7) | 1u;  // u0 2^25
@@ -218,10 +236,7 @@ __host__ __device__ __forceinline__ double radius28(uint32_t r, const Tables &T)
   X += static_cast<int64_t>(::rintf(tail));
   const double x = add_hi(static_cast<double>(X), -(sh << 20));
 #endif
-  const double y = rsqrt_seed(x), h = add_hi(y, -(1 << 20));  // y / 2
-  double g = x * y;
-  g = fma64(fma64(-g, g, x), h, g);
-  return fma64(fma64(-g, g, x), h, g);
+  return sqrt_newton(x);
 }
 
 // 2^-28 (cos, sin) of 2 pi u1, u1 = ((r >> 8) + 1/2) 2^-24.

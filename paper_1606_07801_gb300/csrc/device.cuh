@@ -504,6 +504,14 @@ __host__ __device__ __forceinline__ R noise_amplitude(R x) {
   return Math<R>::sqrt(x);
 }
 template <>
+__host__ __device__ __forceinline__ double noise_amplitude<double>(double x) {
+#ifdef __CUDA_ARCH__
+  return bm64::sqrt_any(x);
+#else
+  return ::sqrt(x);
+#endif
+}
+template <>
 __host__ __device__ __forceinline__ float noise_amplitude<float>(float x) {
 #ifdef __CUDA_ARCH__
   return sqrt_sfu(x);
@@ -695,6 +703,21 @@ __host__ __device__ __forceinline__ V flat_variate(V k) {
   return mul_rn(cst<V>(kSqrt3), fma_rn(splat<V>(R(2)), u, splat<V>(R(-1))));
 }
 
+// The variates of call j from its words: z[k] for the moments 4j + k < NMOM.
+template <typename R, int NMOM, bool GAUSS>
+__host__ __device__ __forceinline__ void call_variates(R (&z)[4], const uint4 &r, int j) {
+  const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+  if constexpr (GAUSS) {
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+      if (4 * j + 2 * p < NMOM) BoxMuller<R>::pair(w[2 * p], w[2 * p + 1], z[2 * p], z[2 * p + 1]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (4 * j + k < NMOM) z[k] = flat_variate<R>(static_cast<R>(w[k] >> 8));
+  }
+}
+
 template <typename R, int NMOM, bool GAUSS>
 __host__ __device__ __forceinline__ void draw_variates_t(R (&z)[NMOM], uint32_t site, const PhiloxStep &P) {
   constexpr int NCALL = (NMOM + 3) / 4;
@@ -702,23 +725,11 @@ __host__ __device__ __forceinline__ void draw_variates_t(R (&z)[NMOM], uint32_t 
   const uint32_t s_hi = static_cast<uint32_t>(sp >> 32), s_lo = static_cast<uint32_t>(sp);
 #pragma unroll
   for (int j = 0; j < NCALL; ++j) {
-    const uint4 r = philox_site(s_hi, s_lo, P, j);
-    const uint32_t w[4] = {r.x, r.y, r.z, r.w};
-    if constexpr (GAUSS) {
+    R c[4];
+    call_variates<R, NMOM, GAUSS>(c, philox_site(s_hi, s_lo, P, j), j);
 #pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        if (4 * j + 2 * p < NMOM) {
-          R z0, z1;
-          BoxMuller<R>::pair(w[2 * p], w[2 * p + 1], z0, z1);
-          z[4 * j + 2 * p] = z0;
-          if (4 * j + 2 * p + 1 < NMOM) z[4 * j + 2 * p + 1] = z1;
-        }
-      }
-    } else {
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        if (4 * j + k < NMOM) z[4 * j + k] = flat_variate<R>(static_cast<R>(w[k] >> 8));
-    }
+    for (int k = 0; k < 4; ++k)
+      if (4 * j + k < NMOM) z[4 * j + k] = c[k];
   }
 }
 

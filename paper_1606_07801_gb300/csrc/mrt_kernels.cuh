@@ -124,7 +124,7 @@ __device__ __forceinline__ void mrt_given(V (&f)[Lattice<LAT>::Q], const ZF &z, 
   V moved = splat<V>(R(0));
   auto keep = [&](int i, const V &x) {
     f[i] = x;
-    moved = add_rn(moved, x);
+    moved = i == 1 ? x : add_rn(moved, x);
   };
   if constexpr (LAT == kD2Q5) {
     const V w = splat<V>(p.w);
@@ -164,6 +164,10 @@ struct MrtCollide {
       else
         draw_variates_t<R, Q - 1, NOISE == kStepNoiseGauss>(z, s, ph);
     }
+  }
+  __device__ __forceinline__ void shape(R (&t)[kAhead], const R (&z)[kAhead]) const {
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) t[k] = z[k];
   }
   template <typename V, class ZF>
   __device__ __forceinline__ void given(V (&f)[Q], const ZF &z, const StepArgs &a) const {

@@ -73,7 +73,7 @@ __device__ __forceinline__ void collide_given(V (&f)[Lattice<LAT>::Q], const TF 
     } else {
       f[i] = fma_rn(omega, f[i], fma_rn(wsig[k], T(i), wrel[k]));
     }
-    moved = add_rn(moved, f[i]);
+    moved = i == 1 ? f[i] : add_rn(moved, f[i]);
   });
   f[0] = sub_rn(rho, moved);
 }
@@ -135,6 +135,14 @@ struct SrtCollide {
 #pragma unroll
     for (int k = 0; k < kAhead; ++k) t[k] = T[k + 1];
   }
+  // the same values from a site's variates
+  __device__ __forceinline__ void shape(R (&t)[kAhead], const R (&z)[kAhead]) const {
+    R T[kAhead + 1];
+    NoiseTransform<LAT, R>::apply(z, T);
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) t[k] = T[k + 1];
+  }
+  static constexpr int kNoise = NOISE;
   template <typename V, class TF>
   __device__ __forceinline__ void given(V (&f)[Lattice<LAT>::Q], const TF &t, const StepArgs &a) const {
     collide_given<LAT, R, NOISE, DEV>(f, [&](int i) -> V { return t(i - 1); }, a);
