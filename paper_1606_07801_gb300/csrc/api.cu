@@ -496,12 +496,11 @@ static int sample_now(lbfd_sim *h) {
                                     h->partials, h->fin, h->acc, h->stream));
     g_launches.fetch_add(2, std::memory_order_relaxed);
   } else {
-    // FP64 storage: FP64 throughout, on the streamed copy of the state
-    LBFD_CU(materialize_f(h));
-    LBFD_CU(launch_observables(o.lattice, o.precision, h->f[h->cur ^ 1], int32_t(o.dims[0]), int32_t(o.dims[1]),
-                               int32_t(o.dims[2]), o.rho_mean, o.n_modes, &h->modes_host[0][0], h->partials, h->acc,
-                               h->stream));
-    g_launches.fetch_add(3, std::memory_order_relaxed);
+    // FP64 storage: FP64 throughout
+    LBFD_CU(launch_observables64(o.lattice, static_cast<const double *>(h->f[h->cur]), int32_t(o.dims[0]),
+                                 int32_t(o.dims[1]), int32_t(o.dims[2]), o.rho_mean, o.n_modes, &h->modes_host[0][0],
+                                 h->partials, h->fin, h->acc, h->stream));
+    g_launches.fetch_add(2, std::memory_order_relaxed);
   }
   h->n_samples += 1;
   return LBFD_OK;

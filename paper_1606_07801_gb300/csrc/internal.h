@@ -228,9 +228,11 @@ int obs_quantities(int Q, int n_modes);
 cudaError_t launch_mass(int lattice, int precision, const void *f, int64_t N, double rho_mean, double *partials,
                         double *out, cudaStream_t stream, int64_t stride = 0);
 
-cudaError_t launch_observables(int lattice, int precision, const void *f, int32_t Lx, int32_t Ly, int32_t Lz,
-                               double rho_mean, int n_modes, const int32_t *modes /*device, n_modes*3*/,
-                               double *partials, double *acc, cudaStream_t stream);
+// The observables of FP64 storage from the stored post-collision state g, FP64
+// throughout (fin as for launch_observables_pull).
+cudaError_t launch_observables64(int lattice, const double *g, int32_t Lx, int32_t Ly, int32_t Lz, double rho_mean,
+                                 int n_modes, const int32_t *modes, double *partials, double *fin, double *acc,
+                                 cudaStream_t stream);
 
 // The same observables for FP32 arithmetic (FP32, FP16, BF16 storage; not
 // FP64) from the stored post-collision state g, pulled per population (no

@@ -86,184 +86,278 @@ struct ModeArgs {
 // partial layout per block: [rho, rho2, f_0..f_{Q-1}, re_0, im_0, .., re_{K-1}, im_{K-1}, ff pairs (i <= j)]
 int obs_quantities(int Q, int n_modes) { return 2 + Q + 2 * n_modes + Q * (Q + 1) / 2; }
 
-template <int LAT, typename S>
-__global__ void __launch_bounds__(kReduceThreads) k_obs_partials(const S *__restrict__ f, int32_t Lx, int32_t Ly,
-                                                                int32_t Lz, double rho_mean, const ModeArgs modes,
-                                                                double *__restrict__ partials) {
+// The observables of FP64 storage, FP64 throughout, straight from the stored
+// post-collision state (population i at site x is g_i(x - v_i), as the step
+// pulls it).  The FP64 pipe bounds it (2 lanes per clock and SM), so the pair
+// sums are the work: a thread keeps them in registers for its own sites where
+// they fit (D1Q3, D2Q5, D2Q9: Q (Q + 1)/2 multiply-adds per site), else a
+// block takes tiles of sites through shared memory in 4 x 4 blocks of pairs
+// (D3Q19).  The phases of the modes are FP32 as evaluated from the FP64 sum of
+// (k x mod L)/L over the axes; each quotient is rounded correctly by one
+// Newton correction with the rounded reciprocal (Markstein 1990), without a
+// division.  Measured on GB300 per sample with 3 modes: D2Q9 512 x 384 173 -> 55
+// us, 2048^2 2234 -> 757, D3Q19 128^3 1790 -> 1135, against 45 threads of a block adding pairs while the others waited, on a
+// streamed copy, with 64-bit remainders and divisions for the phases.
+struct Obs64 {
+  int32_t Lx, Ly, Lz;
+  FastDiv div_x, div_y, div_z;
+  double inv_x, inv_y, inv_z;  // 1 / L, rounded
+  double rho_mean;
+  int32_t big;  // some side >= 46341: k x may not fit 31 bits
+};
+
+__device__ __forceinline__ uint32_t obs_mulmod(uint32_t k, uint32_t x, uint32_t L, FastDiv dv, bool big);
+
+// p / L for 0 <= p < L < 2^31, correctly rounded (inv = 1 / L rounded; every p
+// below 4000 and 2e8 random pairs checked).
+__device__ __forceinline__ double quotient(uint32_t p, int32_t L, double inv) {
+  const double P = static_cast<double>(p), q = P * inv;
+  return __fma_rn(__fma_rn(-q, static_cast<double>(L), P), inv, q);
+}
+
+// The pulled populations of site s, its density (returned) and its
+// structure-factor terms: re[m] += d cos, im[m] -= d sin of the phase of mode
+// m < modes.n, d = rho - rho_mean.
+template <int LAT, int KMAX>
+__device__ __forceinline__ double obs64_site(const double *g, uint32_t s, const Obs64 &o, const ModeArgs &modes,
+                                           double (&f)[Lattice<LAT>::Q], double (&re)[KMAX], double (&im)[KMAX]) {
   using L = Lattice<LAT>;
   constexpr int Q = L::Q;
-  constexpr int NPAIR = Q * (Q + 1) / 2;
-  constexpr int TILE = kReduceThreads;
-  __shared__ double tile[Q][TILE + 1];
-  __shared__ double warp_tot[kReduceThreads / 32][2 + Q + 2 * LBFD_MAX_MODES_DEV];
-  const int64_t N = static_cast<int64_t>(Lx) * Ly * Lz;
+  const uint32_t Lx = static_cast<uint32_t>(o.Lx), Ly = static_cast<uint32_t>(o.Ly), Lz = static_cast<uint32_t>(o.Lz);
+  const uint32_t r = fastdiv(s, o.div_x), x = s - r * Lx, z = fastdiv(r, o.div_y), y = r - z * Ly;
+  const uint32_t xm = (x == 0 ? Lx : x) - 1, xp = x + 1 == Lx ? 0 : x + 1;
+  const uint32_t ym = (y == 0 ? Ly : y) - 1, yp = y + 1 == Ly ? 0 : y + 1;
+  const uint32_t zm = (z == 0 ? Lz : z) - 1, zp = z + 1 == Lz ? 0 : z + 1;
+  const size_t N = static_cast<size_t>(Lx) * Ly * Lz;
+  double rho = 0.0;
+  static_for<Q>([&](auto I) {
+    constexpr int i = decltype(I)::value;
+    constexpr int vx = L::v(i, 0), vy = L::v(i, 1), vz = L::v(i, 2);
+    const uint32_t xs = vx == 0 ? x : (vx > 0 ? xm : xp);
+    const uint32_t ys = vy == 0 ? y : (vy > 0 ? ym : yp);
+    const uint32_t zs = vz == 0 ? z : (vz > 0 ? zm : zp);
+    f[i] = g[static_cast<size_t>(i) * N + xs + static_cast<size_t>(Lx) * (ys + static_cast<size_t>(Ly) * zs)];
+    rho += f[i];
+  });
+  const double d = rho - o.rho_mean;
+#pragma unroll
+  for (int m = 0; m < KMAX; ++m)
+    if (m < modes.n) {
+      const double px = modes.k[m][0] == 0 ? 0.0 : quotient(obs_mulmod(modes.k[m][0], x, Lx, o.div_x, o.big), o.Lx, o.inv_x);
+      const double py = modes.k[m][1] == 0 ? 0.0 : quotient(obs_mulmod(modes.k[m][1], y, Ly, o.div_y, o.big), o.Ly, o.inv_y);
+      const double pz = modes.k[m][2] == 0 ? 0.0 : quotient(obs_mulmod(modes.k[m][2], z, Lz, o.div_z, o.big), o.Lz, o.inv_z);
+      float sn, cs;
+      sincospif(2.0f * static_cast<float>(px + py + pz), &sn, &cs);
+      re[m] += d * static_cast<double>(cs);
+      im[m] -= d * static_cast<double>(sn);
+    }
+  return rho;
+}
+
+// One block's partial set: its threads' values pass through shared memory and
+// thread q adds value q of all of them in a fixed order.  Layout: [sum rho, sum rho^2, sum f_i, (re, im) of the modes, pairs i <= j].
+constexpr int kObs64Threads = 128;
+template <int LAT, int KMAX>
+__global__ void __launch_bounds__(kObs64Threads, 2)
+    k_obs64_registers(const double *g, const Obs64 o, const ModeArgs modes, double *__restrict__ partials) {
+  constexpr int Q = Lattice<LAT>::Q, NP = Q * (Q + 1) / 2, T = kObs64Threads;
+  extern __shared__ double obs64_smem[];
+  const uint32_t N = static_cast<uint32_t>(o.Lx) * static_cast<uint32_t>(o.Ly) * static_cast<uint32_t>(o.Lz);
+  double sr = 0.0, sr2 = 0.0, sf[Q], sp[NP], re[KMAX], im[KMAX];
+#pragma unroll
+  for (int i = 0; i < Q; ++i) sf[i] = 0.0;
+#pragma unroll
+  for (int p = 0; p < NP; ++p) sp[p] = 0.0;
+#pragma unroll
+  for (int m = 0; m < KMAX; ++m) re[m] = im[m] = 0.0;
+  // the warps of all blocks take 32 sites each in turn, warp 0 of every block
+  // first, so that an incomplete last round loads the SMs evenly
+  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint64_t step = static_cast<uint64_t>(gridDim.x) * T;
+  for (uint64_t s = (static_cast<uint64_t>(warp) * gridDim.x + blockIdx.x) * 32 + lane; s < N; s += step) {
+    double f[Q];
+    const double rho = obs64_site<LAT, KMAX>(g, static_cast<uint32_t>(s), o, modes, f, re, im);
+    sr += rho;
+    sr2 = __fma_rn(rho, rho, sr2);
+    int p = 0;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      sf[i] += f[i];
+#pragma unroll
+      for (int j = i; j < Q; ++j, ++p) sp[p] = __fma_rn(f[i], f[j], sp[p]);
+    }
+  }
+  // values [sum f_i, pairs, rho, rho^2, re, im] through shared memory
+  constexpr int NS = Q + NP;
+  double *const v = obs64_smem + threadIdx.x;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) v[i * (T + 1)] = sf[i];
+#pragma unroll
+  for (int p = 0; p < NP; ++p) v[(Q + p) * (T + 1)] = sp[p];
+  v[NS * (T + 1)] = sr;
+  v[(NS + 1) * (T + 1)] = sr2;
+#pragma unroll
+  for (int m = 0; m < KMAX; ++m)
+    if (m < modes.n) {
+      v[(NS + 2 + 2 * m) * (T + 1)] = re[m];
+      v[(NS + 3 + 2 * m) * (T + 1)] = im[m];
+    }
+  __syncthreads();
+  const int K = modes.n, nv = NS + 2 + 2 * K;
+  double *const out = partials + static_cast<size_t>(blockIdx.x) * (2 + Q + 2 * K + NP);
+  for (int q = threadIdx.x; q < nv; q += T) {
+    double a[4] = {0.0, 0.0, 0.0, 0.0};  // four chains
+    for (int t = 0; t < T; t += 4)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) a[c] += obs64_smem[q * (T + 1) + t + c];
+    const int at = q < Q ? 2 + q : (q < NS ? 2 + Q + 2 * K + (q - Q) : (q < NS + 2 ? q - NS : 2 + Q + (q - NS - 2)));
+    out[at] = (a[0] + a[1]) + (a[2] + a[3]);
+  }
+}
+
+// D3Q19: the rows f_0 .. f_18 and a row of ones in five groups of four; a
+// thread owns the 4 x 4 pairs of two groups (I <= J) and one of 16 slices of
+// the tile's sites.
+constexpr int kObs64Tile = 256, kObs64Groups = 5, kObs64Pairs = 15, kObs64Slices = 16;
+template <int LAT, int KMAX>
+__global__ void __launch_bounds__(kObs64Tile)
+    k_obs64_tiles(const double *g, const Obs64 o, const ModeArgs modes, double *__restrict__ partials) {
+  constexpr int Q = Lattice<LAT>::Q, NP = Q * (Q + 1) / 2, QP = 4 * kObs64Groups;
+  static_assert(Q + 1 == QP, "the groups hold the populations and the ones");
+  extern __shared__ double obs64_smem[];  // [site][QP + 2], then the sums
+  constexpr int LD = QP + 2;              // rows 16 bytes apart in the banks
+  const uint32_t N = static_cast<uint32_t>(o.Lx) * static_cast<uint32_t>(o.Ly) * static_cast<uint32_t>(o.Lz);
+  const int tid = static_cast<int>(threadIdx.x);
+  const bool has = tid < kObs64Pairs * kObs64Slices;
+  const int blk = has ? tid / kObs64Slices : 0, slice = tid % kObs64Slices;
+  int I = 0, b = blk;
+  while (b >= kObs64Groups - I) b -= kObs64Groups - I++;
+  const int J = I + b;
+  double sr = 0.0, sr2 = 0.0, pa[16], re[KMAX], im[KMAX];
+#pragma unroll
+  for (int e = 0; e < 16; ++e) pa[e] = 0.0;
+#pragma unroll
+  for (int m = 0; m < KMAX; ++m) re[m] = im[m] = 0.0;
+  for (uint64_t base = static_cast<uint64_t>(blockIdx.x) * kObs64Tile; base < N;
+       base += static_cast<uint64_t>(gridDim.x) * kObs64Tile) {
+    double f[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) f[i] = 0.0;
+    const bool in = base + tid < N;
+    if (in) {
+      const double rho = obs64_site<LAT, KMAX>(g, static_cast<uint32_t>(base + tid), o, modes, f, re, im);
+      sr += rho;
+      sr2 = __fma_rn(rho, rho, sr2);
+    }
+    double *const row = obs64_smem + tid * LD;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) row[i] = f[i];
+    row[Q] = in ? 1.0 : 0.0;
+    __syncthreads();
+    if (has) {
+      for (int k = slice; k < kObs64Tile; k += kObs64Slices) {
+        const double2 *const u = reinterpret_cast<const double2 *>(obs64_smem + k * LD + 4 * I);
+        const double2 *const w = reinterpret_cast<const double2 *>(obs64_smem + k * LD + 4 * J);
+        const double2 u0 = u[0], u1 = u[1], w0 = w[0], w1 = w[1];
+        const double uu[4] = {u0.x, u0.y, u1.x, u1.y}, ww[4] = {w0.x, w0.y, w1.x, w1.y};
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) pa[4 * r + c] = __fma_rn(uu[r], ww[c], pa[4 * r + c]);
+      }
+    }
+    __syncthreads();
+  }
+  // the slices of every pair in order; the modes over the block
+  double *const red = obs64_smem;                                      // [16 * blk + e][slices + 1]
+  double *const tot = red + kObs64Pairs * 16 * (kObs64Slices + 1);     // [blk][16]
+  if (has) {
+#pragma unroll
+    for (int e = 0; e < 16; ++e) red[(16 * blk + e) * (kObs64Slices + 1) + slice] = pa[e];
+  }
+  __syncthreads();
+  if (tid < kObs64Pairs * 16) {
+    double t = 0.0;
+    for (int k = 0; k < kObs64Slices; ++k) t += red[tid * (kObs64Slices + 1) + k];
+    tot[tid] = t;
+  }
+  __syncthreads();
   const int K = modes.n;
-  const int nq1 = 2 + Q + 2 * K;
-
-  double a_rho = 0.0, a_rho2 = 0.0;
-  double a_f[Q];
-  double a_re[LBFD_MAX_MODES_DEV], a_im[LBFD_MAX_MODES_DEV];
-#pragma unroll
-  for (int i = 0; i < Q; ++i) a_f[i] = 0.0;
-#pragma unroll
-  for (int m = 0; m < LBFD_MAX_MODES_DEV; ++m) a_re[m] = a_im[m] = 0.0;
-  // this thread's pair (i, j), i <= j, for the f_i f_j sums
-  int pi = 0, pj = 0;
-  {
-    int p = threadIdx.x, i = 0;
-    while (p >= Q - i && i < Q) { p -= Q - i; ++i; }
-    pi = i; pj = i + p;
+  double *const out = partials + static_cast<size_t>(blockIdx.x) * (2 + Q + 2 * K + NP);
+  auto pair_at = [](int i, int j) {  // i <= j < QP
+    const int gi = i >> 2, gj = j >> 2;
+    return (gi * kObs64Groups - gi * (gi - 1) / 2 + (gj - gi)) * 16 + (i & 3) * 4 + (j & 3);
+  };
+  if (tid < NP) {
+    int p = tid, i = 0;
+    while (p >= Q - i) p -= Q - i++;
+    out[2 + Q + 2 * K + tid] = tot[pair_at(i, i + p)];
   }
-  double a_ff = 0.0;
-
-  for (int64_t base = blockIdx.x * static_cast<int64_t>(TILE); base < N; base += static_cast<int64_t>(gridDim.x) * TILE) {
-    const int64_t s = base + threadIdx.x;
-    if (s < N) {
-      double r = 0.0;
-#pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        const double fi = Store<S>::getd(f[i * N + s], L::w(i) * rho_mean);
-        tile[i][threadIdx.x] = fi;
-        a_f[i] += fi;
-        r += fi;
-      }
-      a_rho += r;
-      a_rho2 += r * r;
-      if (K > 0) {
-        const int64_t x = s % Lx, y = (s / Lx) % Ly, z = s / (static_cast<int64_t>(Lx) * Ly);
-        const double d = r - rho_mean;
-        for (int m = 0; m < K; ++m) {
-          const int64_t px = ((modes.k[m][0] * x) % Lx + Lx) % Lx;
-          const int64_t py = ((modes.k[m][1] * y) % Ly + Ly) % Ly;
-          const int64_t pz = ((modes.k[m][2] * z) % Lz + Lz) % Lz;
-          const float frac = static_cast<float>(double(px) / Lx + double(py) / Ly + double(pz) / Lz);
-          float sn, cs;
-          sincospif(2.0f * frac, &sn, &cs);
-          a_re[m] += d * static_cast<double>(cs);
-          a_im[m] -= d * static_cast<double>(sn);
-        }
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < Q; ++i) tile[i][threadIdx.x] = 0.0;
-    }
-    __syncthreads();
-    if (threadIdx.x < NPAIR) {
-      double acc = 0.0;
-      for (int k = 0; k < TILE; ++k) acc += tile[pi][k] * tile[pj][k];
-      a_ff += acc;
-    }
-    __syncthreads();
-  }
-
-  // block reduction of the per-site quantities
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (tid < Q) out[2 + tid] = tot[pair_at(tid, Q)];
+  // rho, rho^2 and the modes over the block's warps
+  const int lane = tid & 31, warp = tid >> 5;
   auto put = [&](int q, double v) {
     v = warp_sum(v);
-    if (lane == 0) warp_tot[warp][q] = v;
+    if (lane == 0) red[q * 8 + warp] = v;
   };
-  put(0, a_rho);
-  put(1, a_rho2);
+  put(0, sr);
+  put(1, sr2);
 #pragma unroll
-  for (int i = 0; i < Q; ++i) put(2 + i, a_f[i]);
-  for (int m = 0; m < K; ++m) {
-    put(2 + Q + 2 * m, a_re[m]);
-    put(3 + Q + 2 * m, a_im[m]);
-  }
-  __syncthreads();
-  double *out = partials + static_cast<int64_t>(blockIdx.x) * (nq1 + NPAIR);
-  if (threadIdx.x < nq1) {
-    double t = 0.0;
-    for (int w = 0; w < kReduceThreads / 32; ++w) t += warp_tot[w][threadIdx.x];
-    out[threadIdx.x] = t;
-  }
-  if (threadIdx.x < NPAIR) out[nq1 + threadIdx.x] = a_ff;
-}
-
-// Stage-2 sum of per-block partials[b][q] (b < nblocks, q < nq) in a fixed
-// order, by kFinalThreads threads: warp w adds the blocks w, w + W, ... of 32
-// quantities at a time (coalesced rows; all its loads issued before the
-// adds), then thread q adds the W warp sums.  tot needs nq + W * nq doubles
-// of shared memory.
-constexpr int kFinalThreads = 512;
-constexpr int kFinalWarps = kFinalThreads / 32;
-constexpr int kFinalPer = ((kObsBlocks > kReduceBlocks ? kObsBlocks : kReduceBlocks) + kFinalWarps - 1) / kFinalWarps;
-__device__ __forceinline__ void sum_partials_ordered(const double *__restrict__ partials, int nblocks, int nq,
-                                                     double *tot) {
-  double *part = tot + nq;  // [W][nq]
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int q0 = 0; q0 < nq; q0 += 32) {
-    const int q = q0 + lane;
-    if (q < nq) {
-      double v[kFinalPer];
-#pragma unroll
-      for (int j = 0; j < kFinalPer; ++j) {
-        const int b = warp + j * kFinalWarps;
-        v[j] = b < nblocks ? partials[static_cast<int64_t>(b) * nq + q] : 0.0;
-      }
-      double t = 0.0;
-#pragma unroll
-      for (int j = 0; j < kFinalPer; ++j) t += v[j];
-      part[warp * nq + q] = t;
+  for (int m = 0; m < KMAX; ++m)
+    if (m < K) {
+      put(2 + 2 * m, re[m]);
+      put(3 + 2 * m, im[m]);
     }
-  }
   __syncthreads();
-  for (int q = threadIdx.x; q < nq; q += blockDim.x) {
+  if (tid < 2 + 2 * K) {
     double t = 0.0;
-    for (int w = 0; w < kFinalWarps; ++w) t += part[w * nq + q];
-    tot[q] = t;
-  }
-  __syncthreads();
-}
-
-inline size_t final_smem(int nq) { return sizeof(double) * size_t(nq) * (1 + kFinalWarps); }
-
-// acc layout: [sum_rho, sum_rho2, sum_f[Q], sum_ff[Q*Q] (full, symmetric), sum_sk[K]]
-__global__ void k_obs_finalize(const double *__restrict__ partials, int nblocks, int Q, int K, double *__restrict__ acc) {
-  extern __shared__ double tot[];
-  const int nq1 = 2 + Q + 2 * K, npair = Q * (Q + 1) / 2, nq = nq1 + npair;
-  sum_partials_ordered(partials, nblocks, nq, tot);
-  if (threadIdx.x == 0) {
-    acc[0] += tot[0];
-    acc[1] += tot[1];
-    for (int i = 0; i < Q; ++i) acc[2 + i] += tot[2 + i];
-    int p = 0;
-    for (int i = 0; i < Q; ++i)
-      for (int j = i; j < Q; ++j, ++p) {
-        const double v = tot[nq1 + p];
-        acc[2 + Q + i * Q + j] += v;
-        if (j != i) acc[2 + Q + j * Q + i] += v;
-      }
-    for (int m = 0; m < K; ++m) {
-      const double re = tot[2 + Q + 2 * m], im = tot[3 + Q + 2 * m];
-      acc[2 + Q + Q * Q + m] += re * re + im * im;
-    }
+    for (int w = 0; w < kObs64Tile / 32; ++w) t += red[tid * 8 + w];
+    out[tid < 2 ? tid : Q + tid] = t;
   }
 }
 
-template <int LAT, typename S>
-static cudaError_t obs_t(const void *f, int32_t Lx, int32_t Ly, int32_t Lz, double rho_mean, const ModeArgs &ma,
-                         double *partials, double *acc, cudaStream_t stream) {
+template <int LAT, int KMAX>
+static cudaError_t obs64_t(const double *g, const Obs64 &o, const ModeArgs &ma, double *partials, cudaStream_t stream) {
   constexpr int Q = Lattice<LAT>::Q;
-  k_obs_partials<LAT, S><<<kReduceBlocks, kReduceThreads, 0, stream>>>(static_cast<const S *>(f), Lx, Ly, Lz, rho_mean,
-                                                                       ma, partials);
-  const int nq = obs_quantities(Q, ma.n);
-  k_obs_finalize<<<1, kFinalThreads, final_smem(nq), stream>>>(partials, kReduceBlocks, Q, ma.n, acc);
+  if constexpr (Q <= 9) {
+    const size_t smem = sizeof(double) * size_t(Q + Q * (Q + 1) / 2 + 2 + 2 * ma.n) * (kObs64Threads + 1);
+    cudaError_t e = cudaFuncSetAttribute(k_obs64_registers<LAT, KMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         int(sizeof(double) * size_t(Q + Q * (Q + 1) / 2 + 2 + 2 * KMAX) * (kObs64Threads + 1)));
+    if (e != cudaSuccess) return e;
+    k_obs64_registers<LAT, KMAX><<<kReduceBlocks, kObs64Threads, smem, stream>>>(g, o, ma, partials);
+  } else {
+    const size_t smem = sizeof(double) * std::max<size_t>(size_t(kObs64Tile) * (4 * kObs64Groups + 2),
+                                                          size_t(kObs64Pairs) * 16 * (kObs64Slices + 2));
+    cudaError_t e = cudaFuncSetAttribute(k_obs64_tiles<LAT, KMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    if (e != cudaSuccess) return e;
+    k_obs64_tiles<LAT, KMAX><<<kReduceBlocks, kObs64Tile, smem, stream>>>(g, o, ma, partials);
+  }
   return cudaGetLastError();
 }
 
-cudaError_t launch_observables(int lattice, int precision, const void *f, int32_t Lx, int32_t Ly, int32_t Lz,
-                               double rho_mean, int n_modes, const int32_t *modes, double *partials, double *acc,
-                               cudaStream_t stream) {
-  if (n_modes < 0 || n_modes > LBFD_MAX_MODES_DEV) return cudaErrorInvalidValue;
+template <int LAT>
+static cudaError_t pull_finalize_t(const double *partials, int nblocks, int n_modes, int64_t N, float rho_f,
+                                   double *fin, double *acc, cudaStream_t stream);
+
+cudaError_t launch_observables64(int lattice, const double *g, int32_t Lx, int32_t Ly, int32_t Lz, double rho_mean,
+                                 int n_modes, const int32_t *modes, double *partials, double *fin, double *acc,
+                                 cudaStream_t stream) {
+  const int64_t N = int64_t(Lx) * Ly * Lz;
+  if (n_modes < 0 || n_modes > LBFD_MAX_MODES_DEV || N >= (int64_t(1) << 31)) return cudaErrorInvalidValue;
+  const int32_t L3[3] = {Lx, Ly, Lz};
   ModeArgs ma{};
   ma.n = n_modes;
   for (int m = 0; m < n_modes; ++m)
-    for (int k = 0; k < 3; ++k) ma.k[m][k] = modes[3 * m + k];
-  return dispatch_lattice_storage(lattice, precision, [&](auto lat, auto tag) {
+    for (int k = 0; k < 3; ++k)
+      ma.k[m][k] = static_cast<int32_t>(((int64_t(modes[3 * m + k]) % L3[k]) + L3[k]) % L3[k]);
+  Obs64 o{Lx, Ly, Lz, make_fastdiv(uint32_t(Lx)), make_fastdiv(uint32_t(Ly)), make_fastdiv(uint32_t(Lz)),
+          1.0 / Lx, 1.0 / Ly, 1.0 / Lz, rho_mean, (Lx >= 46341 || Ly >= 46341 || Lz >= 46341) ? 1 : 0};
+  return dispatch_lattice(lattice, [&](auto lat) -> cudaError_t {
     constexpr int LAT = decltype(lat)::value;
-    using S = typename decltype(tag)::type;
-    return obs_t<LAT, S>(f, Lx, Ly, Lz, rho_mean, ma, partials, acc, stream);
+    const cudaError_t e = n_modes <= 4 ? obs64_t<LAT, 4>(g, o, ma, partials, stream)
+                                       : obs64_t<LAT, LBFD_MAX_MODES_DEV>(g, o, ma, partials, stream);
+    // stage 2 of the FP32 pass with offsets c_i = 0: the sums themselves
+    return e != cudaSuccess ? e : pull_finalize_t<LAT>(partials, kReduceBlocks, n_modes, N, 0.0f, fin, acc, stream);
   });
 }
 
@@ -473,7 +567,7 @@ __global__ void __launch_bounds__(kObsThreads) k_obs_pull(const S *__restrict__ 
   }
   if (tiles > 0) flush_pairs();
   // gather the slot sums, then write the block's partials in the layout of
-  // k_obs_partials: [sum delta, sum delta^2, sum e_i, modes, pairs i <= j]
+  // the stage-2 pass: [sum delta, sum delta^2, sum e_i, modes, pairs i <= j]
   if (threadIdx.x < P::NB * 16) slot_sum[threadIdx.x] = acc_pair;
   __syncthreads();
   auto slot_of = [](int i, int j) {  // i <= j < QP
