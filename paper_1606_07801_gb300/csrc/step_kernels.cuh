@@ -624,7 +624,9 @@ struct StepLaunch {
 template <int LAT, typename S, int NOISE, typename Idx>
 cudaError_t step_noise_idx(const S *s, S *d, const StepArgs &a, int vx, cudaStream_t stream) {
   dim3 grid, block;
-  step_shape(a.Lx, a.Ly, a.Lz, grid, block, vx, step_threads(LAT, sizeof(typename Store<S>::R) == 8 ? kStoreF64 : kStoreF32));
+  step_shape(a.Lx, a.Ly, a.Lz, grid, block, vx,
+             step_threads(LAT, sizeof(typename Store<S>::R) == 8 ? kStoreF64 : kStoreF32,
+                          NOISE == kStepNoiseOff && !(LAT == kD3Q19 && Store<S>::kDeviation)));
   StepLaunch launch(grid, block, stream);
   const SrtCollideFor<LAT, S, NOISE> c;
   using C = SrtCollideFor<LAT, S, NOISE>;

@@ -51,9 +51,12 @@ inline int step_vec_width(int lattice, int precision, int32_t Lx, int64_t sites 
 // 18.8 us with 256 threads and two sites each, 6.1 with 32 and one; D3Q19
 // 64^3 168.8 and 147.4).  FP32 arithmetic: 128 for the lattices whose
 // registers fill the SM, a finer last wave at the same occupancy (D3Q19 FP32
-// 64^3 9.3 -> 8.3 us, 128^3 54.5 -> 53.6, FP16 128^3 51.3 -> 49.1).
-inline int step_threads(int lattice, int precision) {
-  return precision == kStoreF64 ? 32 : (lattice == kD1Q3 ? 256 : 128);
+// 64^3 9.3 -> 8.3 us, 128^3 54.5 -> 53.6, FP16 128^3 51.3 -> 49.1), but 256
+// where they do not (`few`): without noise (D2Q9 FP32 623 x 1187 7.1 against
+// 7.6, D3Q19 FP32 50^3 3.9 against 4.2), but for D3Q19 in a 16-bit format
+// (100^3 11.4 against 9.8 with 128).
+inline int step_threads(int lattice, int precision, bool few = false) {
+  return precision == kStoreF64 ? 32 : (lattice == kD1Q3 || few ? 256 : 128);
 }
 
 // Block and grid of the one-launch-per-step kernels for vx sites per thread:
