@@ -383,7 +383,7 @@ int lbfd_mass_noalloc(int32_t lattice, int32_t precision, const void *f_dev, int
  * same noise keys).  Members share one precision, noise mode and law, and
  * each member has Q * sites < 2^32.  Work decomposition: a work item is 1
  * or 2 sites of a row (neighbours where Lx is even, else one of each half of
- * the row), a tile is at most `passes` x 256 items of one member, and the tiles go to blocks in one of the orders
+ * the row), a tile is at most `passes` x 128 items of one member, and the tiles go to blocks in one of the orders
  * LBFD_WALK_* (see lbfd_ensemble_tune / lbfd_ensemble_plan). */
 typedef struct lbfd_member {
     int64_t dims[3];    /* Lx, Ly, Lz; trailing dims of lower-D lattices must be 1 */

@@ -31,7 +31,7 @@ int batch_build_params(const BatchMember *members, int n, int64_t ntiles, int no
 // wave that is nearly empty costs more than longer tiles save).
 int batch_passes(const BatchMember *members, int n, int passes, int64_t slots);
 
-// Assigns consecutive tiles of passes x 256 items to members[0..n) in order
+// Assigns consecutive tiles of passes x 128 items to members[0..n) in order
 // (tile0 and tile_start[m]); returns the number of tiles.
 int64_t batch_assign_tiles(BatchMember *members, int n, int passes, int64_t *tile_start);
 

@@ -10,7 +10,7 @@
 // the stored state is in block t & 1 and the step writes block (t & 1) ^ 1.
 //
 // Work.  Member m owns tiles [tile_start[m], tile_start[m + 1]) of a flat
-// tile list; a tile is `passes` x 256 consecutive work items of one member,
+// tile list; a tile is `passes` x 128 consecutive work items of one member,
 // and an item is vx sites of a row: neighbours where Lx is even, a site of the
 // row's first half and its twin in the second where it is odd (twin_update;
 // D3Q19 takes one site there).
@@ -35,7 +35,12 @@
 
 namespace lbfd {
 
-constexpr int kBatchThreads = 256;
+// Threads of a block: small blocks end a launch more evenly.  128 against 256
+// in the parameter-space launches on GB300, GLUPS: 60 D2Q9 members of 96..512
+// a side 78.5 and 75.7 (FP16 78.1 and 76.8), 20 of 30..80 24.8 and 21.1, 40
+// D3Q19 members of 32..128 38.5 and 37.8, 8 of 30..60 32.0 and 30.2, 600 D2Q9
+// members 83.7 and 83.2.
+constexpr int kBatchThreads = 128;
 // Order in which blocks take tiles: a persistent grid whose blocks take every
 // grid-th tile (strided) or one run of consecutive tiles (contiguous), one
 // block per tile, or one block per tile with the members' arguments in the
@@ -118,12 +123,12 @@ __device__ __forceinline__ int batch_find_member(const int64_t *__restrict__ til
 }
 
 // Minimum resident blocks per SM asked of the register allocator: occupancy
-// variant 0 is 4 blocks (64 registers; D3Q19 with its arguments in shared
-// memory, which the compiler cannot keep as uniform operands, 3; FP64 2),
-// variant 1 one block fewer; the tuner picks between them.
+// variant 0 is 8 blocks (64 registers; D3Q19 with its arguments in shared
+// memory, which the compiler cannot keep as uniform operands, 6; FP64 4),
+// variant 1 two blocks fewer; the tuner picks between them.
 template <int LAT, typename S, int OCC, bool PARAM>
 constexpr int batch_min_blocks() {
-  return (sizeof(typename Store<S>::R) != 4 ? 2 : (LAT == kD3Q19 && !PARAM ? 3 : 4)) - OCC;
+  return (sizeof(typename Store<S>::R) != 4 ? 4 : (LAT == kD3Q19 && !PARAM ? 6 : 8)) - 2 * OCC;
 }
 
 // The collision of pairs without the packed form (FP64, no noise): one site
