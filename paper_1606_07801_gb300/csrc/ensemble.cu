@@ -20,6 +20,7 @@ using namespace lbfd;
 namespace {
 
 constexpr int kGraphSteps = 16;  // steps per captured graph
+constexpr size_t kPieceBytes = size_t(512) << 10;  // a piece of a read-out (stage)
 
 int ens_fail(int code, const std::string &msg) { return set_last_error(code, msg); }
 
@@ -78,6 +79,10 @@ struct lbfd_ens {
   static constexpr int kSide = 4;
   cudaStream_t side[kSide] = {};
   cudaEvent_t fork_ev = nullptr, join_ev[kSide] = {};
+  // pinned staging of the read-outs, two pieces: one is copied while the other
+  // is decoded (made by the first read-out)
+  char *stage = nullptr;
+  cudaEvent_t stage_ev[2] = {};
   // member m's block holding its stored state (which = 0) or the spare one (1)
   char *block(int m, int which) const {
     const int p = static_cast<int>(t & 1) ^ which;
@@ -171,6 +176,9 @@ static void ens_free(lbfd_ens *e) {
     if (e->join_ev[k]) cudaEventDestroy(e->join_ev[k]);
   }
   if (e->fork_ev) cudaEventDestroy(e->fork_ev);
+  for (cudaEvent_t ev : e->stage_ev)
+    if (ev) cudaEventDestroy(ev);
+  cudaFreeHost(e->stage);
   if (e->owns_stream) cudaStreamDestroy(e->stream);
   delete e;
 }
@@ -463,26 +471,45 @@ int lbfd_ensemble_query(lbfd_ens_t e, int32_t *n_members, int64_t *total_sites, 
 
 static int ens_member_ok(lbfd_ens_t e, int32_t m) { return e && m >= 0 && m < e->n; }
 
+// The state leaves in pieces through pinned memory, each decoded while the
+// next is copied: pageable memory is copied through the driver's own staging
+// and has to be allocated, cleared and read once more.
 int lbfd_ensemble_get_f(lbfd_ens_t e, int32_t member, double *f_host) {
   if (!ens_member_ok(e, member) || !f_host) return ens_fail(LBFD_EINVAL, "lbfd_ensemble_get_f: bad argument");
   DevGuard g(e->device);
   const BatchMember &bm = e->hmem[member];
-  const size_t count = size_t(e->Q) * bm.N;
+  const size_t count = size_t(e->Q) * bm.N, piece = kPieceBytes / e->elem, pieces = (count + piece - 1) / piece;
+  for (cudaEvent_t &ev : e->stage_ev)
+    if (!ev) ENS_CU(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+  if (!e->stage) ENS_CU(cudaHostAlloc(reinterpret_cast<void **>(&e->stage), 2 * kPieceBytes, cudaHostAllocDefault));
   ENS_CU(launch_shift(e->lattice, e->elem, e->block(member, 0), e->block(member, 1), bm.Lx, bm.Ly, bm.Lz, +1,
                       e->stream));
-  std::vector<uint8_t> raw(count * e->elem);
-  ENS_CU(cudaMemcpyAsync(raw.data(), e->block(member, 1), raw.size(), cudaMemcpyDeviceToHost, e->stream));
-  ENS_CU(cudaStreamSynchronize(e->stream));
+  const char *from = e->block(member, 1);
+  auto fetch = [&](size_t k) -> cudaError_t {
+    const size_t n = std::min(piece, count - k * piece);
+    const cudaError_t err = cudaMemcpyAsync(e->stage + (k & 1) * kPieceBytes, from + k * piece * e->elem, n * e->elem,
+                                            cudaMemcpyDeviceToHost, e->stream);
+    return err == cudaSuccess ? cudaEventRecord(e->stage_ev[k & 1], e->stream) : err;
+  };
   int Q = 0, D = 0, v[LBFD_MAX_Q * 3];
   double w[LBFD_MAX_Q];
   lattice_table(e->lattice, &Q, &D, v, w);
-  dispatch_storage(e->precision, [&](auto tag) {
-    using S = typename decltype(tag)::type;
-    const S *p = reinterpret_cast<const S *>(raw.data());
-    for (int i = 0; i < Q; ++i)
-      for (int64_t s = 0; s < bm.N; ++s) f_host[i * bm.N + s] = Store<S>::getd(p[i * bm.N + s], w[i] * bm.rho_mean);
-    return cudaSuccess;
-  });
+  ENS_CU(fetch(0));
+  for (size_t k = 0; k < pieces; ++k) {
+    if (k + 1 < pieces) ENS_CU(fetch(k + 1));
+    ENS_CU(cudaEventSynchronize(e->stage_ev[k & 1]));
+    dispatch_storage(e->precision, [&](auto tag) {
+      using S = typename decltype(tag)::type;
+      const S *p = reinterpret_cast<const S *>(e->stage + (k & 1) * kPieceBytes);
+      const size_t end = std::min(count, (k + 1) * piece);
+      for (size_t at = k * piece; at < end;) {  // the piece's part of one population after the other
+        const size_t i = at / size_t(bm.N), stop = std::min(end, (i + 1) * size_t(bm.N));
+        const double wr = w[i] * bm.rho_mean;
+        for (; at < stop; ++at) f_host[at] = Store<S>::getd(*p++, wr);
+      }
+      return cudaSuccess;
+    });
+  }
   return LBFD_OK;
 }
 
