@@ -582,7 +582,7 @@ int lbfd_step(lbfd_t h, int64_t n) {
     vec_width = step_vec_width(o.lattice, o.precision, a.Lx, h->N);
     if (vec_width == 1) vec_width = 2;  // asked for by step_kernel: Lx is even
   }
-  const bool fusable = o.sample_every > 0 && !h->mrt &&
+  const bool fusable = o.sample_every > 0 && !h->mrt && sample_fused_pays(o.lattice, h->N) &&
                        sample_fusable(o.lattice, o.precision, a.Lx, a.Ly, a.Lz, o.n_modes, h->phase);
   int64_t extra = 0;  // launches besides one step kernel per step
   for (int64_t k = 0; k < n; ++k) {

@@ -266,6 +266,32 @@ __host__ __device__ __forceinline__ float obs_offset(int i, float rho_f) {
   return mul_rn(static_cast<float>(Lattice<LAT>::w(i)), rho_f);
 }
 
+// sum delta and sum delta^2 of a partial set, delta = sum_i e_i, from its sums
+// of e_i and its pair sums: sum(i), and pair(i, j, p) for the p-th pair i <= j.
+// Called by one full warp (one thread's chain of Q (Q + 1) / 2 dependent FP64
+// additions took 6 us of every block's end for D3Q19 on GB300).
+template <int Q, class Sum, class Pair>
+__device__ __forceinline__ void obs_delta_sums(Sum sum, Pair pair, double *out, int lane) {
+  double sd = lane < Q ? sum(lane) : 0.0, sd2 = 0.0;
+  for (int p0 = lane; p0 < Q * (Q + 1) / 2; p0 += 32) {
+    int p = p0, i = 0;
+    while (p >= Q - i) {
+      p -= Q - i;
+      ++i;
+    }
+    sd2 += (p == 0 ? 1.0 : 2.0) * pair(i, i + p, p0);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    sd += __shfl_xor_sync(0xffffffffu, sd, o);
+    sd2 += __shfl_xor_sync(0xffffffffu, sd2, o);
+  }
+  if (lane == 0) {
+    out[0] = sd;
+    out[1] = sd2;
+  }
+}
+
 // Entry k of the observable accumulators ([sum rho, sum rho^2, sum f_i (Q),
 // sum f_i f_j (Q x Q), |rho(k_m)|^2 (K)]) from the totals tt of a sample's
 // deviation sums in the layout of the FP32 observable pass ([sum delta,
@@ -316,6 +342,25 @@ inline bool sample_fusable(int lattice, int precision, int32_t Lx, int32_t Ly, i
   dim3 grid, block;
   step_shape(Lx, Ly, Lz, grid, block, step_vec_width(lattice, precision, Lx) >= 2 ? 2 : 1);
   return block.x * block.y == 256 && block.x % 32 == 0;
+}
+// LBFD_SAMPLE_STAGED = 1: D3Q19 samples in the staged kernel (step_sample_t).
+inline bool sample_staged_default() {
+  static const bool v = [] {
+    const char *e = getenv("LBFD_SAMPLE_STAGED");
+    return e && atoi(e) == 1;
+  }();
+  return v;
+}
+
+// Whether a sampled step of a lattice that can fuse takes the fused kernel,
+// or the separate pass and a plain step: a large D3Q19 lattice's plain step
+// gains more from blocks and registers of its own than one pull saves.  On
+// GB300, microseconds per step at a sample every 5 steps, fused and separate:
+// D3Q19 FP32 64^3 11.1 and 13.5, 128^3 65.8 and 66.5, 200^3 298.8 and 287.3,
+// 256^3 491.2 and 490.9, FP16 200^3 285.2 and 270.9; D2Q9 FP32 512^2 5.5 and
+// 7.0, 2048^2 54.6 and 55.4.
+inline bool sample_fused_pays(int lattice, int64_t N) {
+  return lattice != kD3Q19 || N < (int64_t(1) << 22) || sample_staged_default();
 }
 cudaError_t launch_step_sample_d1q3(int precision, const void *src, void *dst, const StepArgs &a, int n_modes,
                                     const void *phase, double *partials, int *nblocks, bool staged_ok,

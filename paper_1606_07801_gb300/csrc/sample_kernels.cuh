@@ -296,7 +296,7 @@ struct WarpSampler {
 // populations (D1Q3, D2Q9): every lane adds its own sites' products into
 // FP32 registers (the Q(Q+1)/2 pair sums e_i e_j, i <= j, the Q sums e_i and
 // the mode sums), with no shared memory and no exchange per site.  After at
-// most kThreadFoldSites sites a butterfly adds each value over the warp in
+// most kThreadFoldSites sites every value is added over the warp in
 // FP32 (5 more roundings), and the lanes add the totals, two per lane, to the
 // warp's FP64 values.  Same interface as WarpSampler.
 constexpr int kThreadFoldSites = 128;
@@ -326,21 +326,31 @@ struct ThreadSampler {
     __syncwarp();
   }
 
-  // FP32 sums over the warp (butterfly), then into the FP64 values: lane l
-  // adds totals l and l + 32.  Called by all lanes.
+  // FP32 sums over the warp, then into the FP64 values.  Each exchange halves
+  // the values a lane holds (those whose next index bit is the lane's), so all
+  // sums take NV exchanges instead of five each, with the additions of a
+  // butterfly; lane l ends with the totals kEach l .. kEach (l + 1) - 1.
+  // Called by all lanes.
+  static constexpr int kEach = NV <= 32 ? 1 : 2;
   __device__ __forceinline__ void flush(int) {
-    float t0 = 0.0f, t1 = 0.0f;
+    float v[32 * kEach];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      float t = acc[k];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      if (k == lane) t0 = t;
-      if (k == lane + 32) t1 = t;
-      acc[k] = 0.0f;
+    for (int k = 0; k < 32 * kEach; ++k) {
+      v[k] = k < NV ? acc[k < NV ? k : 0] : 0.0f;
+      if (k < NV) acc[k < NV ? k : 0] = 0.0f;
     }
-    if (lane < NV) sm->v[lane] += static_cast<double>(t0);
-    if (lane + 32 < NV) sm->v[lane + 32] += static_cast<double>(t1);
+    static_for<5>([&](auto B) {
+      constexpr int o = 16 >> decltype(B)::value, n = o * kEach;  // n values stay
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int k = 0; k < n; ++k) {
+        const float other = __shfl_xor_sync(0xffffffffu, up ? v[k] : v[k + n], o);
+        v[k] = (up ? v[k + n] : v[k]) + other;
+      }
+    });
+#pragma unroll
+    for (int k = 0; k < kEach; ++k)
+      if (lane * kEach + k < NV) sm->v[lane * kEach + k] += static_cast<double>(v[k]);
     iters = 0;
   }
 
@@ -360,13 +370,22 @@ struct ThreadSampler {
                                       : sub_rn(static_cast<float>(f[k][i]), obs_offset<LAT>(i, sa.rho_f));
           delta += e[i];
         }
-        int p = 0;
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-#pragma unroll
-          for (int j = i; j < Q; ++j, ++p) acc[p] = fmaf(e[i], e[j], acc[p]);
-          acc[NP + i] += e[i];
-        }
+        // two pairs an instruction, (e_i e_j, e_i e_{j+1}) with j even and e_Q =
+        // 1 for the sum of e_i: 29 instructions a D2Q9 site instead of 54
+        static_assert(Q % 2 == 1, "(Q - 1, Q) is such a pair");
+        static_for<Q>([&](auto I) {
+          constexpr int i = decltype(I)::value, row = i * Q - i * (i - 1) / 2;  // pair (i, i)
+          const float2 ei = make_float2(e[i], e[i]);
+          if constexpr (i % 2 == 1) acc[row] = fma_rn(e[i], e[i], acc[row]);
+          static_for<Q / 2 + 1 - (i + 1) / 2>([&](auto J) {
+            constexpr int j = (i + 1) / 2 * 2 + 2 * decltype(J)::value;
+            constexpr int p0 = row + j - i, p1 = j + 1 < Q ? p0 + 1 : NP + i;
+            const float2 r = fma_rn(ei, make_float2(e[j], j + 1 < Q ? e[j + 1 < Q ? j + 1 : j] : 1.0f),
+                                    make_float2(acc[p0], acc[p1]));
+            acc[p0] = r.x;
+            acc[p1] = r.y;
+          });
+        });
         // structure factor, x part: sum_k d_k e^{-2 pi i k_x x / Lx}
         const float d = delta + sa.d_off;
 #pragma unroll
@@ -409,16 +428,8 @@ struct ThreadSampler {
     for (int p = tid; p < NP; p += nthreads) out[nq1 + p] = v[p];
     if (tid < Q) out[2 + tid] = v[NP + tid];
     if (tid < 2 * K) out[2 + Q + tid] = v[NP + Q + tid];
-    if (tid == 0) {
-      double sd = 0.0, sd2 = 0.0;
-      int p = 0;
-      for (int i = 0; i < Q; ++i) {
-        sd += v[NP + i];
-        for (int j = i; j < Q; ++j, ++p) sd2 += (i == j ? 1.0 : 2.0) * v[p];
-      }
-      out[0] = sd;
-      out[1] = sd2;
-    }
+    if (tid < 32)
+      obs_delta_sums<Q>([&](int i) { return v[NP + i]; }, [&](int, int, int p) { return v[p]; }, out, tid);
   }
 };
 
@@ -455,16 +466,9 @@ __device__ __forceinline__ void warp_sampler_partials(typename WarpSampler<LAT, 
   }
   if (tid < Q) out[2 + tid] = sl0[WS::slot(tid, Q)];
   if (tid < 2 * K) out[2 + Q + tid] = w[0].modes[tid];
-  if (tid == 0) {
-    double sd = 0.0, sd2 = 0.0;
-    for (int i = 0; i < Q; ++i) {
-      sd += sl0[WS::slot(i, Q)];
-      sd2 += sl0[WS::slot(i, i)];
-      for (int j = i + 1; j < Q; ++j) sd2 += 2.0 * sl0[WS::slot(i, j)];
-    }
-    out[0] = sd;
-    out[1] = sd2;
-  }
+  if (tid < 32)
+    obs_delta_sums<Q>([&](int i) { return sl0[WS::slot(i, Q)]; },
+                      [&](int i, int j, int) { return sl0[WS::slot(i, j)]; }, out, tid);
 }
 
 template <int LAT, int VX>
@@ -572,16 +576,31 @@ __global__ void __launch_bounds__(kSampleThreads, 2)
   const int warp = tid >> 5;
   WS ws;
   ws.init(&wsm[warp], tid & 31);
-  for (int vb = blockIdx.x; vb < sa.nvb; vb += gridDim.x) {
+  // the next sites are on their way while these are added: at 16 warps per SM
+  // (the accumulators) the loads' latency bound the pass (D2Q9 2048^2 62 -> 51
+  // us a sample on GB300)
+  R f[VX][Q], g[VX][Q];
+  int x0 = 0, y = 0, z = 0;
+  auto pull = [&](int vb, R (&to)[VX][Q]) -> bool {
     const int vbx = vb % sa.gx, vr = vb / sa.gx;
-    const int vby = vr % sa.gy, vbz = vr / sa.gy;
-    const int x0 = (vbx * static_cast<int>(blockDim.x) + static_cast<int>(threadIdx.x)) * VX;
-    const int y = vby * static_cast<int>(blockDim.y) + static_cast<int>(threadIdx.y);
-    const int z = vbz;
-    const bool active = x0 < a.Lx && y < a.Ly;
-    R f[VX][Q];
-    if (active) (void)vec_pull<LAT, S, VX, Idx>(src, a, x0, y, z, f);
-    ws.template add<S>(f, active, x0, y, z, a.Lx, a.Ly, a.Lz, sa);
+    const int vby = vr % sa.gy;
+    z = vr / sa.gy;
+    x0 = (vbx * static_cast<int>(blockDim.x) + static_cast<int>(threadIdx.x)) * VX;
+    y = vby * static_cast<int>(blockDim.y) + static_cast<int>(threadIdx.y);
+    const bool active = vb < sa.nvb && x0 < a.Lx && y < a.Ly;
+    if (active) (void)vec_pull<LAT, S, VX, Idx>(src, a, x0, y, z, to);
+    return active;
+  };
+  bool active = pull(blockIdx.x, f);
+  for (int vb = blockIdx.x; vb < sa.nvb; vb += gridDim.x) {
+    const int px = x0, py = y, pz = z;
+    const bool next = pull(vb + gridDim.x, g);
+    ws.template add<S>(f, active, px, py, pz, a.Lx, a.Ly, a.Lz, sa);
+#pragma unroll
+    for (int k = 0; k < VX; ++k)
+#pragma unroll
+      for (int i = 0; i < Q; ++i) f[k][i] = g[k][i];
+    active = next;
   }
   ws.flush(sa.K);
   __syncthreads();

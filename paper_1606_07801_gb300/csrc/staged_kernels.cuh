@@ -461,14 +461,6 @@ cudaError_t staged_t(const void *src, void *dst, const StepArgs &a, const Staged
 // staged kernel for D3Q19 where the lattice meets its requirements and two
 // of its blocks fit the 228 KB of shared memory of an SM (a tuning knob; the
 // results agree within FP32 rounding of the sums, and the state bit for bit).
-inline bool sample_staged_default() {
-  static const bool v = [] {
-    const char *e = getenv("LBFD_SAMPLE_STAGED");
-    return e && atoi(e) == 1;
-  }();
-  return v;
-}
-
 template <int LAT, typename S>
 cudaError_t step_sample_t(const void *src, void *dst, const StepArgs &a, int n_modes, const void *phase,
                           double *partials, int *nblocks, bool staged_ok, int *status, cudaStream_t stream) {
