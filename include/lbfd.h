@@ -85,9 +85,9 @@ extern "C" {
                                  global memory (Lx even); FP32-arithmetic formats collide two sites at a time
                                  on the packed FP32 instructions where that is faster, with the same result */
 #define LBFD_KERNEL_SCALAR 2  /* k_step: one site per thread (any Lx) */
-#define LBFD_KERNEL_SMALL 3   /* k_step_small: many steps per launch in one block's shared memory (small
+#define LBFD_KERNEL_SMALL 3   /* k_step_resident on one block: many steps per launch in its shared memory (small
                                  lattices, n >= 2; chosen automatically) */
-#define LBFD_KERNEL_CLUSTER 4 /* k_step_cluster: the same over a thread-block cluster (chosen automatically) */
+#define LBFD_KERNEL_CLUSTER 4 /* k_step_resident over a thread-block cluster (chosen automatically) */
 #define LBFD_KERNEL_MRT 5     /* k_step_mrt: moment-space collision (D2Q5, multiple relaxation times) */
 #define LBFD_KERNEL_STAGED 6  /* k_step_staged: persistent; each tile's source rows are copied into shared
                                  memory by the TMA unit (bulk asynchronous copies on an mbarrier), the sites
