@@ -95,13 +95,23 @@ BatchMember make_batch_member(int lattice, const int64_t dims[3], double tau, do
   return m;
 }
 
-int batch_build_params(const BatchMember *members, int n, int64_t ntiles, int noise_mode, int noise_dist,
+int batch_build_params(const BatchMember *members, int n, int64_t ntiles, int noise_mode, int noise_dist, int parts,
                        std::vector<BatchParams> &groups) {
   groups.clear();
-  for (int first = 0; first < n; first += kParamMembers) {
+  const int G = std::max((n + kParamMembers - 1) / kParamMembers, std::min(parts, n));
+  int64_t total = 0, sites = 0;
+  for (int m = 0; m < n; ++m) total += members[m].N;
+  for (int first = 0, g = 0; g < G; ++g) {
+    // up to the group's share of the sites; the groups after it can hold the rest and have a member each
+    const int after = G - 1 - g;
+    int last = first;
+    sites += members[last++].N;
+    while (last < n - after && last < first + kParamMembers &&
+           (n - last > after * kParamMembers || double(sites) * G < double(total) * (g + 1)))
+      sites += members[last++].N;
     BatchParams p{};
     p.first = first;
-    p.n = std::min(kParamMembers, n - first);
+    p.n = last - first;
     const int64_t base = members[first].tile0;
     for (int k = 0; k < p.n; ++k) {
       const BatchMember &mb = members[first + k];
@@ -114,6 +124,7 @@ int batch_build_params(const BatchMember *members, int n, int64_t ntiles, int no
     const int64_t end = first + p.n < n ? members[first + p.n].tile0 : ntiles;
     p.tile_start[p.n] = static_cast<int32_t>(end - base);
     groups.push_back(p);
+    first = last;
   }
   return static_cast<int>(groups.size());
 }

@@ -20,11 +20,21 @@ inline int batch_vx(int lattice, int32_t Lx, int vx_max, int precision) {
 BatchMember make_batch_member(int lattice, const int64_t dims[3], double tau, double rho_mean, uint64_t seed, uint32_t lattice_id,
                               int64_t off0, int64_t off1, uint64_t t0, int vx_max, int precision);
 
-// Groups of at most kParamMembers consecutive members with their
-// t-independent arguments, for the parameter-space launches (tile order 3);
-// tile0 of every member must be assigned.  Returns the number of groups.
-int batch_build_params(const BatchMember *members, int n, int64_t ntiles, int noise_mode, int noise_dist,
+// Groups of at most kParamMembers consecutive members of about equal sites
+// with their t-independent arguments, for the parameter-space launches (tile
+// order 3), at least `parts` of them where there are as many members; tile0 of
+// every member must be assigned.  Returns the number of groups.
+int batch_build_params(const BatchMember *members, int n, int64_t ntiles, int noise_mode, int noise_dist, int parts,
                        std::vector<BatchParams> &groups);
+
+// Parts of a set of members that step on streams of their own: while one's
+// launch ends, the other's blocks take the SMs.  Measured on GB300, GLUPS with
+// one part and two (three and four are no better): 60 D2Q9 members of 96..512
+// a side 78.5 and 83.0, 4 of 300..500 71.4 and 76.9, 40 of 60..100 57.8 and
+// 64.9, D3Q19 40 of 32..128 38.5 and 40.2, 8 of 30..60 32.0 and 37.1; but 20
+// D2Q9 members of 30..80 (51000 sites) 24.6 and 24.2.  The server keeps one
+// (24 mixed requests 59.5 and 59.0 ms: its types already overlap).
+inline int batch_parts(int64_t sites) { return sites >= (int64_t(1) << 17) ? 2 : 1; }
 
 // Tile passes for a launch of the members: at most `passes`, fewer where the
 // tiles would not fill the GPU's `slots` resident blocks four times (a last

@@ -152,7 +152,9 @@ static int ens_plan(lbfd_ens *e, int vx_max, int passes, int occ, int walk) {
   e->occ = occ;
   e->walk = walk;
   e->groups.clear();
-  if (walk == kWalkParam) batch_build_params(e->hmem.data(), e->n, e->ntiles, e->noise_mode, e->noise_dist, e->groups);
+  if (walk == kWalkParam)
+    batch_build_params(e->hmem.data(), e->n, e->ntiles, e->noise_mode, e->noise_dist, batch_parts(e->total_sites),
+                       e->groups);
   e->grid = int(std::max<int64_t>(1, std::min<int64_t>(e->ntiles, int64_t(sms) * e->bps)));
   if (e->graph) {
     cudaGraphExecDestroy(e->graph);

@@ -437,7 +437,7 @@ int upload_tables(lbfd_server *s) {
                            : s->opt.passes;
     s->seg_tiles[L] = batch_assign_tiles(hm + s->seg_off[L], s->seg_n[L], s->seg_passes[L], hts + s->seg_off[L]);
     if (s->opt.walk == LBFD_WALK_PARAM)
-      batch_build_params(hm + s->seg_off[L], s->seg_n[L], s->seg_tiles[L], s->opt.noise_mode, s->opt.noise_dist,
+      batch_build_params(hm + s->seg_off[L], s->seg_n[L], s->seg_tiles[L], s->opt.noise_mode, s->opt.noise_dist, 1,
                          s->groups[L]);
   }
   // (the parameter-space launches take everything from the groups)
