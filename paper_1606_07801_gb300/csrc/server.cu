@@ -515,6 +515,14 @@ int launch_params(lbfd_server *s, bool changed) {
     SRV_CU(mark(L, s->ls[L]));
   }
   const int nst = std::min<int>(lbfd_server::kSoloStreams, int(s->solo.size()));
+  if (changed && nst > 0) {
+    // a changed set may move a large simulation to another of these streams
+    // (they are dealt out in the order of the types): they wait for each other
+    for (int k = 0; k < lbfd_server::kSoloStreams; ++k) SRV_CU(cudaEventRecord(s->solo_ev[k], s->ss[k]));
+    for (int k = 0; k < nst; ++k)
+      for (int o = 0; o < lbfd_server::kSoloStreams; ++o)
+        if (o != k) SRV_CU(cudaStreamWaitEvent(s->ss[k], s->solo_ev[o], 0));
+  }
   for (int k = 0; k < nst; ++k) {
     if (changed) SRV_CU(cudaStreamWaitEvent(s->ss[k], s->fork_ev, 0));
     for (size_t m = size_t(k); m < s->solo.size(); m += size_t(nst)) {
