@@ -152,9 +152,10 @@ __host__ __device__ constexpr int batch_column() {
 // FP32 instructions with its noise parked in `column`, in FP64 and without
 // noise one site at a time.  Measured on GB300 in the parameter-space
 // launches, against one site at a time from registers with the arguments
-// prepared by a launch of its own: 60 D2Q9 members of 96..512 a side 62.8 ->
-// 80.0 GLUPS with even rows, 59.4 -> 73.3 odd; 40 D3Q19 members of 32..128 a
-// side 36.9 -> 42.1 even, 33.4 -> 36.0 odd.
+// prepared by a launch of its own (blocks of 256 threads, one launch a step; for
+// the present figures see kBatchThreads and batch_parts): 60 D2Q9 members of
+// 96..512 a side 62.8 -> 80.0 GLUPS with even rows, 59.4 -> 73.3 odd; 40 D3Q19
+// members of 32..128 a side 36.9 -> 42.1 even, 33.4 -> 36.0 odd.
 // ready() is called before an item's first load.
 template <int LAT, typename S, int NOISE, int VXMAX, class F>
 __device__ __forceinline__ void batch_tile_items(S *base, const BatchStep &b, int rel, int passes, float2 *column,
