@@ -921,92 +921,6 @@ struct NoiseTransform<kD2Q9, R> {
   }
 };
 
-// D3Q19: the rows split by their parities in the three axes (the seed
-// monomial's exponents modulo 2), so that on the four velocities of a plane
-// T(sa, sb) = S + sa sb X + sa A + sb B, S even in both axes, X the one row
-// v_a v_b, A odd in the first axis alone and B in the second; on an axis
-// T(+-) = S +- A.  The second-order rows 4, 7, 9 enter S through their sum
-// u, the odd rows of an axis share their first terms between the axis and its
-// two planes.  69 operations against 110 for the even and odd part of each
-// pair of velocities, on the pipe that bounds the D3Q19 kernels (the FMA
-// pipe that also takes Philox' multiplies, 77% busy); measured on GB300,
-// microseconds per step of 256^3: FP16 366.9 -> 351.7, FP32 405.1 -> 390.4.
-template <typename R>
-struct NoiseTransform<kD3Q19, R> {
-  static constexpr bool kWeighted = false;
-  static constexpr int L = kD3Q19;
-  // velocities: +x 1, +y 3, +z 5; (+x +y) 7, (+x -y) 9, (+x +z) 11, (+x -z) 13, (+y +z) 15, (+y -z) 17,
-  // each followed by its opposite
-  template <int A, int I>
-  static constexpr double m = kBasis<L, A, I>;
-  static constexpr bool near(double x, double y) { return x - y < 1e-12 && y - x < 1e-12; }
-  // the shape of the rows that apply() relies on (h: 4, 7, 9 are -h, 2h or -h + 3h by axis; o, p, q the odd rows)
-  static constexpr double h = -m<7, 1>, o = m<1, 1>, p = m<12, 1>, q = m<13, 1>;
-  static_assert(near(m<4, 1>, 2 * h) && near(m<9, 1>, -h) && near(m<4, 3>, -h) && near(m<7, 3>, 2 * h) &&
-                    near(m<9, 3>, -h) && near(m<4, 5>, -h) && near(m<7, 5>, -h) && near(m<9, 5>, 2 * h) &&
-                    near(m<4, 7>, 2 * h) && near(m<7, 7>, 2 * h) && near(m<9, 7>, -h) && near(m<4, 11>, 2 * h) &&
-                    near(m<7, 11>, -h) && near(m<9, 11>, 2 * h) && near(m<4, 15>, -h) && near(m<7, 15>, 2 * h) &&
-                    near(m<9, 15>, 2 * h) && near(m<7, 0>, m<4, 0>) && near(m<9, 0>, m<4, 0>),
-                "second-order rows");
-  static_assert(near(m<1, 7>, o) && near(m<1, 11>, o) && near(m<2, 3>, o) && near(m<2, 7>, o) && near(m<2, 15>, o) &&
-                    near(m<3, 5>, o) && near(m<3, 11>, o) && near(m<3, 15>, o),
-                "first-order rows");
-  static_assert(near(m<12, 7>, -2 * p) && near(m<12, 11>, p) && near(m<13, 11>, -q) && near(m<10, 3>, p) &&
-                    near(m<10, 7>, -2 * p) && near(m<10, 15>, p) && near(m<15, 3>, q) && near(m<15, 15>, -q) &&
-                    near(m<11, 5>, p) && near(m<11, 11>, -2 * p) && near(m<11, 15>, p) && near(m<14, 5>, q) &&
-                    near(m<14, 15>, -q) && m<13, 7> == 0.0 && m<15, 7> == 0.0 && m<14, 11> == 0.0,
-                "third-order rows");
-  static_assert(m<18, 1> == 0.0 && m<17, 7> == 0.0 && m<18, 7> == 0.0 && m<18, 11> == 0.0, "fourth-order rows");
-  // T on the plane of velocities I (+ +), I + 1 (- -), J (+ -), J + 1 (- +)
-  template <int X, int I, int J, typename V>
-  __host__ __device__ static __forceinline__ void plane(const V &S, const V &A, const V &B, const V &zx, V (&T)[19]) {
-    const V e = fma_rn(cst<V>(m<X, I>), zx, S), d = fma_rn(cst<V>(-m<X, I>), zx, S);
-    const V a = add_rn(A, B), b = sub_rn(A, B);
-    T[I] = add_rn(e, a);
-    T[I + 1] = sub_rn(e, a);
-    T[J] = add_rn(d, b);
-    T[J + 1] = sub_rn(d, b);
-  }
-  template <typename V>
-  __host__ __device__ static __forceinline__ void apply(const V (&zz)[18], V (&T)[19]) {
-    auto z = [&](int a) -> const V & { return zz[a - 1]; };
-    // odd rows of x (1, 12, 13), y (2, 10, 15) and z (3, 11, 14): on the axis, on its first plane and its second
-    auto odd = [](const V &z1, const V &z2, const V &z3, V &plane2, V &axis, V &plane3) {
-      const V first = mul_rn(cst<V>(o), z1), common = fma_rn(cst<V>(p), z2, first);
-      plane2 = fma_rn(cst<V>(-2 * p), z2, first);
-      axis = fma_rn(cst<V>(q), z3, common);
-      plane3 = fma_rn(cst<V>(-q), z3, common);
-    };
-    V x_xy, x_x, x_xz, y_xy, y_y, y_yz, z_xz, z_z, z_yz;
-    odd(z(1), z(12), z(13), x_xy, x_x, x_xz);
-    odd(z(2), z(10), z(15), y_xy, y_y, y_yz);
-    odd(z(3), z(11), z(14), z_xz, z_z, z_yz);
-    // even rows
-    const V u = mul_rn(cst<V>(-h), add_rn(add_rn(z(4), z(7)), z(9))), u2 = mul_rn(cst<V>(-2.0), u);
-    const V Sx = fma_rn(cst<V>(m<16, 1>), z(16), fma_rn(cst<V>(m<17, 1>), z(17), fma_rn(cst<V>(3 * h), z(4), u)));
-    const V Sy = fma_rn(cst<V>(m<16, 3>), z(16),
-                        fma_rn(cst<V>(m<17, 3>), z(17), fma_rn(cst<V>(m<18, 3>), z(18), fma_rn(cst<V>(3 * h), z(7), u))));
-    const V Sz = fma_rn(cst<V>(m<16, 5>), z(16),
-                        fma_rn(cst<V>(m<17, 5>), z(17), fma_rn(cst<V>(m<18, 5>), z(18), fma_rn(cst<V>(3 * h), z(9), u))));
-    const V Sxy = fma_rn(cst<V>(m<16, 7>), z(16), fma_rn(cst<V>(-3 * h), z(9), u2));
-    const V Sxz = fma_rn(cst<V>(m<16, 11>), z(16), fma_rn(cst<V>(m<17, 11>), z(17), fma_rn(cst<V>(-3 * h), z(7), u2)));
-    const V Syz = fma_rn(cst<V>(m<16, 15>), z(16),
-                         fma_rn(cst<V>(m<17, 15>), z(17), fma_rn(cst<V>(m<18, 15>), z(18), fma_rn(cst<V>(-3 * h), z(4), u2))));
-    // the rest population's T_0 (kernels that take it from mass conservation leave it out)
-    T[0] = mul_rn(cst<V>(m<4, 0>), add_rn(add_rn(z(4), z(7)), z(9)));
-    T[0] = fma_rn(cst<V>(m<16, 0>), z(16), fma_rn(cst<V>(m<17, 0>), z(17), fma_rn(cst<V>(m<18, 0>), z(18), T[0])));
-    T[1] = add_rn(Sx, x_x);
-    T[2] = sub_rn(Sx, x_x);
-    T[3] = add_rn(Sy, y_y);
-    T[4] = sub_rn(Sy, y_y);
-    T[5] = add_rn(Sz, z_z);
-    T[6] = sub_rn(Sz, z_z);
-    plane<5, 7, 9>(Sxy, x_xy, y_xy, z(5), T);
-    plane<6, 11, 13>(Sxz, x_xz, z_xz, z(6), T);
-    plane<8, 15, 17>(Syz, y_yz, z_yz, z(8), T);
-  }
-};
-
 // D1Q3: T(0) = -z^2/sqrt2, T(+-1) = +-sqrt3 z^1 + sqrt2 z^2.
 template <typename R>
 struct NoiseTransform<kD1Q3, R> {
