@@ -98,6 +98,7 @@ struct lbfd_sim {
   int *status_host = nullptr;
   int *status_dev = nullptr;
   bool staged_ok = false;  // the lattice and buffers meet the staged kernel's requirements
+  int vec_most = 4;        // values per vector access that the buffers' addresses allow
   bool alt_sweep = true;  // one-launch-per-step kernels sweep every other step in reverse (sweep_default)
   // the stored lattice: dims itself, or for a slab its n owned planes plus
   // a halo plane on each side along the slowest axis
@@ -273,7 +274,8 @@ static int step_path(const lbfd_sim *h, int64_t n) {
   if (h->mrt) return LBFD_KERNEL_MRT;
   if (o.step_kernel != LBFD_KERNEL_AUTO) return o.step_kernel;
   if (h->staged_ok && staged_default()) return LBFD_KERNEL_STAGED;
-  return step_vec_width(o.lattice, o.precision, int32_t(o.dims[0]), h->N) >= 2 ? LBFD_KERNEL_VEC : LBFD_KERNEL_SCALAR;
+  return step_vec_width(o.lattice, o.precision, int32_t(o.dims[0]), h->N, h->vec_most) >= 2 ? LBFD_KERNEL_VEC
+                                                                                            : LBFD_KERNEL_SCALAR;
 }
 
 static void free_sim(lbfd_sim *h) {
@@ -375,6 +377,7 @@ int lbfd_create_ex(lbfd_t *out, const lbfd_options *opt) {
   }
   h->alt_sweep = sweep_default();
   if (e == cudaSuccess) {
+    h->vec_most = vec_most(h->f[0], h->f[1], h->elem);
     h->staged_ok = !h->mrt && staged_fits(opt->lattice, opt->precision, opt->dims[0], h->NS, h->f[0], h->f[1]);
     if (h->slab && !h->staged_ok) {
       free_sim(h);
@@ -472,9 +475,10 @@ int lbfd_destroy(lbfd_t h) {
 static int sample_now(lbfd_sim *h) {
   const lbfd_options &o = h->opt;
   LBFD_CU(obs_join(h));
+  const int width = sample_width(o.lattice, o.precision, int32_t(o.dims[0]), h->vec_most);
   if ((o.lattice == LBFD_D1Q3 || o.lattice == LBFD_D2Q9) && !h->slab &&
       sample_fusable(o.lattice, o.precision, int32_t(o.dims[0]), int32_t(o.dims[1]), int32_t(o.dims[2]), o.n_modes,
-                     h->phase)) {
+                     h->phase, width)) {
     // FP32 arithmetic, register sampler: the fused step's sampler as a pass
     // of its own over the lattice's register-pull blocks, then stage 2
     StepArgs a{};
@@ -485,7 +489,7 @@ static int sample_now(lbfd_sim *h) {
     fill_step_params(a, o.tau, o.rho_mean);
     int nblocks = 0;
     LBFD_CU(launch_obs_sample(o.lattice, o.precision, h->f[h->cur], a, o.n_modes, h->phase, h->partials, &nblocks,
-                              h->stream));
+                              width, h->stream));
     LBFD_CU(launch_obs_pull_finalize(o.lattice, h->partials, nblocks, o.n_modes, h->N, o.rho_mean, h->fin, h->acc,
                                      h->stream));
     g_launches.fetch_add(2, std::memory_order_relaxed);
@@ -579,11 +583,12 @@ int lbfd_step(lbfd_t h, int64_t n) {
   const int kernel = step_path(h, 1);
   int vec_width = 1;
   if (kernel == LBFD_KERNEL_VEC) {
-    vec_width = step_vec_width(o.lattice, o.precision, a.Lx, h->N);
-    if (vec_width == 1) vec_width = 2;  // asked for by step_kernel: Lx is even
+    vec_width = step_vec_width(o.lattice, o.precision, a.Lx, h->N, h->vec_most);
+    if (vec_width == 1) vec_width = std::min(2, h->vec_most);  // asked for by step_kernel: Lx is even
   }
+  const int width = sample_width(o.lattice, o.precision, a.Lx, h->vec_most);
   const bool fusable = o.sample_every > 0 && !h->mrt && sample_fused_pays(o.lattice, h->N) &&
-                       sample_fusable(o.lattice, o.precision, a.Lx, a.Ly, a.Lz, o.n_modes, h->phase);
+                       sample_fusable(o.lattice, o.precision, a.Lx, a.Ly, a.Lz, o.n_modes, h->phase, width);
   int64_t extra = 0;  // launches besides one step kernel per step
   for (int64_t k = 0; k < n; ++k) {
     a.ph = make_philox_step(o.seed, o.lattice_id, uint64_t(h->t));
@@ -598,7 +603,7 @@ int lbfd_step(lbfd_t h, int64_t n) {
         int nblocks = 0;
         if (e == cudaSuccess)
           e = launch_step_sample(o.lattice, o.precision, src, dst, a, o.n_modes, h->phase, h->partials, &nblocks,
-                                 h->staged_ok, h->status_dev, h->stream);
+                                 h->staged_ok, h->status_dev, width, h->stream);
         if (e == cudaSuccess && !h->obs_stream) {
           e = cudaStreamCreateWithFlags(&h->obs_stream, cudaStreamNonBlocking);
           if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_sampled, cudaEventDisableTiming);

@@ -330,17 +330,22 @@ cudaError_t launch_obs_pull_finalize(int lattice, const double *partials, int nb
 // per-axis structure-factor tables (obs_phase_fill); n_modes <=
 // kFusedModes.
 constexpr int kFusedModes = 4;
+// Sites per thread of the sampling kernels (1 or 2), for buffers that allow
+// vectors of `most` values (vec_most).
+inline int sample_width(int lattice, int precision, int32_t Lx, int most) {
+  return step_vec_width(lattice, precision, Lx, INT64_MAX, most) >= 2 ? 2 : 1;
+}
 // Whether a lattice can take the fused step-and-sample kernel: FP32
 // arithmetic, fewer than 2^31 sites, at most kFusedModes modes with their
 // phase tables, and a work block of 256 threads with whole warps along x
-// (the one-launch-per-step kernel's shape).
+// (the one-launch-per-step kernel's shape) at vx sites per thread (sample_width).
 inline bool sample_fusable(int lattice, int precision, int32_t Lx, int32_t Ly, int32_t Lz, int n_modes,
-                           const void *phase) {
+                           const void *phase, int vx) {
   if (lattice != kD1Q3 && lattice != kD2Q9 && lattice != kD3Q19) return false;
   if (precision == kStoreF64 || n_modes > kFusedModes || (n_modes > 0 && !phase)) return false;
   if (int64_t(Lx) * Ly * Lz >= (int64_t(1) << 31)) return false;
   dim3 grid, block;
-  step_shape(Lx, Ly, Lz, grid, block, step_vec_width(lattice, precision, Lx) >= 2 ? 2 : 1);
+  step_shape(Lx, Ly, Lz, grid, block, vx);
   return block.x * block.y == 256 && block.x % 32 == 0;
 }
 // LBFD_SAMPLE_STAGED = 1: D3Q19 samples in the staged kernel (step_sample_t).
@@ -364,27 +369,27 @@ inline bool sample_fused_pays(int lattice, int64_t N) {
 }
 cudaError_t launch_step_sample_d1q3(int precision, const void *src, void *dst, const StepArgs &a, int n_modes,
                                     const void *phase, double *partials, int *nblocks, bool staged_ok,
-                                    int *status, cudaStream_t stream);
+                                    int *status, int vx, cudaStream_t stream);
 cudaError_t launch_step_sample_d2q9(int precision, const void *src, void *dst, const StepArgs &a, int n_modes,
                                     const void *phase, double *partials, int *nblocks, bool staged_ok,
-                                    int *status, cudaStream_t stream);
+                                    int *status, int vx, cudaStream_t stream);
 cudaError_t launch_step_sample_d3q19(int precision, const void *src, void *dst, const StepArgs &a, int n_modes,
                                      const void *phase, double *partials, int *nblocks, bool staged_ok,
-                                     int *status, cudaStream_t stream);
+                                     int *status, int vx, cudaStream_t stream);
 // staged_ok: the lattice and buffers meet the staged kernel's requirements
-// (staged_fits); status: its bounded waits' status word.
+// (staged_fits); status: its bounded waits' status word; vx: sample_width.
 inline cudaError_t launch_step_sample(int lattice, int precision, const void *src, void *dst, const StepArgs &a,
                                       int n_modes, const void *phase, double *partials, int *nblocks, bool staged_ok,
-                                      int *status, cudaStream_t stream) {
+                                      int *status, int vx, cudaStream_t stream) {
   switch (lattice) {
     case kD1Q3:
-      return launch_step_sample_d1q3(precision, src, dst, a, n_modes, phase, partials, nblocks, staged_ok, status,
+      return launch_step_sample_d1q3(precision, src, dst, a, n_modes, phase, partials, nblocks, staged_ok, status, vx,
                                      stream);
     case kD2Q9:
-      return launch_step_sample_d2q9(precision, src, dst, a, n_modes, phase, partials, nblocks, staged_ok, status,
+      return launch_step_sample_d2q9(precision, src, dst, a, n_modes, phase, partials, nblocks, staged_ok, status, vx,
                                      stream);
     case kD3Q19:
-      return launch_step_sample_d3q19(precision, src, dst, a, n_modes, phase, partials, nblocks, staged_ok, status,
+      return launch_step_sample_d3q19(precision, src, dst, a, n_modes, phase, partials, nblocks, staged_ok, status, vx,
                                       stream);
   }
   return cudaErrorInvalidValue;
@@ -394,15 +399,15 @@ inline cudaError_t launch_step_sample(int lattice, int precision, const void *sr
 // lattices (D1Q3, D2Q9; FP32 arithmetic; the shape sample_fusable accepts):
 // the sampler of the fused step as the separate sampling pass, in the
 // partials layout of k_obs_pull (then launch_obs_pull_finalize).
-// cudaErrorInvalidValue for other lattices.
+// cudaErrorInvalidValue for other lattices.  vx: sample_width.
 cudaError_t launch_obs_sample_d1q3(int precision, const void *src, const StepArgs &a, int n_modes,
-                                   const void *phase, double *partials, int *nblocks, cudaStream_t stream);
+                                   const void *phase, double *partials, int *nblocks, int vx, cudaStream_t stream);
 cudaError_t launch_obs_sample_d2q9(int precision, const void *src, const StepArgs &a, int n_modes,
-                                   const void *phase, double *partials, int *nblocks, cudaStream_t stream);
+                                   const void *phase, double *partials, int *nblocks, int vx, cudaStream_t stream);
 inline cudaError_t launch_obs_sample(int lattice, int precision, const void *src, const StepArgs &a, int n_modes,
-                                     const void *phase, double *partials, int *nblocks, cudaStream_t stream) {
-  if (lattice == kD1Q3) return launch_obs_sample_d1q3(precision, src, a, n_modes, phase, partials, nblocks, stream);
-  if (lattice == kD2Q9) return launch_obs_sample_d2q9(precision, src, a, n_modes, phase, partials, nblocks, stream);
+                                     const void *phase, double *partials, int *nblocks, int vx, cudaStream_t stream) {
+  if (lattice == kD1Q3) return launch_obs_sample_d1q3(precision, src, a, n_modes, phase, partials, nblocks, vx, stream);
+  if (lattice == kD2Q9) return launch_obs_sample_d2q9(precision, src, a, n_modes, phase, partials, nblocks, vx, stream);
   return cudaErrorInvalidValue;
 }
 

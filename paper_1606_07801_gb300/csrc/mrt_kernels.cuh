@@ -244,7 +244,7 @@ cudaError_t step_mrt_t(const void *src, void *dst, const StepArgs &a, const doub
   return mrt_collide_t<LAT, S>(a, m, w, tau, [&](auto c) -> cudaError_t {
     using C = decltype(c);
     constexpr int NOISE = C::kNoise;
-    const int vx = step_vec_width(LAT, precision, a.Lx, a.N);
+    const int vx = step_vec_width(LAT, precision, a.Lx, a.N, vec_most(src, dst, sizeof(S)));
     dim3 grid, block;
     step_shape(a.Lx, a.Ly, a.Lz, grid, block, vx, std::min(step_threads(LAT, precision), 128));
     StepLaunch launch(grid, block, stream);

@@ -6,18 +6,18 @@ namespace lbfd {
 
 cudaError_t launch_step_sample_d1q3(int precision, const void *src, void *dst, const StepArgs &a, int n_modes,
                                    const void *phase, double *partials, int *nblocks, bool staged_ok,
-                                   int *status, cudaStream_t stream) {
+                                   int *status, int vx, cudaStream_t stream) {
   return dispatch_storage(precision, [&](auto tag) {
     using S = typename decltype(tag)::type;
-    return step_sample_t<kD1Q3, S>(src, dst, a, n_modes, phase, partials, nblocks, staged_ok, status, stream);
+    return step_sample_t<kD1Q3, S>(src, dst, a, n_modes, phase, partials, nblocks, staged_ok, status, vx, stream);
   });
 }
 
 cudaError_t launch_obs_sample_d1q3(int precision, const void *src, const StepArgs &a, int n_modes,
-                                   const void *phase, double *partials, int *nblocks, cudaStream_t stream) {
+                                   const void *phase, double *partials, int *nblocks, int vx, cudaStream_t stream) {
   return dispatch_storage(precision, [&](auto tag) {
     using S = typename decltype(tag)::type;
-    return obs_sample_t<kD1Q3, S>(src, a, n_modes, phase, partials, nblocks, stream);
+    return obs_sample_t<kD1Q3, S>(src, a, n_modes, phase, partials, nblocks, vx, stream);
   });
 }
 

@@ -687,8 +687,7 @@ inline SampleArgs make_sample_args(const StepArgs &a, int n_modes, const void *p
 // The fused step-and-sample launch on the register-pull kernel's blocks.
 template <int LAT, typename S>
 cudaError_t sample_vec_t(const void *src, void *dst, const StepArgs &a, int n_modes, const void *phase,
-                         double *partials, int *nblocks, cudaStream_t stream) {
-  const int vx = step_vec_width(LAT, Store<S>::kDeviation ? kStoreF16 : kStoreF32, a.Lx) >= 2 ? 2 : 1;
+                         double *partials, int *nblocks, int vx, cudaStream_t stream) {
   dim3 grid, block;
   step_shape(a.Lx, a.Ly, a.Lz, grid, block, vx);
   if (block.x * block.y != kSampleThreads || block.x % 32 != 0) return cudaErrorInvalidValue;
@@ -711,12 +710,11 @@ cudaError_t sample_vec_t(const void *src, void *dst, const StepArgs &a, int n_mo
 // D2Q9, FP32 arithmetic, the shape sample_fusable accepts).
 template <int LAT, typename S>
 cudaError_t obs_sample_t(const void *src, const StepArgs &a, int n_modes, const void *phase, double *partials,
-                         int *nblocks, cudaStream_t stream) {
+                         int *nblocks, int vx, cudaStream_t stream) {
   if constexpr (sizeof(typename Store<S>::R) != 4 || Lattice<LAT>::Q > 9) {
     return cudaErrorInvalidValue;
   } else {
     if (n_modes < 0 || n_modes > kFusedModes || (n_modes > 0 && !phase)) return cudaErrorInvalidValue;
-    const int vx = step_vec_width(LAT, Store<S>::kDeviation ? kStoreF16 : kStoreF32, a.Lx) >= 2 ? 2 : 1;
     dim3 grid, block;
     step_shape(a.Lx, a.Ly, a.Lz, grid, block, vx);
     if (block.x * block.y != kSampleThreads || block.x % 32 != 0) return cudaErrorInvalidValue;

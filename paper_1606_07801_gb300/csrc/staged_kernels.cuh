@@ -463,12 +463,12 @@ cudaError_t staged_t(const void *src, void *dst, const StepArgs &a, const Staged
 // results agree within FP32 rounding of the sums, and the state bit for bit).
 template <int LAT, typename S>
 cudaError_t step_sample_t(const void *src, void *dst, const StepArgs &a, int n_modes, const void *phase,
-                          double *partials, int *nblocks, bool staged_ok, int *status, cudaStream_t stream) {
+                          double *partials, int *nblocks, bool staged_ok, int *status, int vx, cudaStream_t stream) {
   if constexpr (sizeof(typename Store<S>::R) != 4) {
     return cudaErrorInvalidValue;  // FP64 storage samples in FP64 by its own pass
   } else if constexpr (Lattice<LAT>::Q <= 9) {
     if (n_modes < 0 || n_modes > kFusedModes || (n_modes > 0 && !phase)) return cudaErrorInvalidValue;
-    return sample_vec_t<LAT, S>(src, dst, a, n_modes, phase, partials, nblocks, stream);
+    return sample_vec_t<LAT, S>(src, dst, a, n_modes, phase, partials, nblocks, vx, stream);
   } else {
     if (n_modes < 0 || n_modes > kFusedModes || (n_modes > 0 && !phase)) return cudaErrorInvalidValue;
     using SH = StagedShape<LAT, S>;
@@ -476,7 +476,7 @@ cudaError_t step_sample_t(const void *src, void *dst, const StepArgs &a, int n_m
     constexpr bool fits = kStagedSampleMinBlocks * (SH::kSmemBytes + SH::kConsumerWarps * sizeof(typename WS::Smem) +
                                                     1024) <= 228 * 1024;
     if (!(fits && staged_ok && sample_staged_default()))
-      return sample_vec_t<LAT, S>(src, dst, a, n_modes, phase, partials, nblocks, stream);
+      return sample_vec_t<LAT, S>(src, dst, a, n_modes, phase, partials, nblocks, vx, stream);
     const SampleArgs sa = make_sample_args<LAT>(a, n_modes, phase, dim3(1, 1, 1));
     const StagedRows rows{0, static_cast<uint32_t>(a.Ly) * static_cast<uint32_t>(a.Lz), 0};
     if (a.noise_mode == kNoiseOff)

@@ -10,6 +10,16 @@
 
 namespace lbfd {
 
+// Values per vector access at most (4, 2 or 1) that the addresses of a
+// lattice's two buffers allow: a vector lies on a multiple of its size, and
+// with Lx a multiple of the vector every row and population starts as the
+// buffer does.
+inline int vec_most(const void *a, const void *b, int value_bytes) {
+  const uintptr_t at = reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b);
+  const uintptr_t bytes = static_cast<uintptr_t>(value_bytes);
+  return at % (4 * bytes) == 0 ? 4 : (at % (2 * bytes) == 0 ? 2 : 1);
+}
+
 // Sites per thread of the register-pull step kernel (k_step_vec; 1 is
 // k_step), where Lx allows: several share the address and load instructions,
 // but are updated one after the other, which a lattice of few warps per SM
@@ -28,8 +38,9 @@ namespace lbfd {
 //   1 in FP64, whose narrow pipe hides the extra instructions: D2Q9 512 x 384
 //     47.0 against 50.3 with two, 60 x 50 6.1 against 10.3.
 // A tuning knob only; results do not depend on it.  LBFD_STEP_VX = 1, 2 or 4
-// overrides the choice where Lx allows.
-inline int step_vec_width(int lattice, int precision, int32_t Lx, int64_t sites = INT64_MAX) {
+// overrides the choice where Lx allows.  At most `most` sites (vec_most of the
+// buffers).
+inline int step_vec_width(int lattice, int precision, int32_t Lx, int64_t sites = INT64_MAX, int most = 4) {
   static int forced = [] {
     const char *e = getenv("LBFD_STEP_VX");
     const int r = e ? atoi(e) : 0;
@@ -42,8 +53,8 @@ inline int step_vec_width(int lattice, int precision, int32_t Lx, int64_t sites 
     vx = precision == kStoreF64 || sites <= few ? 1 : (lattice == kD2Q5 || (four && sites >= (1 << 19)) ? 4 : 2);
   }
   if (vx == 4 && precision == kStoreF64) vx = 2;
-  if (Lx % vx == 0) return vx;
-  return Lx % 2 == 0 ? 2 : 1;
+  while (vx > most || Lx % vx != 0) vx /= 2;
+  return vx;
 }
 
 // Threads of a block of the one-launch-per-step kernels.  FP64: one warp, so
