@@ -130,11 +130,11 @@ __host__ __device__ __forceinline__ V cst(double c) {
   return splat<V>(static_cast<typename LaneOf<V>::type>(c));
 }
 // On the device these are the PTX instructions add/sub/mul/fma.rn.f32x2 in
-// inline assembly: an explicit rounding modifier keeps the assembler from
-// fusing a multiply into a following add, and the compiler cannot see into
-// the assembly to fuse them earlier, so a packed product added to something
-// rounds twice, as __fmul_rn and __fadd_rn do.  (Before sm_100, and on the
-// host, two scalar operations.)
+// inline assembly.  A packed product that feeds a packed add or subtraction
+// may still be fused with it (seen on GB300 in the moment-space update, where
+// the results were those of one rounding; the scalar __fmul_rn and __fadd_rn
+// never are), so such sums take add_apart / sub_apart: two scalar operations.
+// (Before sm_100, and on the host, all of these are.)
 #if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
 #define LBFD_F32X2 1
 __device__ __forceinline__ uint64_t f32x2_bits(float2 a) {
@@ -183,6 +183,22 @@ __host__ __device__ __forceinline__ float2 fma_rn(float2 a, float2 b, float2 c) 
 #else
   return make_float2(fma_rn(a.x, b.x, c.x), fma_rn(a.y, b.y, c.y));
 #endif
+}
+// a + b and a - b where an operand is a product: rounded on its own in both
+// forms.
+template <typename V>
+__host__ __device__ __forceinline__ V add_apart(const V &a, const V &b) {
+  if constexpr (LaneOf<V>::kLanes == 2)
+    return make_float2(add_rn(a.x, b.x), add_rn(a.y, b.y));
+  else
+    return add_rn(a, b);
+}
+template <typename V>
+__host__ __device__ __forceinline__ V sub_apart(const V &a, const V &b) {
+  if constexpr (LaneOf<V>::kLanes == 2)
+    return make_float2(sub_rn(a.x, b.x), sub_rn(a.y, b.y));
+  else
+    return sub_rn(a, b);
 }
 // x where x > 0, else +0 (also for NaN), lane by lane.
 template <typename V>

@@ -72,25 +72,29 @@ __device__ __forceinline__ void mrt_forward(const V (&f)[Lattice<LAT>::Q], V (&M
       M[a - 1] = acc;
     });
   } else {
-    // one axis of the product basis: (f_0, f_+, f_-) to (mu^0, mu^1, mu^2)
-    auto axis = [](const V &f0, const V &fp, const V &fm, V &m0, V &m1, V &m2) {
-      const V s = add_rn(fp, fm);
-      m0 = add_rn(f0, s);
-      m1 = mul_rn(cst<V>(kSqrt3), sub_rn(fp, fm));
+    // one axis of the product basis: (f_0, f_+, f_-) to (mu^0, mu^1, mu^2);
+    // products: the inputs are products
+    auto axis = [](auto products, const V &f0, const V &fp, const V &fm, V &m0, V &m1, V &m2) {
+      constexpr bool apart = decltype(products)::value;
+      const V s = apart ? add_apart(fp, fm) : add_rn(fp, fm);
+      m0 = apart ? add_apart(f0, s) : add_rn(f0, s);
+      m1 = mul_rn(cst<V>(kSqrt3), apart ? sub_apart(fp, fm) : sub_rn(fp, fm));
       m2 = fma_rn(cst<V>(kSqrt2), s, mul_rn(cst<V>(-kInvSqrt2), f0));
     };
+    constexpr std::false_type sums{};
+    constexpr std::true_type products{};
     if constexpr (LAT == kD1Q3) {
       V m0;
-      axis(f[0], f[1], f[2], m0, M[0], M[1]);
+      axis(sums, f[0], f[1], f[2], m0, M[0], M[1]);
     } else {
       V G[3][3];  // [cx][q]
-      axis(f[0], f[2], f[4], G[0][0], G[0][1], G[0][2]);
-      axis(f[1], f[5], f[8], G[1][0], G[1][1], G[1][2]);
-      axis(f[3], f[6], f[7], G[2][0], G[2][1], G[2][2]);
+      axis(sums, f[0], f[2], f[4], G[0][0], G[0][1], G[0][2]);
+      axis(sums, f[1], f[5], f[8], G[1][0], G[1][1], G[1][2]);
+      axis(sums, f[3], f[6], f[7], G[2][0], G[2][1], G[2][2]);
       V m00;
-      axis(G[0][0], G[1][0], G[2][0], m00, M[2], M[5]);
-      axis(G[0][1], G[1][1], G[2][1], M[0], M[3], M[6]);
-      axis(G[0][2], G[1][2], G[2][2], M[1], M[4], M[7]);
+      axis(sums, G[0][0], G[1][0], G[2][0], m00, M[2], M[5]);
+      axis(products, G[0][1], G[1][1], G[2][1], M[0], M[3], M[6]);
+      axis(sums, G[0][2], G[1][2], G[2][2], M[1], M[4], M[7]);
     }
   }
 }
@@ -121,15 +125,16 @@ __device__ __forceinline__ void mrt_given(V (&f)[Lattice<LAT>::Q], const ZF &z, 
     });
   }
   // back transform; the rest population from mass conservation
+  constexpr bool kProducts = LAT != kD3Q19;  // x is one
   V moved = splat<V>(R(0));
   auto keep = [&](int i, const V &x) {
     f[i] = x;
-    moved = i == 1 ? x : add_rn(moved, x);
+    moved = i == 1 ? x : (kProducts ? add_apart(moved, x) : add_rn(moved, x));
   };
   if constexpr (LAT == kD2Q5) {
     const V w = splat<V>(p.w);
     const V q = fma_rn(splat<V>(p.m41), M[3], rho), d = mul_rn(splat<V>(p.m3), M[2]);
-    const V ex = add_rn(q, d), ey = sub_rn(q, d);
+    const V ex = add_apart(q, d), ey = sub_apart(q, d);
     keep(1, mul_rn(w, fma_rn(splat<V>(p.m1), M[0], ex)));
     keep(2, mul_rn(w, fma_rn(splat<V>(-p.m1), M[0], ex)));
     keep(3, mul_rn(w, fma_rn(splat<V>(p.m2), M[1], ey)));
