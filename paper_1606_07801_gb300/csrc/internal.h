@@ -297,19 +297,22 @@ __device__ __forceinline__ void obs_delta_sums(Sum sum, Pair pair, double *out, 
 // deviation sums in the layout of the FP32 observable pass ([sum delta,
 // sum delta^2, sum e_i (Q), (re, im) of the K modes, pairs i <= j
 // row-major]), with cs[i] = c_i, C = sum_i c_i and Nd sites: rho = C +
-// delta and f_i = c_i + e_i expanded, in FP64.
+// delta and f_i = c_i + e_i expanded, in FP64.  Without offsets (C = 0: FP64
+// storage) the totals are the sums themselves, infinite ones too (a zero
+// offset times an infinite sum would be NaN).
 template <int Q>
 __host__ __device__ __forceinline__ double obs_restore(int k, const double *tt, const double *cs, double C, double Nd,
                                                        int K) {
   const int nq1 = 2 + Q + 2 * K;
+  const bool bare = C == 0.0;
   if (k == 0) return tt[0] + Nd * C;
-  if (k == 1) return tt[1] + 2.0 * C * tt[0] + Nd * C * C;
+  if (k == 1) return bare ? tt[1] : tt[1] + 2.0 * C * tt[0] + Nd * C * C;
   if (k < 2 + Q) return tt[k] + Nd * cs[k - 2];
   if (k < 2 + Q + Q * Q) {
     const int r = k - 2 - Q, a = r / Q, b = r - a * Q;
     const int i = a < b ? a : b, j = a < b ? b : a;
     const int p = i * Q - i * (i - 1) / 2 + (j - i);
-    return tt[nq1 + p] + cs[j] * tt[2 + i] + cs[i] * tt[2 + j] + Nd * cs[i] * cs[j];
+    return bare ? tt[nq1 + p] : tt[nq1 + p] + cs[j] * tt[2 + i] + cs[i] * tt[2 + j] + Nd * cs[i] * cs[j];
   }
   const int m = k - 2 - Q - Q * Q;
   const double re = tt[2 + Q + 2 * m], im = tt[3 + Q + 2 * m];
