@@ -416,11 +416,12 @@ int lbfd_ensemble_sync(lbfd_ens_t e);
 
 /* Times the candidate work decompositions (at most 1 or 2 sites per item,
  * times tiles of 1, 2, 4 or 8 passes, times two register/occupancy variants
- * of the kernel, times the four tile orders LBFD_WALK_*) over `steps`
- * launches each that write only the spare buffers, keeps the fastest and
- * reports it: sites per item at most, passes, resident blocks per SM (any
- * output may be NULL; lbfd_ensemble_query also gives the tile order).  The
- * state and t are unchanged.  Synchronous. */
+ * of the kernel, times the four tile orders LBFD_WALK_*) over `steps` steps
+ * each (rounded up to chunks of 16 up to 2^20 sites), launched as
+ * lbfd_ensemble_step launches them but writing only the spare buffers, keeps
+ * the fastest and reports it: sites per item at most, passes, resident blocks
+ * per SM (any output may be NULL; lbfd_ensemble_query also gives the tile
+ * order).  The state and t are unchanged.  Synchronous. */
 int lbfd_ensemble_tune(lbfd_ens_t e, int32_t steps, int32_t *vx_chosen, int32_t *passes_chosen,
                        int32_t *blocks_per_sm);
 

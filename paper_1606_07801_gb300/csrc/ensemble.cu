@@ -90,26 +90,21 @@ struct lbfd_ens {
   }
 };
 
-// Kernel launches of one step of the batched kernel.
-static int ens_step_launches(const lbfd_ens *e) {
-  return e->walk == kWalkParam ? static_cast<int>(e->groups.size()) : 1;
-}
-
 // `steps` steps of the parameter-space launches from the device clock on
 // (which stays).  The groups are independent of each other, so each runs all
 // of its steps on one side stream, as dependent launches, and the streams
 // fork from the ensemble's and join it once: no launch of a step waits for
 // another group's, nor for a launch that prepares it.  Measured on GB300, 60
 // D2Q9 members of 96..512 a side, 2000 steps: 126 -> 96 ms, with the items of
-// batch_tile_items.
-static cudaError_t ens_param_steps(lbfd_ens *e, int steps) {
+// batch_tile_items.  still: every step is the first one (see ens_steps).
+static cudaError_t ens_param_steps(lbfd_ens *e, int steps, bool still) {
   const int G = static_cast<int>(e->groups.size());
   const int nside = std::min(G, int(lbfd_ens::kSide));
   auto chain = [&](int g, cudaStream_t st) {
     cudaError_t err = cudaSuccess;
     for (int k = 0; k < steps && err == cudaSuccess; ++k)
       err = launch_batch_param(e->lattice, e->precision, e->buf, &e->groups[g], 1,
-                               BatchWhen{e->t_dev, uint64_t(k), k > 0}, e->tile_passes, e->occ, e->kvx, e->noise_mode,
+                               BatchWhen{e->t_dev, still ? 0 : uint64_t(k), k > 0}, e->tile_passes, e->occ, e->kvx, e->noise_mode,
                                e->noise_dist, st);
     return err;
   };
@@ -122,12 +117,6 @@ static cudaError_t ens_param_steps(lbfd_ens *e, int steps) {
     if (err == cudaSuccess) err = cudaStreamWaitEvent(e->stream, e->join_ev[k], 0);
   }
   return err;
-}
-
-static cudaError_t ens_launch(lbfd_ens *e) {
-  if (e->walk == kWalkParam) return ens_param_steps(e, 1);
-  return launch_batch_step(e->lattice, e->precision, e->buf, e->dsteps, e->dtile_start, e->n, e->ntiles,
-                           e->tile_passes, e->occ, e->walk, e->kvx, e->noise_mode, e->noise_dist, e->grid, e->stream);
 }
 
 // Work decomposition (sites per item, tile passes, occupancy variant, tile
@@ -194,30 +183,39 @@ static cudaError_t ens_sync_t(lbfd_ens *e) {
   return err;
 }
 
-// `steps` steps of every member, and t += steps on the device.
-static cudaError_t ens_steps(lbfd_ens *e, int steps) {
+// `steps` steps of every member, and t += steps on the device.  still: the
+// same launches with the clock held, so that every step reads the stored state
+// and writes the spare block (what the tuner times).
+static cudaError_t ens_steps(lbfd_ens *e, int steps, bool still) {
   cudaError_t err = cudaSuccess;
   if (e->walk == kWalkParam) {
-    err = ens_param_steps(e, steps);
-    if (err == cudaSuccess) err = launch_clock_advance(e->t_dev, e->stream, uint64_t(steps));
+    err = ens_param_steps(e, steps, still);
+    if (err == cudaSuccess) err = launch_clock_advance(e->t_dev, e->stream, still ? 0 : uint64_t(steps));
     return err;
   }
   for (int k = 0; k < steps && err == cudaSuccess; ++k) {
     err = launch_batch_prep(e->dmem, e->n, e->t_dev, 0, e->noise_mode, e->noise_dist, e->dsteps, e->stream);
-    if (err == cudaSuccess) err = ens_launch(e);
-    if (err == cudaSuccess) err = launch_clock_advance(e->t_dev, e->stream, 1);
+    if (err == cudaSuccess)
+      err = launch_batch_step(e->lattice, e->precision, e->buf, e->dsteps, e->dtile_start, e->n, e->ntiles,
+                              e->tile_passes, e->occ, e->walk, e->kvx, e->noise_mode, e->noise_dist, e->grid, e->stream);
+    if (err == cudaSuccess) err = launch_clock_advance(e->t_dev, e->stream, still ? 0 : 1);
   }
   return err;
 }
 
-static cudaError_t ens_build_graph(lbfd_ens *e) {
+// Kernel launches of ens_steps.
+static int64_t ens_launches(const lbfd_ens *e, int64_t steps) {
+  return e->walk == kWalkParam ? steps * int64_t(e->groups.size()) + 1 : steps * 3;
+}
+
+static cudaError_t ens_capture(lbfd_ens *e, int steps, bool still, cudaGraphExec_t *exec) {
   cudaGraph_t g = nullptr;
   cudaError_t err = cudaStreamBeginCapture(e->stream, cudaStreamCaptureModeThreadLocal);
   if (err != cudaSuccess) return err;
-  err = ens_steps(e, kGraphSteps);
+  err = ens_steps(e, steps, still);
   cudaError_t end = cudaStreamEndCapture(e->stream, &g);
   if (err == cudaSuccess) err = end;
-  if (err == cudaSuccess) err = cudaGraphInstantiate(&e->graph, g, 0);
+  if (err == cudaSuccess) err = cudaGraphInstantiate(exec, g, 0);
   if (g) cudaGraphDestroy(g);
   return err;
 }
@@ -353,17 +351,17 @@ int lbfd_ensemble_step(lbfd_ens_t e, int64_t n) {
     // the kernels take the parity of each member's block from t on the
     // device, so a captured chunk can start at any t
     if (n - done >= kGraphSteps) {
-      if (!e->graph) ENS_CU(ens_build_graph(e));
+      if (!e->graph) ENS_CU(ens_capture(e, kGraphSteps, false, &e->graph));
       ENS_CU(cudaGraphLaunch(e->graph, e->stream));
+      count_launches(ens_launches(e, kGraphSteps));
       done += kGraphSteps;
     } else {
       const int rest = static_cast<int>(n - done);
-      ENS_CU(ens_steps(e, rest));
+      ENS_CU(ens_steps(e, rest, false));
+      count_launches(ens_launches(e, rest));
       done += rest;
     }
   }
-  const int64_t chunks = (n + kGraphSteps - 1) / kGraphSteps;
-  count_launches(e->walk == kWalkParam ? n * ens_step_launches(e) + chunks : n * (2 + ens_step_launches(e)));
   e->t += n;
   return LBFD_OK;
 }
@@ -381,7 +379,7 @@ int lbfd_ensemble_tune(lbfd_ens_t e, int32_t steps, int32_t *vx_chosen, int32_t 
   if (!e || steps < 1) return ens_fail(LBFD_EINVAL, "lbfd_ensemble_tune: bad argument");
   DevGuard g(e->device);
   ENS_CU(ens_sync_t(e));
-  // candidates: sites per item (1, or 2 where Lx is even) x tile passes x
+  // candidates: sites per item (1, or 2: batch_vx) x tile passes x
   // occupancy variant of the kernel x tile order
   const int vx_cand[2] = {1, 2};
   const int pass_cand[4] = {1, 2, 4, 8};
@@ -394,8 +392,10 @@ int lbfd_ensemble_tune(lbfd_ens_t e, int32_t steps, int32_t *vx_chosen, int32_t 
     lbfd_ens *e;
     int vx, passes, occ, walk;
     cudaEvent_t a = nullptr, b = nullptr;
+    cudaGraphExec_t exec = nullptr;
     bool finished = false;
     ~TuneGuard() {
+      if (exec) cudaGraphExecDestroy(exec);
       if (a) cudaEventDestroy(a);
       if (b) cudaEventDestroy(b);
       if (!finished) {
@@ -409,7 +409,14 @@ int lbfd_ensemble_tune(lbfd_ens_t e, int32_t steps, int32_t *vx_chosen, int32_t 
   ENS_CU(cudaEventCreate(&guard.a));
   ENS_CU(cudaEventCreate(&guard.b));
   cudaEvent_t a = guard.a, b = guard.b;
-  // timing launches read the state and write the spare block only (t is not advanced)
+  // timed as lbfd_ensemble_step runs: a captured chunk of dependent or prepared
+  // steps with their clock kernels, which reads the state and writes the spare
+  // block only (t is not advanced).  Timed one step at a time, with a fork and a
+  // join for the parameter-space launches and without the other orders' small
+  // kernels, small ensembles got an order that runs at a third of the speed (20
+  // D2Q9 members of 30..80 a side: 8.1 of 24.6 GLUPS on GB300).
+  const int chunk = e->total_sites <= (int64_t(1) << 20) ? kGraphSteps : std::min(steps, kGraphSteps);
+  const int chunks = (steps + chunk - 1) / chunk;
   int64_t launched = 0;
   for (int walk = 0; walk < 4; ++walk) {
     for (int occ = 0; occ < 2; ++occ) {
@@ -417,15 +424,22 @@ int lbfd_ensemble_tune(lbfd_ens_t e, int32_t steps, int32_t *vx_chosen, int32_t 
         for (int passes : pass_cand) {
           int rc = ens_plan(e, vx, passes, occ, walk);
           if (rc) return rc;
-          ENS_CU(launch_batch_prep(e->dmem, e->n, e->t_dev, 0, e->noise_mode, e->noise_dist, e->dsteps, e->stream));
-          ENS_CU(ens_launch(e));
-          ENS_CU(cudaEventRecord(a, e->stream));
-          for (int k = 0; k < steps; ++k) ENS_CU(ens_launch(e));
-          ENS_CU(cudaEventRecord(b, e->stream));
-          ENS_CU(cudaEventSynchronize(b));
-          launched += 1 + int64_t(1 + steps) * ens_step_launches(e);
+          if (guard.exec) cudaGraphExecDestroy(guard.exec);
+          guard.exec = nullptr;
+          ENS_CU(ens_capture(e, chunk, true, &guard.exec));
+          ENS_CU(cudaGraphLaunch(guard.exec, e->stream));
+          launched += ens_launches(e, chunk);
           float ms = 0.0f;
-          ENS_CU(cudaEventElapsedTime(&ms, a, b));
+          for (int reps : {chunks, 8 * chunks}) {
+            ENS_CU(cudaEventRecord(a, e->stream));
+            for (int k = 0; k < reps; ++k) ENS_CU(cudaGraphLaunch(guard.exec, e->stream));
+            ENS_CU(cudaEventRecord(b, e->stream));
+            ENS_CU(cudaEventSynchronize(b));
+            launched += reps * ens_launches(e, chunk);
+            ENS_CU(cudaEventElapsedTime(&ms, a, b));
+            ms /= static_cast<float>(reps);
+            if (ms > 0.25f) break;  // (a shorter one is timed again)
+          }
           if (best_ms < 0.0f || ms < best_ms) {
             best_ms = ms;
             best_vx = vx;
