@@ -115,7 +115,9 @@ __device__ __forceinline__ void resident_wait() {
   if constexpr (CL)
     asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
   else
-    __syncthreads();
+    // (not __syncthreads(), which all threads have to reach at one place of the
+    // program: the noise threads wait in a loop of their own)
+    asm volatile("barrier.sync 0;" ::: "memory");
 }
 
 // src and dst may be the same buffer (lbfd_step runs an even number of steps
