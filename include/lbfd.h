@@ -82,13 +82,19 @@ extern "C" {
  * choice changes speed only, never a result bit. */
 #define LBFD_KERNEL_AUTO 0    /* the library's choice (option value only) */
 #define LBFD_KERNEL_VEC 1     /* k_step_vec: two or four sites of a row per thread, pulled straight from
-                                 global memory (Lx even); FP32-arithmetic formats collide two sites at a time
-                                 on the packed FP32 instructions where that is faster, with the same result */
-#define LBFD_KERNEL_SCALAR 2  /* k_step: one site per thread (any Lx) */
+                                 global memory (Lx even), or k_step_ahead, which draws the noise first and
+                                 collides two sites at a time on the packed FP32 instructions; the result is
+                                 the same.  Buffers that do not start on a multiple of such a vector are
+                                 stepped one site per thread */
+#define LBFD_KERNEL_SCALAR 2  /* k_step: one site per thread (any Lx).  LBFD_KERNEL_AUTO reports this value for
+                                 rows of odd length, where FP32-arithmetic lattices above the smallest sizes
+                                 run k_step_twin (a site of each half of the row per thread); asked for by
+                                 step_kernel it is always k_step */
 #define LBFD_KERNEL_SMALL 3   /* k_step_resident on one block: many steps per launch in its shared memory (small
                                  lattices, n >= 2; chosen automatically) */
 #define LBFD_KERNEL_CLUSTER 4 /* k_step_resident over a thread-block cluster (chosen automatically) */
-#define LBFD_KERNEL_MRT 5     /* k_step_mrt: moment-space collision (D2Q5, multiple relaxation times) */
+#define LBFD_KERNEL_MRT 5     /* moment-space collision (D2Q5, multiple relaxation times) in k_step, k_step_ahead
+                                 or k_step_mrt; small lattices report SMALL or CLUSTER for n >= 2 */
 #define LBFD_KERNEL_STAGED 6  /* k_step_staged: persistent; each tile's source rows are copied into shared
                                  memory by the TMA unit (bulk asynchronous copies on an mbarrier), the sites
                                  pull from there, and the results go back by bulk stores.  Needs

@@ -581,7 +581,8 @@ int lbfd_step(lbfd_t h, int64_t n) {
     n -= done;
   }
   const int kernel = step_path(h, 1);
-  int vec_width = 1;
+  // (0: the library's own choice; a kernel that step_kernel asks for is the one that runs)
+  int vec_width = o.step_kernel == LBFD_KERNEL_AUTO ? 0 : 1;
   if (kernel == LBFD_KERNEL_VEC) {
     vec_width = step_vec_width(o.lattice, o.precision, a.Lx, h->N, h->vec_most);
     if (vec_width == 1) vec_width = std::min(2, h->vec_most);  // asked for by step_kernel: Lx is even

@@ -25,9 +25,11 @@ namespace lbfd {
 
 cudaError_t launch_step(int lattice, int precision, const void *src, void *dst, const StepArgs &a,
                         cudaStream_t stream, int vec_width) {
-  if (vec_width == 0)
-    vec_width = step_vec_width(lattice, precision, a.Lx, a.N, vec_most(src, dst, storage_bytes(precision)));
-  if (vec_width != 1 && ((vec_width != 2 && vec_width != 4) || a.Lx % vec_width != 0)) return cudaErrorInvalidValue;
+  if (vec_width == 0) {
+    const int own = step_vec_width(lattice, precision, a.Lx, a.N, vec_most(src, dst, storage_bytes(precision)));
+    if (own > 1) vec_width = own;  // (0 stays: one site per thread, or k_step_twin)
+  }
+  if (vec_width > 1 && ((vec_width != 2 && vec_width != 4) || a.Lx % vec_width != 0)) return cudaErrorInvalidValue;
   if (vec_width == 4 && precision == kStoreF64) return cudaErrorInvalidValue;
   switch (lattice) {
     case kD1Q3: return launch_step_d1q3(precision, src, dst, a, stream, vec_width);

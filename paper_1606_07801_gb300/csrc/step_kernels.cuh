@@ -623,6 +623,9 @@ struct StepLaunch {
 
 template <int LAT, typename S, int NOISE, typename Idx>
 cudaError_t step_noise_idx(const S *s, S *d, const StepArgs &a, int vx, cudaStream_t stream) {
+  // vx = 0: one site per thread, or the twin kernel where it is faster
+  const bool twin = vx == 0 && a.Lx % 2 != 0;
+  if (vx == 0) vx = 1;
   dim3 grid, block;
   step_shape(a.Lx, a.Ly, a.Lz, grid, block, vx,
              step_threads(LAT, sizeof(typename Store<S>::R) == 8 ? kStoreF64 : kStoreF32,
@@ -639,7 +642,7 @@ cudaError_t step_noise_idx(const S *s, S *d, const StepArgs &a, int vx, cudaStre
       }
     }
     if constexpr (NOISE != kStepNoiseOff && LAT != kD1Q3) {
-      if (vx == 1 && a.Lx % 2 != 0 && step_vec_width(LAT, kStoreF32, 4, a.N) > 1) {  // above the smallest sizes
+      if (twin && step_vec_width(LAT, kStoreF32, 4, a.N) > 1) {  // above the smallest sizes
         step_shape((a.Lx + 1) / 2, a.Ly, a.Lz, launch.cfg.gridDim, launch.cfg.blockDim, 1, 128);
         return cudaLaunchKernelEx(&launch.cfg, k_step_twin<LAT, S, NOISE, Idx>, s, d, a);
       }

@@ -30,8 +30,8 @@ WALK_STRIDED, WALK_CONTIGUOUS, WALK_PER_TILE, WALK_PARAM = 0, 1, 2, 3
 REQ_UNKNOWN, REQ_QUEUED, REQ_RUNNING, REQ_DONE = -1, 0, 1, 2
 MAX_Q, MAX_MODES = 19, 16
 KERNEL_AUTO, KERNEL_VEC, KERNEL_SCALAR, KERNEL_SMALL, KERNEL_CLUSTER, KERNEL_MRT, KERNEL_STAGED = 0, 1, 2, 3, 4, 5, 6
-KERNEL_NAMES = {KERNEL_VEC: "k_step_vec", KERNEL_SCALAR: "k_step", KERNEL_SMALL: "k_step_small",
-                KERNEL_CLUSTER: "k_step_cluster", KERNEL_MRT: "k_step_mrt", KERNEL_STAGED: "k_step_staged"}
+KERNEL_NAMES = {KERNEL_VEC: "k_step_vec", KERNEL_SCALAR: "k_step", KERNEL_SMALL: "k_step_resident",
+                KERNEL_CLUSTER: "k_step_resident", KERNEL_MRT: "k_step_mrt", KERNEL_STAGED: "k_step_staged"}
 
 Q_OF = {D1Q3: 3, D2Q9: 9, D3Q19: 19, D2Q5: 5}
 D_OF = {D1Q3: 1, D2Q9: 2, D3Q19: 3, D2Q5: 2}
