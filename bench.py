@@ -124,6 +124,13 @@ def job_glups(world: int, sites: int, steps: int, seconds: float) -> float:
     return world * sites * steps / seconds / 1e9
 
 
+def sampled_in_step(launches: int, steps: int, samples: int) -> bool:
+    """Whether the samples of a sampled run were taken inside the step: one
+    launch a step, and one a sample for its stage 2.  A separate pass is two
+    launches a sample; a small lattice's steps share launches."""
+    return launches == steps + samples
+
+
 def measured_peaks():
     path = os.path.join(ROOT, "MEASURED_PEAKS.json")
     if os.path.exists(path):
@@ -630,12 +637,14 @@ def main():
         torch.cuda.synchronize()
         s_steps = max(k, (args.steps // k) * k)
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        s_launches = lb.abi.lbfd_kernel_launches()
         e0.record(stream)
         sim.step(s_steps)
         lb.abi.lbfd_state_device(sim.h)  # the last sample's stage 2 (side stream) before e1
         e1.record(stream)
         torch.cuda.synchronize()
         ms_sampled = e0.elapsed_time(e1)
+        s_launches = lb.abi.lbfd_kernel_launches() - s_launches
         lb.abi.lbfd_set_sample_every(sim.h, 0)
         n_samp = 5
         sim.sample()
@@ -646,10 +655,9 @@ def main():
         e1.record(stream)
         torch.cuda.synchronize()
         ms_sample = e0.elapsed_time(e1) / n_samp
-        fused = bool(kname in ("k_step_vec", "k_step", "k_step_staged") and prec != 1)
         obs = {"sample_every": k, "modes": len(modes), "steps": s_steps,
                "value_with_sampling": job_glups(world, N, s_steps, ms_sampled * 1e-3),
-               "fused": fused,
+               "fused": sampled_in_step(s_launches, s_steps, s_steps // k),
                "ms_per_sampled_step_extra": (ms_sampled / s_steps - ms_per_step) * k,
                "separate_pass": {"ms_per_sample": ms_sample,
                                  "value_with_sampling": job_glups(world, N, k, (k * ms_per_step + ms_sample) * 1e-3),
