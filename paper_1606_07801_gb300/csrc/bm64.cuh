@@ -12,19 +12,23 @@
 //     32-bit integer product M C modulo 2^32 (|r| < 2^-10.8); then
 //       -2 ln u0 = (25 - e) 2 ln 2 + 2 ln c - 2 ln(1 + r),
 //       -2 ln(1 + r) = -2 r + r^2 - (2/3) r^3 + r^4/2 - (2/5) r^5 + O(2^-66),
-//     fixed point with 2^-56, the cubic tail (< 2^-33) in FP32.  Next to u0 =
-//     1, where the result is small, the first terms cancel exactly and the
-//     rest is kept to 2^-64.  One conversion makes it FP64;
-//   - the square root is rsqrt.approx.ftz.f64 and two Newton steps;
+//     fixed point with 2^-56 below u0 = 1/2, where the value is above 1.38, and
+//     with 2^-62 and 2^-65 (the last sixteenth) above, so that its relative
+//     error stays below a quarter of FP64's rounding; the terms from r^4 on are
+//     FP32.  One conversion makes it FP64.  Next to u0 = 1 (the last 2^-11, one
+//     draw in 2048) the logarithm's series in 1 - u0 takes its place;
+//   - the square root is rsqrt.approx.ftz.f64 and sqrt_seeded;
 //   - the angle 2 pi u1 is a quadrant, one of 2048 base angles and an odd
 //     multiple of 2 pi 2^-25 below 2^-11.35, each from a table, joined by the
 //     addition formulas (4 multiply-adds).
-// 13 FP64 operations per pair.  The tables (64 KB) are evaluated by the
+// 14 FP64 operations per pair.  The tables (64 KB) are evaluated by the
 // compiler in double-double arithmetic and read through L1.  Over all 2^24
-// arguments the radius is within 6.6e-16 (rms 7.5e-17, as with the general
-// functions) and the angle's cosine and sine within 2e-16.
-// Measured on GB300: D2Q9 512 x 384, ten steps and a sample, 1827 -> 743 us;
-// D1Q3 256 sites, a thousand steps, 3963 -> 2746 us.
+// arguments the radius is within a relative 1.78e-16, root mean square 5.28e-17
+// (the C library 1.66e-16 and 5.27e-17), and the angle's cosine and sine within
+// 2e-16 absolute; radius times cosine on GB300 within a relative 2.81e-16, root
+// mean square 7.15e-17 (CUDA's functions 2.81e-16 and 7.14e-17).
+// Measured on GB300: D2Q9 512 x 384, a step, 159.8 -> 43.6 us; D1Q3 256 sites,
+// resident, 3.96 -> 1.44 us (both with the kernels around it).
 #pragma once
 
 #include <stdint.h>
@@ -74,22 +78,27 @@ inline constexpr DD kLn2{0.69314718055994528623, 2.3190468138462995584e-17};
 
 constexpr int kLogCells = 1024, kBase = 2048, kFine = 1024;
 constexpr double kScale = 72057594037927936.0;  // 2^56, the fixed point of -2 ln u
+// u0 >= 1/2: log cells from which 9 more bits are kept instead of 6 (u0 > 15/16:
+// -2 ln u0 < 2^-2.9), and from which the series is taken (u0 > 1 - 2^-11)
+constexpr int kFineCell = 896, kSeriesCell = 1023;
+__host__ __device__ constexpr int more_bits(int j) { return j >= kFineCell ? 9 : 6; }
 
 // C of log cell j (M / 2^24 in [1 + j/1024, 1 + (j+1)/1024)); the last cell
 // takes exactly 1/2, so that the terms cancel next to u0 = 1.
 __host__ __device__ constexpr int64_t cell_c(int j) {
   return j == kLogCells - 1 ? 8192 : (static_cast<int64_t>(16384) * 2048 + (2049 + 2 * j) / 2) / (2049 + 2 * j);
 }
-__host__ __device__ constexpr int64_t to_fixed(DD a) {
-  // a.h 2^56 is a whole number wherever |a.h| >= 2^-4; below, it rounds once
-  const double l = a.l * kScale + (a.h * kScale - static_cast<double>(static_cast<int64_t>(a.h * kScale)));
-  return static_cast<int64_t>(a.h * kScale) + static_cast<int64_t>(l + (l < 0 ? -0.5 : 0.5));
+__host__ __device__ constexpr int64_t to_fixed(DD a, int more = 0) {  // a 2^(56 + more), rounded once
+  const double scale = kScale * static_cast<double>(1 << more), h = a.h * scale;
+  const double l = a.l * scale + (h - static_cast<double>(static_cast<int64_t>(h)));
+  return static_cast<int64_t>(h) + static_cast<int64_t>(l + (l < 0 ? -0.5 : 0.5));
 }
 inline constexpr int64_t kTwoLn2 = to_fixed(DD{2 * kLn2.h, 2 * kLn2.l});
 
 struct alignas(16) LogCell {
   int64_t a;  // 2 ln(C 2^-14) 2^56
-  uint32_t c, pad;
+  uint32_t c;
+  int32_t more;  // u0 >= 1/2: what 2 ln 2 + 2 ln(C 2^-14) has beyond (kTwoLn2 + a) in more_bits
 };
 struct alignas(16) CosSin {
   double c, s;
@@ -125,8 +134,10 @@ __host__ __device__ constexpr Tables make_tables() {
       }
       L = add(L, add(at, at));
     }
-    T.log[j] = LogCell{j == kLogCells - 1 ? -kTwoLn2 : to_fixed(DD{2 * L.h, 2 * L.l}), static_cast<uint32_t>(cell_c(j)),
-                       0u};
+    const int64_t a = j == kLogCells - 1 ? -kTwoLn2 : to_fixed(DD{2 * L.h, 2 * L.l});
+    const DD whole = add(DD{2 * L.h, 2 * L.l}, DD{2 * kLn2.h, 2 * kLn2.l});
+    const int64_t more = to_fixed(whole, more_bits(j)) - (kTwoLn2 + a) * (int64_t(1) << more_bits(j));
+    T.log[j] = LogCell{a, static_cast<uint32_t>(cell_c(j)), static_cast<int32_t>(more)};
   }
   // base angles by rotation from pi / 8192 by pi / 4096
   const DD h{kPi.h / 8192.0, kPi.l / 8192.0}, d{kPi.h / 4096.0, kPi.l / 4096.0};
@@ -194,50 +205,73 @@ __host__ __device__ __forceinline__ double add_hi(double x, int32_t hi) {  // ad
 #endif
 }
 
-// sqrt(x) by two Newton steps on x / sqrt(x) from the seed, each correction
-// added with one rounding: within 0.501 units in the last place.  For x in
-// [2^-900, 2^900].  Five dependent FP64 operations, about three fewer than the
-// general square root (each some 50 clocks on the small lattices' chain).
-__host__ __device__ __forceinline__ double sqrt_newton(double x) {
+// sqrt(x) from the seed by Goldschmidt's iteration (1964), for x in [2^-900,
+// 2^900]: g -> sqrt(x) and h -> 1 / (2 sqrt(x)) to about 2^-39 in one step, then
+// the correction h (x - g^2), of an exact remainder, added with one rounding.
+// What is added is off by less than 2^-78 of g, so the result is the nearest
+// number but for one argument in about 2^25.  Five dependent FP64 operations,
+// about three fewer than the general square root (each some 50 clocks on the
+// small lattices' chain).
+__host__ __device__ __forceinline__ double sqrt_seeded(double x) {
   const double y = rsqrt_seed(x), h = add_hi(y, -(1 << 20));  // y / 2
-  double g = x * y;
-  g = fma64(fma64(-g, g, x), h, g);
-  return fma64(fma64(-g, g, x), h, g);
+  const double g = x * y, r = fma64(-g, h, 0.5);
+  const double g1 = fma64(g, r, g), h1 = fma64(h, r, h);
+  return fma64(fma64(-g1, g1, x), h1, g1);
 }
 #ifdef __CUDACC__
 // sqrt(x) for any x.
 __device__ __forceinline__ double sqrt_any(double x) {
   const int hi = __double2hiint(x);  // the sign and exponent: 1023 - 900 .. 1023 + 900
-  return hi >= (123 << 20) && hi < (1923 << 20) ? sqrt_newton(x) : ::sqrt(x);
+  return hi >= (123 << 20) && hi < (1923 << 20) ? sqrt_seeded(x) : ::sqrt(x);
 }
 #endif
+__host__ __device__ __forceinline__ uint32_t mul_high(uint32_t a, uint32_t b) {
+#ifdef __CUDA_ARCH__
+  return __umulhi(a, b);
+#else
+  return static_cast<uint32_t>((static_cast<uint64_t>(a) * b) >> 32);
+#endif
+}
 
-// 2^28 sqrt(-2 ln u0), u0 = ((r >> 8) + 1/2) 2^-24.
-__host__ __device__ __forceinline__ double radius28(uint32_t r, const Tables &T) {
+// 2^56 (-2 ln u0), u0 = ((r >> 8) + 1/2) 2^-24, to half a unit in the last
+// place and a quarter of one.
+__host__ __device__ __forceinline__ double log28(uint32_t r, const Tables &T) {
   const uint32_t K = (r >> 7) | 1u;  // u0 2^25
   const int nz = leading_zeros(K);   // 31 - e, e = floor(log2 K): 7 .. 31
   const uint32_t M = K << (nz - 7);  // in [2^24, 2^25)
   const int j = static_cast<int>((M >> 14) & (kLogCells - 1));
+  if (nz == 7 && j >= kSeriesCell) {
+    // -2 ln(1 - e) = 2 e + 2 e^2 (1/2 + e/3 + ...), e < 2^-11: the first term
+    // exact, the rest added with one rounding
+    const double n = static_cast<double>((1u << 25) - K);
+    const double e = n * 2.98023223876953125e-08, e2 = n * 4294967296.0;  // n 2^-25, 2^56 2 e
+    const double p = fma64(e, fma64(e, fma64(e, fma64(e, 1.0 / 6, 0.2), 0.25), 1.0 / 3), 0.5);
+    return fma64(e2 * e, p, e2);
+  }
   const LogCell cell = T.log[j];
-  const int32_t ri = static_cast<int32_t>(M * cell.c);  // r 2^38
-  // 8 more bits where the first terms cancel (K above 2^25 - 2^14)
-  const int sh = (nz == 7 && j == kLogCells - 1) ? 8 : 0;
-  const float rf = static_cast<float>(ri) * 3.637978807091713e-12f;
-  const float tail = rf * rf * rf * (-0.6666667f + rf * (0.5f - 0.4f * rf)) *
-                     (sh ? 1.8446744073709552e19f : 7.2057594037927936e16f);
-  const int64_t r2 = static_cast<int64_t>(ri) * ri;
-  int64_t X = static_cast<int64_t>(nz - 6) * kTwoLn2 + cell.a;  // (25 - e) 2 ln 2 + 2 ln c; 0 where sh > 0
-  X -= static_cast<int64_t>(ri) << (19 + sh);
-  X += (r2 + (int64_t(1) << (19 - sh))) >> (20 - sh);
+  const int sh = nz == 7 ? more_bits(j) : 0;  // X has 56 + sh bits after the point
+  const int64_t A = ((static_cast<int64_t>(nz - 6) * kTwoLn2 + cell.a) << sh) + (nz == 7 ? cell.more : 0);
+  // -2 ln(1 + r) with 65 bits, then with 56 + sh
+  const int32_t ri = static_cast<int32_t>(M * cell.c);                             // r 2^38
+  const float rf = static_cast<float>(ri) * 3.637978807091713e-12f, rf2 = rf * rf;
+  const float tail = rf2 * rf2 * (0.5f - 0.4f * rf) * 3.6893488147419103e19f;
+  const int64_t r2 = static_cast<int64_t>(ri) * ri;                                // 2^-76
+  const uint32_t q = mul_high(static_cast<uint32_t>(r2 >> 23), 0xAAAAAAABu);       // (2/3) r^2, 2^-53
+  const int64_t r3 = static_cast<int64_t>(ri) * static_cast<int64_t>(q);           // (2/3) r^3, 2^-91
+  int64_t Y = ((r2 + (1 << 10)) >> 11) - (static_cast<int64_t>(ri) << 28) - ((r3 + (1 << 25)) >> 26);
 #ifdef __CUDA_ARCH__
-  X += __float2int_rn(tail);
-  const double x = add_hi(__ll2double_rn(X), -(sh << 20));
+  Y += __float2int_rn(tail);
+  const int64_t X = A + ((Y + ((1 << (9 - sh)) >> 1)) >> (9 - sh));
+  return add_hi(__ll2double_rn(X), -(sh << 20));
 #else
-  X += static_cast<int64_t>(::rintf(tail));
-  const double x = add_hi(static_cast<double>(X), -(sh << 20));
+  Y += static_cast<int64_t>(::rintf(tail));
+  const int64_t X = A + ((Y + ((1 << (9 - sh)) >> 1)) >> (9 - sh));
+  return add_hi(static_cast<double>(X), -(sh << 20));
 #endif
-  return sqrt_newton(x);
 }
+
+// 2^28 sqrt(-2 ln u0).
+__host__ __device__ __forceinline__ double radius28(uint32_t r, const Tables &T) { return sqrt_seeded(log28(r, T)); }
 
 // 2^-28 (cos, sin) of 2 pi u1, u1 = ((r >> 8) + 1/2) 2^-24.
 __host__ __device__ __forceinline__ CosSin angle28(uint32_t r, const Tables &T) {
