@@ -383,11 +383,13 @@ cudaError_t launch_observables64(int lattice, const double *g, int32_t Lx, int32
 // copy of the state is made.  The GPU has few FP64 units, so per site the
 // kernel works in FP32 on deviations e_i = f_i - c_i from the constants
 // c_i = w_i rho_mean (what the 16-bit formats store), delta = sum_i e_i, and
-// d = rho - rho_mean; each block reduces a tile of 256 sites in FP32 and adds
-// the tile totals to FP64 accumulators.  A tile total has at most 256 terms
-// of one sign-mixed quantity, so its relative error is at most 256 x 2^-24 of
-// the sum of the terms' magnitudes; everything after it is FP64.  The final
-// pass restores the sums of f and rho from the deviations in FP64.
+// d = rho - rho_mean.  A block takes tiles of 256 sites.  A mode's terms are
+// rounded five times in FP32 (up to four modes; a warp's sites) or thirteen
+// times (more; the tile) on their way to FP64.  A thread adds its slice of the pair products and of the e_i (the
+// pairs with a row of ones) in FP32 over at most 256 terms before it goes to
+// FP64, so the relative error is at most 256 x 2^-24 of the sum of the terms'
+// magnitudes.  The final pass restores the sums of f and rho from the
+// deviations in FP64.
 // ---------------------------------------------------------------------------
 constexpr int kObsThreads = 256;
 
@@ -426,11 +428,14 @@ struct ObsPairPlan {
   static_assert(NB * SL <= kObsThreads && NB * 16 <= kObsThreads, "pair plan exceeds the block");
 };
 
-// FEW: at most four modes, whose sums each thread keeps over kModeTiles tiles;
-// with more, a warp adds every tile's terms at once (ten exchanges a mode and
-// site).  D3Q19 200^3 with 4 modes on GB300: 309 -> 284 us a sample, with the
-// packed pair sums and the parallel end of the block.
-constexpr int kModeTiles = 16, kFewModes = 4;
+// FEW: at most four modes.  Their eight sums over a warp's sites take nine
+// exchanges a tile, each of which halves the sums that a lane holds; lane l ends
+// with sum l / 4 and adds it to FP64 (five roundings in FP32).  With more modes
+// a warp adds every mode's two terms at once (ten exchanges a mode and site)
+// and the block its warps' sums, in FP32.  D3Q19 200^3 with 4 modes on GB300:
+// 304 -> 264 us a sample, with the packed pair sums and the parallel end of the
+// block.
+constexpr int kFewModes = 4;
 
 template <int LAT, typename S, bool FEW>
 __global__ void __launch_bounds__(kObsThreads) k_obs_pull(const S *__restrict__ g, const ObsDims dm, float rho_f,
@@ -468,29 +473,24 @@ __global__ void __launch_bounds__(kObsThreads) k_obs_pull(const S *__restrict__ 
   float pa[16];
 #pragma unroll
   for (int e = 0; e < 16; ++e) pa[e] = 0.0f;
-  double acc_q = 0.0, acc_pair = 0.0;  // mode sum threadIdx.x (< 2 K), pair slot threadIdx.x (< NB * 16)
-  int tiles = 0, mode_tiles = 0;
-  float mode[2 * kFewModes];
+  // mode sum threadIdx.x (< 2 K), or FEW: this warp's mode sum lane / 4; pair slot threadIdx.x (< NB * 16)
+  double acc_q = 0.0, acc_pair = 0.0;
+  int tiles = 0;
+  // FEW: the warp's sums of the terms v[0 .. 7] of its sites, sum lane / 4 into acc_q
+  auto few_modes = [&](float (&v)[2 * kFewModes]) {
+    static_assert(kFewModes == 4, "three halvings");
 #pragma unroll
-  for (int q = 0; q < 2 * kFewModes; ++q) mode[q] = 0.0f;
-
-  // this block's mode sums of the warps (wsum, after a barrier) into FP64
-  auto add_modes = [&]() {
-    if (threadIdx.x < 2 * K) {
-      float t = 0.0f;
+    for (int n = kFewModes, o = 16; n > 0; n /= 2, o /= 2) {  // n sums stay
+      const bool up = (lane & o) != 0;
 #pragma unroll
-      for (int w = 0; w < NW; ++w) t += wsum[w][threadIdx.x];
-      acc_q += static_cast<double>(t);
+      for (int k = 0; k < n; ++k) {
+        const float other = __shfl_xor_sync(0xffffffffu, up ? v[k] : v[k + n], o);
+        v[k] = (up ? v[k + n] : v[k]) + other;
+      }
     }
-  };
-  // the threads' mode sums into FP64 (between two barriers that the tile takes)
-  auto put_modes = [&]() {
-#pragma unroll
-    for (int q = 0; q < 2 * kFewModes; ++q) {
-      const float v = warp_sum_f(mode[q]);
-      if (lane == 0 && q < 2 * K) wsum[warp][q] = v;
-      mode[q] = 0.0f;
-    }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    acc_q += static_cast<double>(v[0]);
   };
 
   // FP32 block sums of the last tiles into the FP64 slot sums (in slice order)
@@ -553,9 +553,7 @@ __global__ void __launch_bounds__(kObsThreads) k_obs_pull(const S *__restrict__ 
     };
     if (K > 0) {
       const float d = valid ? delta + d_off : 0.0f;
-#pragma unroll (FEW ? kFewModes : 1)
-      for (int m = 0; m < (FEW ? kFewModes : K); ++m) {
-        if (FEW && m >= K) break;
+      auto term = [&](int m) {
         float cs, sn;
         if (phase) {
           // e^{-2 pi i k.x / L} as the product of its three per-axis factors
@@ -574,22 +572,33 @@ __global__ void __launch_bounds__(kObsThreads) k_obs_pull(const S *__restrict__ 
                                   fmaf(static_cast<float>(py), dm.inv_y, static_cast<float>(pz) * dm.inv_z));
           sincospif(2.0f * frac, &sn, &cs);
         }
-        if constexpr (FEW) {
-          mode[2 * m] = fmaf(d, cs, mode[2 * m]);
-          mode[2 * m + 1] = fmaf(-d, sn, mode[2 * m + 1]);
-        } else {
-          put(2 * m, d * cs);
-          put(2 * m + 1, -d * sn);
+        return make_float2(mul_rn(d, cs), mul_rn(-d, sn));
+      };
+      if constexpr (FEW) {
+        float v[2 * kFewModes];
+        static_for<kFewModes>([&](auto M) {
+          constexpr int m = decltype(M)::value;
+          const float2 t = m < K ? term(m) : make_float2(0.0f, 0.0f);
+          v[2 * m] = t.x;
+          v[2 * m + 1] = t.y;
+        });
+        few_modes(v);
+      } else {
+        for (int m = 0; m < K; ++m) {
+          const float2 t = term(m);
+          put(2 * m, t.x);
+          put(2 * m + 1, t.y);
         }
       }
     }
-    const bool fold = FEW && K > 0 && (++mode_tiles == kModeTiles || base + gridDim.x * kObsThreads >= dm.count);
-    if (fold) {
-      put_modes();
-      mode_tiles = 0;
-    }
     __syncthreads();
-    if (!FEW || fold) add_modes();
+    // this tile's mode sums of the warps into FP64
+    if (!FEW && threadIdx.x < 2 * K) {
+      float t = 0.0f;
+#pragma unroll
+      for (int w = 0; w < NW; ++w) t += wsum[w][threadIdx.x];
+      acc_q += static_cast<double>(t);
+    }
     if (has_block) {
 #pragma unroll 4
       for (int kk = 0; kk < SPS; ++kk) {
@@ -620,7 +629,14 @@ __global__ void __launch_bounds__(kObsThreads) k_obs_pull(const S *__restrict__ 
   // gather the slot sums, then write the block's partials in the layout of
   // the stage-2 pass: [sum delta, sum delta^2, sum e_i, modes, pairs i <= j]
   if (threadIdx.x < P::NB * 16) slot_sum[threadIdx.x] = acc_pair;
+  __shared__ double mode_sum[NW][2 * kFewModes];
+  if (FEW && lane % 4 == 0) mode_sum[warp][lane / 4] = acc_q;
   __syncthreads();
+  if (FEW && threadIdx.x < 2 * K) {
+    acc_q = 0.0;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) acc_q += mode_sum[w][threadIdx.x];
+  }
   auto slot_of = [](int i, int j) {  // i <= j < QP
     const int I = i >> 2, J = j >> 2;
     return (I * P::G - I * (I - 1) / 2 + (J - I)) * 16 + (i & 3) * 4 + (j & 3);
