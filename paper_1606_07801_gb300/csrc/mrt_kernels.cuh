@@ -6,7 +6,7 @@
 // rho (2 tau^a - 1) / (tau^a)^2 (eqs. xiglobal, xilocal).  Per site:
 //   M^a   = sum_i m_i^a f_i                      (a >= 1; M^0 = rho)
 //   M^a*  = (1 - 1/tau^a) M^a + sqrt(rho_n) amp_a z^a,  amp_a^2 = (2 tau^a - 1)/(tau^a)^2
-//   f*_i  = w_i (rho + sum_{a>=1} m_i^a M^a*)     (i >= 1; n_i^a = m_i^a w_i)
+//   f*_i  = w_i rho + w_i sum_{a>=1} m_i^a M^a*    (i >= 1; n_i^a = m_i^a w_i)
 //   f*_0  = rho - sum_{i>=1} f*_i                  (mass conservation)
 // The basis and weights are compiled in for D1Q3, D2Q9 and D3Q19; D2Q5, whose
 // weights w_0 = 1 - 2 theta, w_1..4 = theta/2 depend on theta (Sec. II), takes
@@ -124,30 +124,32 @@ __device__ __forceinline__ void mrt_given(V (&f)[Lattice<LAT>::Q], const ZF &z, 
       M[k] = mul_rn(splat<V>(p.omega[k + 1]), M[k]);
     });
   }
-  // back transform; the rest population from mass conservation
-  constexpr bool kProducts = LAT != kD3Q19;  // x is one
+  // back transform, the weighted density added last with one rounding (a sum
+  // of the density and the moments, weighted after it, rounds at the density's
+  // size: its bias over hundreds of steps was several times the error of a
+  // step); the rest population from mass conservation
   V moved = splat<V>(R(0));
   auto keep = [&](int i, const V &x) {
     f[i] = x;
-    moved = i == 1 ? x : (kProducts ? add_apart(moved, x) : add_rn(moved, x));
+    moved = i == 1 ? x : add_rn(moved, x);
   };
   if constexpr (LAT == kD2Q5) {
-    const V w = splat<V>(p.w);
-    const V q = fma_rn(splat<V>(p.m41), M[3], rho), d = mul_rn(splat<V>(p.m3), M[2]);
-    const V ex = add_apart(q, d), ey = sub_apart(q, d);
-    keep(1, mul_rn(w, fma_rn(splat<V>(p.m1), M[0], ex)));
-    keep(2, mul_rn(w, fma_rn(splat<V>(-p.m1), M[0], ex)));
-    keep(3, mul_rn(w, fma_rn(splat<V>(p.m2), M[1], ey)));
-    keep(4, mul_rn(w, fma_rn(splat<V>(-p.m2), M[1], ey)));
+    const V w = splat<V>(p.w), wr = mul_rn(w, rho), e = mul_rn(splat<V>(p.m41), M[3]);
+    const V ex = fma_rn(splat<V>(p.m3), M[2], e), ey = fma_rn(splat<V>(-p.m3), M[2], e);
+    keep(1, fma_rn(w, fma_rn(splat<V>(p.m1), M[0], ex), wr));
+    keep(2, fma_rn(w, fma_rn(splat<V>(-p.m1), M[0], ex), wr));
+    keep(3, fma_rn(w, fma_rn(splat<V>(p.m2), M[1], ey), wr));
+    keep(4, fma_rn(w, fma_rn(splat<V>(-p.m2), M[1], ey), wr));
   } else {
     V T[Q];
     NoiseTransform<LAT, R>::apply(M, T);
     static_for<Q - 1>([&](auto I) {
       constexpr int i = decltype(I)::value + 1;
+      const V w = cst<V>(L::w(i));
       if constexpr (NoiseTransform<LAT, R>::kWeighted)
-        keep(i, fma_rn(cst<V>(L::w(i)), rho, T[i]));
+        keep(i, fma_rn(w, rho, T[i]));
       else
-        keep(i, mul_rn(cst<V>(L::w(i)), add_rn(rho, T[i])));
+        keep(i, fma_rn(w, T[i], mul_rn(w, rho)));
     });
   }
   f[0] = sub_rn(rho, moved);
