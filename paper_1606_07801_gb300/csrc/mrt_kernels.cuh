@@ -263,7 +263,10 @@ cudaError_t step_mrt_t(const void *src, void *dst, const StepArgs &a, const doub
         if (vx == 2) return cudaLaunchKernelEx(&launch.cfg, k_step_ahead<LAT, S, 2, NOISE, uint32_t, C>, s, d, a, c);
       if (vx == 4) return cudaLaunchKernelEx(&launch.cfg, k_step_mrt<LAT, S, 4, NOISE>, s, d, a, c);
     }
-    return cudaLaunchKernelEx(&launch.cfg, k_step_mrt<LAT, S, 2, NOISE>, s, d, a, c);
+    if constexpr (sizeof(S) == 8 || NOISE == kStepNoiseOff)
+      return cudaLaunchKernelEx(&launch.cfg, k_step_mrt<LAT, S, 2, NOISE>, s, d, a, c);
+    else
+      return cudaErrorInvalidValue;  // (the widths are 1, 2 and 4)
   });
 }
 

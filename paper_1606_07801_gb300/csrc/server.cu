@@ -10,7 +10,10 @@
 // block t & 1, and its noise is keyed by (its seed, its lattice id, t), as if
 // it ran alone.
 //
-// One time step (tick) of the server, on the compute stream:
+// One time step (tick) of the server.  With the members' arguments in the
+// kernel parameters (LBFD_WALK_PARAM) it is one launch per lattice type and
+// group and one per simulation of >= solo_sites sites, each on its own stream
+// (launch_params).  In the other tile orders, on the compute stream:
 //   [table upload, when the resident set changed]  one copy from pinned staging
 //   k_batch_prep                                   step arguments of every member
 //   batched step per lattice type                  one launch covers all members of that type
@@ -18,7 +21,7 @@
 //   k_step per simulation of >= solo_sites sites   the single-lattice kernel, parameters as
 //                                                  kernel arguments
 // (forked onto side streams when there is more than one launch, joined after)
-// then, for each member that has taken its steps, a result kernel (streaming
+// Then, for each member that has taken its steps, a result kernel (streaming
 // shift or density) into its spare block, and on the copy stream the
 // device-to-host copy of that result.  The host sees the copy's event
 // complete, stamps the completion time and returns the range to the pool.
@@ -718,9 +721,10 @@ int lbfd_server_create(lbfd_server_t *out, const lbfd_server_options *opt) {
   if (err == cudaSuccess) err = cudaStreamCreateWithFlags(&s->cs, cudaStreamNonBlocking);
   if (err == cudaSuccess) err = cudaStreamCreateWithFlags(&s->xs, cudaStreamNonBlocking);
   if (err == cudaSuccess) err = cudaMalloc(&s->arena, size_t(s->pool->capacity()));
-  if (err == cudaSuccess) err = cudaMalloc(&s->d_members, sizeof(BatchMember) * size_t(o.max_active));
-  if (err == cudaSuccess) err = cudaMalloc(&s->d_tile_start, sizeof(int64_t) * size_t(o.max_active));
-  if (err == cudaSuccess) err = cudaMalloc(&s->d_steps, sizeof(BatchStep) * size_t(o.max_active));
+  const bool tables = o.walk != LBFD_WALK_PARAM;  // (the parameter-space launches carry the members themselves)
+  if (err == cudaSuccess && tables) err = cudaMalloc(&s->d_members, sizeof(BatchMember) * size_t(o.max_active));
+  if (err == cudaSuccess && tables) err = cudaMalloc(&s->d_tile_start, sizeof(int64_t) * size_t(o.max_active));
+  if (err == cudaSuccess && tables) err = cudaMalloc(&s->d_steps, sizeof(BatchStep) * size_t(o.max_active));
   for (int k = 0; k < kStageSlots && err == cudaSuccess; ++k) {
     err = cudaHostAlloc(reinterpret_cast<void **>(&s->stage[k]), stage_bytes(s), cudaHostAllocDefault);
     if (err == cudaSuccess) err = cudaEventCreateWithFlags(&s->stage_ev[k], cudaEventDisableTiming);
@@ -737,12 +741,12 @@ int lbfd_server_create(lbfd_server_t *out, const lbfd_server_options *opt) {
     err = cudaStreamCreateWithFlags(&s->ls[L], cudaStreamNonBlocking);
     if (err == cudaSuccess) err = cudaEventCreateWithFlags(&s->lat_ev[L], cudaEventDisableTiming);
   }
-  s->tick_ev.assign(size_t(o.max_ahead), nullptr);
-  for (int k = 0; k < o.max_ahead && err == cudaSuccess; ++k)
-    err = cudaEventCreateWithFlags(&s->tick_ev[k], cudaEventDisableTiming);
+  s->tick_ev.assign(tables ? size_t(o.max_ahead) : 0, nullptr);
+  for (cudaEvent_t &ev : s->tick_ev)
+    if (err == cudaSuccess) err = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
   // the parameter-space launches mark every second of the steps the host may be ahead
   s->ahead_stride = std::max(1, o.max_ahead / 2);
-  for (int k = 0; k < 3 + lbfd_server::kSoloStreams; ++k) {
+  for (int k = 0; k < 3 + lbfd_server::kSoloStreams && !tables; ++k) {
     s->ahead_ev[k].assign(size_t(o.max_ahead) / s->ahead_stride + 2, nullptr);
     s->ahead_set[k].assign(s->ahead_ev[k].size(), 0);
     for (cudaEvent_t &ev : s->ahead_ev[k])

@@ -341,16 +341,15 @@ constexpr int step_min_blocks() {
   return LAT == kD3Q19 ? 3 : 4;
 }
 
-// Whether the vector kernel collides its sites two at a time on the packed
-// FP32 instructions (collide_pair; a tuning choice, results are the same bit
-// for bit).  Pairs cut the instructions per site (D3Q19 FP32: 590 against 695,
-// D2Q9: 244 against 277) but hold two sites' noise variates at once, and pay
-// only where the registers allow.  On GB300, microseconds per step:
+// Whether the vector kernel (k_step_vec; not k_step_ahead, which always does)
+// collides its sites two at a time on the packed FP32 instructions
+// (collide_pair; a tuning choice, results are the same bit for bit).  Pairs cut
+// the instructions per site but hold two sites' noise variates at once, and
+// pay only where the registers allow.  On GB300, microseconds per step of the
+// noisy forms that the kernel runs (step_ahead says which):
 //   D2Q9 FP32 at 2048^2, 2 sites per thread:    46.5 paired, 47.8 not
 //   D2Q9 FP32 at 2048^2, 4 sites per thread:    48.2 paired (spills), 46.3 not
-//   D3Q19 FP32 at 256^3, 2 sites per thread:   472.7 paired (spills), 412.5 not
 //   D3Q19 16-bit at 256^3, 4 sites per thread: 400.6 paired, 419.1 not
-//   D2Q9 16-bit at 2048^2, 4 sites per thread:   41.4 paired, 42.5 not
 //   D1Q3 FP32 at 2^24, 2 sites per thread:       68.1 paired, 72.3 not
 template <int LAT, typename S, int VX>
 __host__ __device__ constexpr bool step_pairs() {
@@ -584,9 +583,12 @@ __global__ void __launch_bounds__(128, 7)
 // 256^3 351 against 356), D2Q9 FP32 below 2^21 sites (1024^2 11.5 -> 10.7,
 // 2048^2 45.1 against 45.3) and D2Q9 16-bit (2048^2 40.0 -> 39.2).
 template <int LAT, typename S>
+constexpr bool ahead_always(int vx) {
+  return LAT == kD3Q19 ? vx == 2 : (LAT == kD2Q9 && Store<S>::kDeviation);
+}
+template <int LAT, typename S>
 inline bool step_ahead(int vx, int64_t sites) {
-  if (LAT == kD3Q19) return vx == 2;
-  return LAT == kD2Q9 && (Store<S>::kDeviation || sites < (int64_t(1) << 21));
+  return ahead_always<LAT, S>(vx) || (LAT == kD2Q9 && sites < (int64_t(1) << 21));
 }
 
 // True when every value offset i N + site of a lattice fits 32 bits.
@@ -647,9 +649,11 @@ cudaError_t step_noise_idx(const S *s, S *d, const StepArgs &a, int vx, cudaStre
         return cudaLaunchKernelEx(&launch.cfg, k_step_twin<LAT, S, NOISE, Idx>, s, d, a);
       }
     }
-    if (vx == 4) return cudaLaunchKernelEx(&launch.cfg, k_step_vec<LAT, S, 4, NOISE, Idx>, s, d, a);
+    if constexpr (NOISE == kStepNoiseOff || !ahead_always<LAT, S>(4))
+      if (vx == 4) return cudaLaunchKernelEx(&launch.cfg, k_step_vec<LAT, S, 4, NOISE, Idx>, s, d, a);
   }
-  if (vx == 2) return cudaLaunchKernelEx(&launch.cfg, k_step_vec<LAT, S, 2, NOISE, Idx>, s, d, a);
+  if constexpr (NOISE == kStepNoiseOff || sizeof(typename Store<S>::R) == 8 || !ahead_always<LAT, S>(2))
+    if (vx == 2) return cudaLaunchKernelEx(&launch.cfg, k_step_vec<LAT, S, 2, NOISE, Idx>, s, d, a);
   return cudaLaunchKernelEx(&launch.cfg, k_step<LAT, S, NOISE, Idx, C>, s, d, a, c);
 }
 
