@@ -12,23 +12,25 @@
 //     32-bit integer product M C modulo 2^32 (|r| < 2^-10.8); then
 //       -2 ln u0 = (25 - e) 2 ln 2 + 2 ln c - 2 ln(1 + r),
 //       -2 ln(1 + r) = -2 r + r^2 - (2/3) r^3 + r^4/2 - (2/5) r^5 + O(2^-66),
-//     fixed point with 2^-56 below u0 = 1/2, where the value is above 1.38, and
+//     fixed point with 2^-57 below u0 = 1/2, where the value is above 1.38, and
 //     with 2^-62 and 2^-65 (the last sixteenth) above, so that its relative
 //     error stays below a quarter of FP64's rounding; the terms from r^4 on are
 //     FP32.  One conversion makes it FP64.  Next to u0 = 1 (the last 2^-11, one
 //     draw in 2048) the logarithm's series in 1 - u0 takes its place;
 //   - the square root is rsqrt.approx.ftz.f64 and sqrt_seeded;
-//   - the angle 2 pi u1 is a quadrant, one of 2048 base angles and an odd
-//     multiple of 2 pi 2^-25 below 2^-11.35, each from a table, joined by the
-//     addition formulas (4 multiply-adds).
-// 14 FP64 operations per pair.  The tables (64 KB) are evaluated by the
+//   - the angle 2 pi u1 is a quadrant, the nearest of 2049 base angles and an
+//     odd multiple of 2 pi 2^-25 below 2^-11.35, each from a table, joined by
+//     the addition formulas (6 operations).
+// 16 FP64 operations per pair.  The tables (96 KB) are evaluated by the
 // compiler in double-double arithmetic and read through L1.  Over all 2^24
-// arguments the radius is within a relative 1.78e-16, root mean square 5.28e-17
-// (the C library 1.66e-16 and 5.27e-17), and the angle's cosine and sine within
-// 2e-16 absolute; radius times cosine on GB300 within a relative 2.81e-16, root
-// mean square 7.15e-17 (CUDA's functions 2.81e-16 and 7.14e-17).
-// Measured on GB300: D2Q9 512 x 384, a step, 159.8 -> 43.6 us; D1Q3 256 sites,
-// resident, 3.96 -> 1.44 us (both with the kernels around it).
+// arguments on the host the radius is within a relative 1.78e-16, root mean
+// square 5.27e-17 (the C library 1.66e-16 and 5.27e-17), and the cosine and sine
+// within a relative 1.88e-16, root mean square 4.3e-17.  On GB300, against
+// CUDA's functions: radius times the first angle's cosine 2.79e-16, root mean
+// square 7.14e-17 (2.81e-16 and 7.14e-17); one radius times all angles 3.05e-16
+// and 8.59e-17 (3.59e-16 and 9.24e-17).
+// Measured on GB300: D2Q9 512 x 384, a step, 159.4 -> 46.9 us; D1Q3 256 sites,
+// resident, 3.95 -> 1.48 us (both with the kernels around it).
 #pragma once
 
 #include <stdint.h>
@@ -94,6 +96,8 @@ __host__ __device__ constexpr int64_t to_fixed(DD a, int more = 0) {  // a 2^(56
   return static_cast<int64_t>(h) + static_cast<int64_t>(l + (l < 0 ? -0.5 : 0.5));
 }
 inline constexpr int64_t kTwoLn2 = to_fixed(DD{2 * kLn2.h, 2 * kLn2.l});
+// what 2 ln 2 has beyond kTwoLn2 in 6 more bits
+inline constexpr int kTwoLn2More = static_cast<int>(to_fixed(DD{2 * kLn2.h, 2 * kLn2.l}, 6) - (kTwoLn2 << 6));
 
 struct alignas(16) LogCell {
   int64_t a;  // 2 ln(C 2^-14) 2^56
@@ -105,7 +109,8 @@ struct alignas(16) CosSin {
 };
 struct Tables {
   LogCell log[kLogCells];
-  CosSin base[kBase];  // 2^-28 (cos, sin) of (a + 1/2) pi / 4096
+  CosSin base[kBase + 1];  // 2^-28 (cos, sin) of a pi / 4096
+  CosSin low[kBase + 1];   // what they are beyond FP64
   CosSin fine[kFine];  // (cos - 1, sin) of (2 k + 1) 2 pi 2^-25
 };
 
@@ -139,16 +144,19 @@ __host__ __device__ constexpr Tables make_tables() {
     const int64_t more = to_fixed(whole, more_bits(j)) - (kTwoLn2 + a) * (int64_t(1) << more_bits(j));
     T.log[j] = LogCell{a, static_cast<uint32_t>(cell_c(j)), static_cast<int32_t>(more)};
   }
-  // base angles by rotation from pi / 8192 by pi / 4096
-  const DD h{kPi.h / 8192.0, kPi.l / 8192.0}, d{kPi.h / 4096.0, kPi.l / 4096.0};
-  DD c = series(h, false), s = series(h, true);
+  // base angles by rotation by pi / 4096
+  const DD d{kPi.h / 4096.0, kPi.l / 4096.0};
+  DD c{1.0, 0.0}, s{0.0, 0.0};
   const DD dc = series(d, false), ds = series(d, true);
   for (int a = 0; a < kBase; ++a) {
     T.base[a] = CosSin{c.h * 3.7252902984619140625e-09, s.h * 3.7252902984619140625e-09};
+    T.low[a] = CosSin{c.l * 3.7252902984619140625e-09, s.l * 3.7252902984619140625e-09};
     const DD c2 = add(mul(c, dc), neg(mul(s, ds))), s2 = add(mul(s, dc), mul(c, ds));
     c = c2;
     s = s2;
   }
+  T.base[kBase] = CosSin{0.0, 3.7252902984619140625e-09};
+  T.low[kBase] = CosSin{0.0, 0.0};
   // fine angles likewise, from 2 pi 2^-25 by 2 pi 2^-24; cos - 1 = -2 sin^2(x/2)
   for (int k = 0; k < kFine; ++k) {
     const double n = 2.0 * k + 1.0, u = 1.0 / 16777216.0;
@@ -249,8 +257,11 @@ __host__ __device__ __forceinline__ double log28(uint32_t r, const Tables &T) {
     return fma64(e2 * e, p, e2);
   }
   const LogCell cell = T.log[j];
-  const int sh = nz == 7 ? more_bits(j) : 0;  // X has 56 + sh bits after the point
-  const int64_t A = ((static_cast<int64_t>(nz - 6) * kTwoLn2 + cell.a) << sh) + (nz == 7 ? cell.more : 0);
+  const int sh = nz == 7 ? more_bits(j) : 1;  // X has 56 + sh bits after the point
+  // (25 - e) 2 ln 2 + 2 ln c; below u0 = 1/2 what it has beyond 56 bits goes into the one more bit
+  const int beyond = (cell.more >> (more_bits(j) - 6)) + (nz - 7) * kTwoLn2More;
+  const int64_t A = ((static_cast<int64_t>(nz - 6) * kTwoLn2 + cell.a) << sh) +
+                    (nz == 7 ? cell.more : (beyond + 16) >> 5);
   // -2 ln(1 + r) with 65 bits, then with 56 + sh
   const int32_t ri = static_cast<int32_t>(M * cell.c);                             // r 2^38
   const float rf = static_cast<float>(ri) * 3.637978807091713e-12f, rf2 = rf * rf;
@@ -276,12 +287,16 @@ __host__ __device__ __forceinline__ double radius28(uint32_t r, const Tables &T)
 // 2^-28 (cos, sin) of 2 pi u1, u1 = ((r >> 8) + 1/2) 2^-24.
 __host__ __device__ __forceinline__ CosSin angle28(uint32_t r, const Tables &T) {
   const uint32_t K = (r >> 7) | 1u;
-  const int b = static_cast<int>(K & 4095u) - 2048;  // odd
-  const CosSin A = T.base[(K >> 12) & (kBase - 1)];
+  const uint32_t m = K & 0x7fffffu, a = (m + 2048u) >> 12;  // in the quadrant; the nearest base angle, 0 .. 2048
+  const int b = static_cast<int>(m) - static_cast<int>(a << 12);  // odd, -2047 .. 2047
+  const CosSin A = T.base[a];
   const CosSin B = T.fine[(b < 0 ? -b : b) >> 1];
   const double sb = add_hi(B.s, b < 0 ? static_cast<int32_t>(0x80000000u) : 0);  // odd in b (B.s > 0)
-  const double c = fma64(A.c, B.c, fma64(-A.s, sb, A.c));
-  const double s = fma64(A.s, B.c, fma64(A.c, sb, A.s));
+  // the small part first, with what the base is beyond FP64, so that the result
+  // is rounded about once
+  const CosSin low = T.low[a];
+  const double c = A.c + fma64(A.c, B.c, fma64(-A.s, sb, low.c));
+  const double s = A.s + fma64(A.s, B.c, fma64(A.c, sb, low.s));
   // the quadrant: (c, s), (-s, c), (-c, -s), (s, -c)
   const uint32_t q = K >> 23;
   CosSin out;
