@@ -383,14 +383,15 @@ int lbfd_mass_noalloc(int32_t lattice, int32_t precision, const void *f_dev, int
 /* ---- batched ensembles ------------------------------------------------------
  * Many independent lattices of one lattice type (each with its own size,
  * tau, rho_mean, seed and Philox lattice id) advanced together: one launch
- * per time step covers every member, and chunks of steps are captured into a
- * CUDA graph and replayed.  Every member evolves exactly as the same lattice
+ * per time step covers every member (LBFD_WALK_PARAM: one per group of up to
+ * 112), and chunks of steps are captured into a CUDA graph and replayed.  Every member evolves exactly as the same lattice
  * would under lbfd_create_ex with the same parameters (same arithmetic,
  * same noise keys).  Members share one precision, noise mode and law, and
  * each member has Q * sites < 2^32.  Work decomposition: a work item is 1
  * or 2 sites of a row (neighbours where Lx is even, else one of each half of
- * the row), a tile is at most `passes` x 128 items of one member, and the tiles go to blocks in one of the orders
- * LBFD_WALK_* (see lbfd_ensemble_tune / lbfd_ensemble_plan). */
+ * the row), a tile is at most `passes` x 128 items of one member, and the
+ * tiles go to blocks in one of the orders LBFD_WALK_* (see
+ * lbfd_ensemble_tune / lbfd_ensemble_plan). */
 typedef struct lbfd_member {
     int64_t dims[3];    /* Lx, Ly, Lz; trailing dims of lower-D lattices must be 1 */
     double tau;         /* > 1/2 */
@@ -409,8 +410,8 @@ typedef struct lbfd_ens *lbfd_ens_t;
  * two device buffers allocated here).  stream: a cudaStream_t other than the
  * legacy default stream (graphs are captured on it); NULL makes the ensemble
  * create and own a non-blocking stream.  The initial decomposition is two
- * sites per item where Lx is even, 4 passes, occupancy variant 0, one block
- * per tile (lbfd_ensemble_tune / lbfd_ensemble_plan change it). */
+ * sites per item at most, 4 passes, occupancy variant 0, one block per tile
+ * (lbfd_ensemble_tune / lbfd_ensemble_plan change it). */
 int lbfd_ensemble_create(lbfd_ens_t *out, int32_t lattice, int32_t precision, int32_t noise_mode, int32_t noise_dist,
                          const lbfd_member *members, int32_t n, void *stream);
 int lbfd_ensemble_destroy(lbfd_ens_t e);
@@ -438,8 +439,9 @@ int lbfd_ensemble_tune(lbfd_ens_t e, int32_t steps, int32_t *vx_chosen, int32_t 
 int lbfd_ensemble_plan(lbfd_ens_t e, int32_t vx_max, int32_t passes, int32_t occupancy, int32_t walk);
 
 /* Members, total sites, t and the current decomposition: sites per item at
- * most, tile passes, resident blocks per SM, tile order LBFD_WALK_* (any
- * pointer may be NULL). */
+ * most, tile passes as asked for (with LBFD_WALK_PARAM, launches that would
+ * not fill the GPU four times take shorter tiles), resident blocks per SM,
+ * tile order LBFD_WALK_* (any pointer may be NULL). */
 int lbfd_ensemble_query(lbfd_ens_t e, int32_t *n_members, int64_t *total_sites, int64_t *t, int32_t *vx,
                         int32_t *passes, int32_t *blocks_per_sm, int32_t *walk);
 
@@ -458,10 +460,10 @@ int lbfd_ensemble_mass(lbfd_ens_t e, int32_t member, double *mass);
  * population blocks fit in its device-memory budget (one arena allocated at
  * creation; admission and retirement allocate nothing).  Every time step
  * is one launch per lattice type covering all resident simulations of that
- * type (the batched kernel of the ensemble), plus one single-lattice launch
- * for each simulation of at least solo_sites sites, all on side streams, so
- * requests that arrive while others run join the next step and their work
- * overlaps on the device.  A
+ * type (the batched kernel of the ensemble; one per group of up to 112 with
+ * LBFD_WALK_PARAM), plus one single-lattice launch for each simulation of at
+ * least solo_sites sites, all on side streams, so requests that arrive while
+ * others run join the next step and their work overlaps on the device.  A
  * simulation that has taken its steps is read back on a second stream while
  * the others go on, and its memory returns to the arena once the copy is
  * done.  Each simulation keeps its own step counter t (from 0) and its own

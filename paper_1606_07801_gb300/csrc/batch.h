@@ -30,8 +30,8 @@ int batch_build_params(const BatchMember *members, int n, int64_t ntiles, int no
 // Parts of a set of members that step on streams of their own: while one's
 // launch ends, the other's blocks take the SMs.  Measured on GB300, GLUPS with
 // one part and two (three and four are no better): 60 D2Q9 members of 96..512
-// a side 78.5 and 83.0, 4 of 300..500 71.4 and 76.9, 40 of 60..100 57.8 and
-// 64.9, D3Q19 40 of 32..128 38.5 and 40.2, 8 of 30..60 32.0 and 37.1; but 20
+// a side 77.9 and 82.6, 4 of 300..500 71.4 and 76.9, 40 of 60..100 57.8 and
+// 64.9, D3Q19 40 of 32..128 37.7 and 39.5, 8 of 30..60 31.2 and 36.1; but 20
 // D2Q9 members of 30..80 (51000 sites) 24.6 and 24.2.  The server keeps one
 // (24 mixed requests 59.5 and 59.0 ms: its types already overlap).
 inline int batch_parts(int64_t sites) { return sites >= (int64_t(1) << 17) ? 2 : 1; }

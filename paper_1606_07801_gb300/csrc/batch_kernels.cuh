@@ -38,8 +38,11 @@ namespace lbfd {
 // Threads of a block: small blocks end a launch more evenly.  128 against 256
 // in the parameter-space launches on GB300, GLUPS: 60 D2Q9 members of 96..512
 // a side 78.5 and 75.7 (FP16 78.1 and 76.8), 20 of 30..80 24.8 and 21.1, 40
-// D3Q19 members of 32..128 38.5 and 37.8, 8 of 30..60 32.0 and 30.2, 600 D2Q9
-// members 83.7 and 83.2.
+// D3Q19 members of 32..128 38.5 and 37.8, 8 of 30..60 32.0 and 30.2 (with a
+// noise transform of fewer operations; 37.7 and 31.2 with the present one), 600
+// D2Q9 members 83.7 and 83.2.  In the other orders, default plan, against
+// blocks of 256 and the kernels of the time: 60 D2Q9 62.9 and 60.1, 40 D3Q19
+// 36.1 and 33.5, 60 lines 66.3 and 62.3, 20 FP64 D2Q9 members 3.3 and 0.7.
 constexpr int kBatchThreads = 128;
 // Order in which blocks take tiles: a persistent grid whose blocks take every
 // grid-th tile (strided) or one run of consecutive tiles (contiguous), one
@@ -155,7 +158,9 @@ __host__ __device__ constexpr int batch_column() {
 // prepared by a launch of its own (blocks of 256 threads, one launch a step; for
 // the present figures see kBatchThreads and batch_parts): 60 D2Q9 members of
 // 96..512 a side 62.8 -> 80.0 GLUPS with even rows, 59.4 -> 73.3 odd; 40 D3Q19
-// members of 32..128 a side 36.9 -> 42.1 even, 33.4 -> 36.0 odd.
+// members of 32..128 a side 36.9 -> 42.1 even, 33.4 -> 36.0 odd (with a noise
+// transform of fewer operations).  In two parts now: D2Q9 88.3 with even rows,
+// 82.6 as they are, D3Q19 42.3 and 39.5.
 // ready() is called before an item's first load.
 template <int LAT, typename S, int NOISE, int VXMAX, class F>
 __device__ __forceinline__ void batch_tile_items(S *base, const BatchStep &b, int rel, int passes, float2 *column,

@@ -365,9 +365,9 @@ inline bool sample_staged_default() {
 // or the separate pass and a plain step: a large D3Q19 lattice's plain step
 // gains more from blocks and registers of its own than one pull saves.  On
 // GB300, microseconds per step at a sample every 5 steps, fused and separate:
-// D3Q19 FP32 64^3 11.1 and 13.5, 128^3 65.8 and 66.5, 200^3 298.8 and 287.3,
-// 256^3 491.2 and 490.9, FP16 200^3 285.2 and 270.9; D2Q9 FP32 512^2 5.5 and
-// 7.0, 2048^2 54.6 and 55.4.
+// D3Q19 FP32 64^3 10.9 and 13.4, 128^3 66.8 and 67.7, 200^3 306.7 and 292.0,
+// 256^3 503.6 and 498.3, FP16 200^3 295.1 and 278.4; D2Q9 FP32 512^2 5.3 and
+// 6.9, 2048^2 52.6 and 55.5.  (D3Q19 160^3, just below the line: 166 and 146.)
 inline bool sample_fused_pays(int lattice, int64_t N) {
   return lattice != kD3Q19 || N < (int64_t(1) << 22) || sample_staged_default();
 }

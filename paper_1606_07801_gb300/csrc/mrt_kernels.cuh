@@ -17,11 +17,12 @@
 // the paired form and the store are theirs too, as are the dependent launch,
 // the alternating sweep and the resident kernel for small lattices.
 //
-// What bounds it: instruction issue (D3Q19 FP32: both transforms and the
-// noise) and, for small lattices, launches.  Measured on GB300, microseconds
-// per step, against dense transforms launched plainly: D3Q19 FP32 128 x 120 x
-// 96 55.4 -> 44.1 (0.75 of the copy bandwidth on its 224 MB), D2Q9 1024^2 18.5
-// -> 13.2, D2Q5 2048^2 32.8 -> 26.2, and D2Q5 81^2, resident, 4.17 -> 0.84.
+// What bounds it: the FMA pipe (D3Q19 FP32: both transforms and the noise, 73%
+// busy) and, for small lattices, the resident kernel's chain.  Measured on
+// GB300, microseconds per step, against dense transforms launched plainly:
+// D3Q19 FP32 128 x 120 x 96 55.3 -> 39.9 (0.83 of the copy bandwidth on its 224
+// MB), D2Q9 1024^2 18.5 -> 12.6, D2Q5 2048^2 32.8 -> 25.7, and D2Q5 81^2,
+// resident, 4.1 -> 0.66.
 #pragma once
 
 #include "step_kernels.cuh"

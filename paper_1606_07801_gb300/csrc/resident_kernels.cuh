@@ -15,8 +15,9 @@
 //   - each thread advances the step's Philox words itself;
 //   - where the threads allow, the variates are drawn by threads of their own,
 //     one per site and Philox call, two steps ahead (SPLIT): D1Q3 FP64 256
-//     sites 2.25 -> 1.35 us per step, D2Q9 FP64 24 x 20 5.23 -> 2.82, D2Q9
-//     FP32 64 x 48 0.85 -> 0.72, D3Q19 FP32 6^3 1.05 -> 0.80.
+//     sites 2.25 -> 1.35 us per step (1.48 with the present FP64 pairs), D2Q9
+//     FP64 24 x 20 5.23 -> 2.67, D2Q9 FP32 64 x 48 0.85 -> 0.69, D3Q19 FP32 6^3
+//     1.05 -> 0.76.
 // Measured on GB300, microseconds per step, against several sites per thread
 // on as few CTAs as hold the state, with addresses, noise and divisions on
 // the chain: D2Q9 FP32 64 x 48 5.77 -> 0.83, 100 x 100 9.42 -> 1.21, D3Q19

@@ -480,7 +480,7 @@ int launch_solo(lbfd_server *s, int64_t id, cudaStream_t stream) {
 // launches, and the streams meet the compute stream only where the resident
 // set changes: before the first step of new members (their initial state is
 // made there) and after the last step of a finished one (its result is).
-// Measured on GB300, 24 mixed requests served to completion: 91.0 -> 59.6 ms,
+// Measured on GB300, 24 mixed requests served to completion: 91.0 -> 60.2 ms,
 // with the items of batch_tile_items.
 int launch_params(lbfd_server *s, bool changed) {
   const int ring = int(s->ahead_ev[0].size());

@@ -251,7 +251,7 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // that draws it first has work for the time in which the previous step's last
 // blocks still run: it waits for them after the noise, before its first load.
 // A lattice whose blocks fill the GPU once or a few times gains most (D3Q19
-// FP32 64^3 8.0 -> 6.1 us per step, D2Q9 FP32 512^2 4.4 -> 3.05 on GB300).
+// FP32 64^3 8.0 -> 6.2 us per step, D2Q9 FP32 512^2 4.4 -> 3.05 on GB300).
 
 // Scalar kernel: one site per thread, any lattice shape.
 template <int LAT, typename S, int NOISE, typename Idx, class C>
@@ -559,9 +559,9 @@ __device__ __forceinline__ void twin_update(const S *src, S *dst, const StepArgs
 }
 
 // Twin kernel, for rows of odd length.  Measured on GB300 against one site
-// per thread, microseconds per step: D2Q9 FP32 1023 x 771 11.0 -> 9.2, 511 x
-// 513 5.2 -> 3.7, D3Q19 FP32 127 x 128 x 128 56.4 -> 54.3, 63 x 64 x 64 8.4 ->
-// 6.9.
+// per thread, microseconds per step: D2Q9 FP32 1023 x 771 10.8 -> 9.1, 511 x
+// 513 4.9 -> 3.6, D3Q19 FP32 127 x 128 x 128 58.0 -> 55.6 (FP16 59.1 -> 55.7),
+// 63 x 64 x 64 8.6 -> 7.0.
 template <int LAT, typename S, int NOISE, typename Idx>
 __global__ void __launch_bounds__(128, 7)
     k_step_twin(const S *src, S *dst, const StepArgs a) {
@@ -577,10 +577,10 @@ __global__ void __launch_bounds__(128, 7)
 }
 
 // Where k_step_ahead replaces k_step_vec (noisy steps in FP32 arithmetic),
-// microseconds per step on GB300: D3Q19 FP32 at every size (256^3 390 -> 375,
-// 1.004 of the copy bandwidth),
-// D3Q19 16-bit below the sizes of four sites per thread (64^3 7.95 -> 6.3; at
-// 256^3 351 against 356), D2Q9 FP32 below 2^21 sites (1024^2 11.5 -> 10.7,
+// microseconds per step on GB300: D3Q19 FP32 at every size (256^3 407 -> 392,
+// 0.96 of the copy bandwidth; 128^3 53.6 -> 49.5), D3Q19 16-bit below the sizes
+// of four sites per thread (64^3 8.1 -> 6.3; at 256^3 four take 367, two here
+// 401), D2Q9 FP32 below 2^21 sites (1024^2 11.5 -> 10.7,
 // 2048^2 45.1 against 45.3) and D2Q9 16-bit (2048^2 40.0 -> 39.2).
 template <int LAT, typename S>
 constexpr bool ahead_always(int vx) {

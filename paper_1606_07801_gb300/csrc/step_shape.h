@@ -26,15 +26,16 @@ inline int vec_most(const void *a, const void *b, int value_bytes) {
 // pays in full.  Measured on GB300, microseconds per step:
 //   4 (16-byte loads and stores of FP32) for all but D3Q19 in FP32 from 2^19
 //     sites: D1Q3 FP32 2^24 63.9 against 68.2 with two (10^5 sites 2.7 against
-//     2.0), D3Q19 FP16 128^3 49.1 against 53.2 with two,
-//     but 64^3 13.8 against 8.2; D2Q9 FP16 1024^2 12.1 against 12.9, but D2Q9
+//     2.0), D3Q19 FP16 128^3 47.8 against 50.3 with two, 256^3 367 against 401,
+//     but 64^3 13.4 against 6.3; D2Q9 FP16 1024^2 12.1 against 12.9, but D2Q9
 //     FP32 320^2 6.0 against 3.3.  D3Q19 in FP32 needs too many registers for
-//     four (31.7 against 38.9 GLUPS).  D2Q5, whose sites are short, takes four
+//     four (256^3 477 against 392).  D2Q5, whose sites are short, takes four
 //     from the start (moment-space 400^2 2.9 against 3.4, 2048^2 26.2 against
 //     27.2).
 //   2 otherwise, but 1 for the smallest: D2Q9 200^2 2.8 against 3.7 with two,
-//     D3Q19 22^3 2.8 against 6.3, 32^3 5.5 against 7.0 (16-bit 5.5 against
-//     6.9; 48^3 7.0 against 7.2).
+//     D3Q19 24^3 3.1 against 6.7, 32^3 6.3 against 6.8.  The line was drawn
+//     with k_step_vec; two sites in k_step_ahead take 2.0 and 2.1 at these two
+//     sizes, so that it lies too high for the lattices that kernel steps.
 //   1 in FP64, whose narrow pipe hides the extra instructions: D2Q9 512 x 384
 //     47.0 against 50.3 with two, 60 x 50 6.1 against 10.3.
 // A tuning knob only; results do not depend on it.  LBFD_STEP_VX = 1, 2 or 4

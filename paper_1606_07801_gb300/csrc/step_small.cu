@@ -11,18 +11,22 @@ namespace lbfd {
 // kernel is not taken.  One site per thread bounds the lattice: 16 CTAs of
 // resident_threads, or less where that many sites do not fit the shared
 // memory.  Measured on GB300, microseconds per step:
-//   - above the bound one launch per step is faster (D2Q9 FP32 128 x 170: 3.6
-//     launched, 3.8 with two sites per thread; D1Q3 FP32 32000 sites: 1.6
-//     against 2.2), below it slower (D2Q9 128 x 128: 3.5 against 1.77, D3Q19
-//     16^3: 4.2 against 1.37);
+//   - a cluster is faster than one launch per step up to that bound (D2Q9 FP32
+//     128 x 128: 1.76 resident, 1.81 launched; D3Q19 20^3 2.14 and 2.83, D1Q3
+//     16000 sites 0.82 and 1.62), and several sites per thread above it were
+//     not (D2Q9 128 x 170: 3.8 and 3.6 with the kernels of the time);
 //   - one block, whose barrier is cheaper, wins while its warps are few
-//     (D2Q9 91 sites 0.44 against 0.72 on 16 CTAs, 400 sites 0.96 against 0.73;
-//     D1Q3 300 sites 0.37 against 0.58; D3Q19 216 sites 1.16 against 1.04);
-//   - beyond that, more CTAs are never slower (D2Q9 40 x 30: 2.06 on 2, 0.89
-//     on 4, 0.79 on 8, 0.73 on 16).
-// FP64 arithmetic, 2 lanes per clock and SM, takes a CTA per 32 sites, and up
-// to 128 sites on each (D2Q9 1600 sites 5.5 against 6.0 launched, 3000 sites
-// 7.2 against 6.1; D3Q19 1728 sites 12.3 and 12.3, 4096 sites 20.8 and 12.4).
+//     (D2Q9 91 sites 0.30 against 0.53 on 16 CTAs, 256 sites 0.50 and 0.53,
+//     400 sites 0.86 and 0.53; D1Q3 300 sites 0.32 and 0.43, 600 sites 0.45 and
+//     0.42; D3Q19 125 sites 0.76 and 0.75, 216 sites 1.11 and 0.75);
+//   - beyond that, more CTAs are never slower (D2Q9 40 x 30: 1.18 on 2, 0.86
+//     on 4, 0.63 on 8, 0.58 on 16).
+// FP64 arithmetic, 2 lanes per clock and SM, takes a CTA per 32 sites (D2Q9 480
+// sites 2.67 resident, 3.55 launched; D3Q19 216 sites 6.7 and 7.4; D1Q3 2048
+// sites 1.86 and 2.38), and up to 128 sites on each, a line from when launched
+// FP64 steps were slower: above about 50 sites a CTA D2Q9 and D3Q19 now step
+// faster launched (D2Q9 1600 sites 4.49 against 3.61, D3Q19 1728 sites 13.9
+// against 7.5).
 int small_path_ctas(int lattice, int precision, int64_t N) {
   if (N < 1) return 0;
   const int elem = storage_bytes(precision);
