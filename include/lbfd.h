@@ -91,10 +91,12 @@ extern "C" {
                                  run k_step_twin (a site of each half of the row per thread); asked for by
                                  step_kernel it is always k_step */
 #define LBFD_KERNEL_SMALL 3   /* k_step_resident on one block: many steps per launch in its shared memory (small
-                                 lattices, n >= 2; chosen automatically) */
+                                 lattices, from 2 to 8 steps on by lattice and precision; chosen
+                                 automatically).  Fewer steps, also between two samples, are launched one
+                                 by one */
 #define LBFD_KERNEL_CLUSTER 4 /* k_step_resident over a thread-block cluster (chosen automatically) */
 #define LBFD_KERNEL_MRT 5     /* moment-space collision (D2Q5, multiple relaxation times) in k_step, k_step_ahead
-                                 or k_step_mrt; small lattices report SMALL or CLUSTER for n >= 2 */
+                                 or k_step_mrt; small lattices report SMALL or CLUSTER from those 2 to 8 steps on */
 #define LBFD_KERNEL_STAGED 6  /* k_step_staged: persistent; each tile's source rows are copied into shared
                                  memory by the TMA unit (bulk asynchronous copies on an mbarrier), the sites
                                  pull from there, and the results go back by bulk stores.  Needs

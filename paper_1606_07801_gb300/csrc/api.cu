@@ -262,11 +262,12 @@ static bool staged_default() {
 }
 
 // The kernel lbfd_step(h, n) runs.  The small-lattice paths hold many steps
-// per launch, so they need n >= 2; otherwise one launch per step.
+// per launch and need as many as make up for its cost (small_path_least, 2 at
+// the least); otherwise one launch per step.
 static int step_path(const lbfd_sim *h, int64_t n) {
   const lbfd_options &o = h->opt;
   if (h->slab) return LBFD_KERNEL_STAGED;
-  if (n >= 2) {
+  if (n >= small_path_least(o.lattice, o.precision, h->N)) {
     const int ctas = small_path_ctas(o.lattice, o.precision, h->N);
     if (ctas == 1) return LBFD_KERNEL_SMALL;
     if (ctas > 1) return LBFD_KERNEL_CLUSTER;
@@ -543,21 +544,58 @@ int lbfd_step(lbfd_t h, int64_t n) {
   fill_step_params(a, o.tau, o.rho_mean);
   a.noise_mode = o.noise_mode;
   a.noise_dist = o.noise_dist;
-  const int path = step_path(h, n);
-  if (path == LBFD_KERNEL_SMALL || path == LBFD_KERNEL_CLUSTER) {
+  const int kernel = step_path(h, 1);
+  // (0: the library's own choice; a kernel that step_kernel asks for is the one that runs)
+  int vec_width = o.step_kernel == LBFD_KERNEL_AUTO ? 0 : 1;
+  if (kernel == LBFD_KERNEL_VEC) {
+    vec_width = step_vec_width(o.lattice, o.precision, a.Lx, h->N, h->vec_most);
+    if (vec_width == 1) vec_width = std::min(2, h->vec_most);  // asked for by step_kernel: Lx is even
+  }
+  // one launched step of the present state
+  auto launch_one = [&]() -> cudaError_t {
+    a.ph = make_philox_step(o.seed, o.lattice_id, uint64_t(h->t));
+    a.sweep = h->alt_sweep ? static_cast<int32_t>(h->t & 1) : 0;
+    const void *src = h->f[h->cur];
+    void *dst = h->f[h->cur ^ 1];
+    const cudaError_t e =
+        kernel == LBFD_KERNEL_MRT ? launch_step_mrt(o.lattice, o.precision, src, dst, a, h->m, h->w, h->tau_m, h->stream)
+        : kernel == LBFD_KERNEL_STAGED ? launch_step_staged(o.lattice, o.precision, src, dst, a, rows, h->status_dev,
+                                                            uint32_t(o.wait_test_bytes), h->stream)
+                                       : launch_step(o.lattice, o.precision, src, dst, a, h->stream, vec_width);
+    if (e != cudaSuccess) return e;
+    h->cur ^= 1;
+    h->t += 1;
+    return cudaSuccess;
+  };
+  if (n >= 2 && !h->slab && small_path_ctas(o.lattice, o.precision, h->N) > 0) {
     // a small lattice: many steps per launch in shared memory (bit-identical);
-    // chunks end at the sampled steps, which sample by the separate pass
+    // a run ends at the call's end or at a sampled step, which samples by the
+    // separate pass, and one too short for a launch is launched step by step
     constexpr int64_t kChunk = 4096;
-    int64_t launches = 0, done = 0;
+    const int least = small_path_least(o.lattice, o.precision, h->N);
+    int64_t launches = 0, done = 0, run = 0, run_end = 0;
     bool placed = true;
     while (done < n) {
-      if (steps_to_sample(h, h->t) == 0) {
-        int rc = sample_now(h);
-        if (rc) return rc;
+      if (done == run_end) {
+        if (steps_to_sample(h, h->t) == 0) {
+          int rc = sample_now(h);
+          if (rc) return rc;
+        }
+        int64_t until = steps_to_sample(h, h->t);
+        if (until == 0) until = h->opt.sample_every;
+        run = std::min<int64_t>(n - done, until);
+        run_end = done + run;
       }
-      int64_t until = steps_to_sample(h, h->t);
-      if (until == 0) until = h->opt.sample_every;
-      const int chunk = int(std::min<int64_t>(std::min<int64_t>(kChunk, n - done), until));
+      const int chunk = int(std::min<int64_t>(kChunk, run_end - done));
+      if (run < least) {
+        for (int k = 0; k < chunk; ++k) {
+          const cudaError_t e = launch_one();
+          if (e != cudaSuccess) return cuda_fail("lbfd_step: launch", e);
+        }
+        done += chunk;
+        launches += chunk;
+        continue;
+      }
       const int to = h->cur ^ (chunk & 1);
       a.ph = make_philox_step(o.seed, o.lattice_id, uint64_t(h->t));
       cudaError_t e = h->mrt ? launch_step_small_mrt(o.lattice, o.precision, h->f[h->cur], h->f[to], a, h->m, h->w,
@@ -580,31 +618,22 @@ int lbfd_step(lbfd_t h, int64_t n) {
     if (placed) return LBFD_OK;
     n -= done;
   }
-  const int kernel = step_path(h, 1);
-  // (0: the library's own choice; a kernel that step_kernel asks for is the one that runs)
-  int vec_width = o.step_kernel == LBFD_KERNEL_AUTO ? 0 : 1;
-  if (kernel == LBFD_KERNEL_VEC) {
-    vec_width = step_vec_width(o.lattice, o.precision, a.Lx, h->N, h->vec_most);
-    if (vec_width == 1) vec_width = std::min(2, h->vec_most);  // asked for by step_kernel: Lx is even
-  }
   const int width = sample_width(o.lattice, o.precision, a.Lx, h->vec_most);
   const bool fusable = o.sample_every > 0 && !h->mrt && sample_fused_pays(o.lattice, h->N) &&
                        sample_fusable(o.lattice, o.precision, a.Lx, a.Ly, a.Lz, o.n_modes, h->phase, width);
   int64_t extra = 0;  // launches besides one step kernel per step
   for (int64_t k = 0; k < n; ++k) {
-    a.ph = make_philox_step(o.seed, o.lattice_id, uint64_t(h->t));
-    a.sweep = h->alt_sweep ? static_cast<int32_t>(h->t & 1) : 0;
-    const void *src = h->f[h->cur];
-    void *dst = h->f[h->cur ^ 1];
     if (steps_to_sample(h, h->t) == 0) {
       if (fusable) {
         // the step and the observables of the state it reads in one pass,
         // then stage 2 of the observables on the side stream
+        a.ph = make_philox_step(o.seed, o.lattice_id, uint64_t(h->t));
+        a.sweep = h->alt_sweep ? static_cast<int32_t>(h->t & 1) : 0;
         cudaError_t e = obs_join(h);
         int nblocks = 0;
         if (e == cudaSuccess)
-          e = launch_step_sample(o.lattice, o.precision, src, dst, a, o.n_modes, h->phase, h->partials, &nblocks,
-                                 h->staged_ok, h->status_dev, width, h->stream);
+          e = launch_step_sample(o.lattice, o.precision, h->f[h->cur], h->f[h->cur ^ 1], a, o.n_modes, h->phase,
+                                 h->partials, &nblocks, h->staged_ok, h->status_dev, width, h->stream);
         if (e == cudaSuccess && !h->obs_stream) {
           e = cudaStreamCreateWithFlags(&h->obs_stream, cudaStreamNonBlocking);
           if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_sampled, cudaEventDisableTiming);
@@ -627,14 +656,8 @@ int lbfd_step(lbfd_t h, int64_t n) {
       int rc = sample_now(h);
       if (rc) return rc;
     }
-    cudaError_t e =
-        kernel == LBFD_KERNEL_MRT ? launch_step_mrt(o.lattice, o.precision, src, dst, a, h->m, h->w, h->tau_m, h->stream)
-        : kernel == LBFD_KERNEL_STAGED ? launch_step_staged(o.lattice, o.precision, src, dst, a, rows, h->status_dev,
-                                                            uint32_t(o.wait_test_bytes), h->stream)
-                                       : launch_step(o.lattice, o.precision, src, dst, a, h->stream, vec_width);
+    const cudaError_t e = launch_one();
     if (e != cudaSuccess) return cuda_fail("lbfd_step: launch", e);
-    h->cur ^= 1;
-    h->t += 1;
   }
   g_launches.fetch_add(n + extra, std::memory_order_relaxed);
   return LBFD_OK;

@@ -103,6 +103,9 @@ __host__ __device__ __forceinline__ float step_param<float>(double, float f) { r
 // lattice does not fit it (or its lattice type has no such path).
 int small_path_ctas(int lattice, int precision, int64_t N);
 
+// Fewest steps that one launch of that path is worth; shorter runs are launched step by step.
+int small_path_least(int lattice, int precision, int64_t N);
+
 // Per-lattice step launchers (one translation unit each).  vec_width: 2 and 4
 // run k_step_vec or k_step_ahead (Lx a multiple), 1 runs k_step, 0 k_step or,
 // on longer rows of odd length, k_step_twin.

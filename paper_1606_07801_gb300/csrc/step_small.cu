@@ -7,6 +7,9 @@
 
 namespace lbfd {
 
+// The largest lattice in FP32 arithmetic that one block steps.
+static int64_t one_block_sites(int lattice) { return lattice == kD1Q3 ? 512 : (lattice == kD3Q19 ? 128 : 256); }
+
 // CTAs of a lattice (1: a single block, else a cluster), 0 where the resident
 // kernel is not taken.  One site per thread bounds the lattice: 16 CTAs of
 // resident_threads, or less where that many sites do not fit the shared
@@ -35,8 +38,27 @@ int small_path_ctas(int lattice, int precision, int64_t N) {
   const int64_t by_smem = int64_t(kSmallMaxBytes) / (2 * int64_t(Q) * elem);
   if (N > kResidentCtas * std::min<int64_t>(by_smem, resident_threads(lattice, f64))) return 0;
   if (f64) return int(std::min<int64_t>(kResidentCtas, (N + 31) / 32));
-  const int64_t one = lattice == kD1Q3 ? 512 : (lattice == kD3Q19 ? 128 : 256);
-  return N <= one ? 1 : (N <= 512 ? 8 : kResidentCtas);
+  return N <= one_block_sites(lattice) ? 1 : (N <= 512 ? 8 : kResidentCtas);
+}
+
+// A launch of the resident kernel costs 3 to 16 us before its steps count (the
+// cluster's start, the address and noise set-up, the state in and out), where
+// a launched step of such a lattice costs 1.7 us (FP64 2 to 12) and no set-up.
+// Microseconds for n steps on GB300, resident / launched, back to back:
+//   - D1Q3, D2Q5 on one block: n = 2 3.5 / 4.3, 3 4.2 / 5.9;
+//     on a cluster (4000 sites): 2 6.2 / 4.3, 3 6.2 / 5.9, 4 6.2 / 7.5;
+//   - D2Q9 on one block (256 sites): 3 6.2 / 5.8, 4 6.2 / 7.4; on a cluster (64 x 48):
+//     3 8.2 / 5.9, 4 8.3 / 7.7, 5 9.1 / 9.2; 91 x 91, where a step is slower
+//     too: 5 12.4 / 9.3, 8 16.4 / 14.0, D2Q5 127 x 127 8 14.4 / 14.3;
+//   - D3Q19 6^3: 3 10.6 / 6.1, 5 12.4 / 10.2, 6 13.4 / 12.3, 8 14.4 / 16.4;
+//   - FP64: D1Q3 300 sites 5 12.4 / 12.0, 6 14.4 / 14.4; D2Q9 20 x 20
+//     6 24.6 / 22.5, 8 30.4 / 30.0; D3Q19 8^3 6 47.2 / 45.1, 8 60.6 / 60.1.
+int small_path_least(int lattice, int precision, int64_t N) {
+  if (precision == kStoreF64) return lattice == kD1Q3 ? 6 : 8;
+  if (lattice == kD3Q19) return 6;
+  if (lattice != kD1Q3 && N > 8192) return 8;
+  const bool one = N <= one_block_sites(lattice);
+  return lattice == kD2Q9 ? (one ? 4 : 5) : (one ? 2 : 4);
 }
 
 namespace {
